@@ -218,10 +218,11 @@ struct BatchMove {
 
 // louvainMove (Algorithm 4) for every open graph at once, with per-graph gains
 // and stopping.  h_live (in/out) flags the graphs still iterating; h_li
-// receives each graph's l_i.  Sweeps after the first replay a CUDA graph.
+// receives each graph's l_i (li: device scratch of G entries).  Sweeps after
+// the first replay a CUDA graph.
 static BatchMove batch_move_loop(const DevGraph &g, const Classes &cl, MoveBuffers &mb, uint32_t G, double tau,
                                  const gsp_opts &o, std::vector<uint8_t> &h_live, std::vector<int> &h_li,
-                                 uint8_t *live, cudaStream_t s) {
+                                 uint8_t *live, int *li, cudaStream_t s) {
     const bool sync = o.move == GSP_MOVE_SYNC;
     const bool fp64 = o.precision == GSP_PREC_FP64;
     const bool rule = o.singleton_rule != 0;
@@ -240,6 +241,24 @@ static BatchMove batch_move_loop(const DevGraph &g, const Classes &cl, MoveBuffe
     cudaGraphExec_t exec = nullptr;
     const bool use_graph = graphs_enabled();
     bool use_persist = sync && persistent_enabled();  // small graphs: one launch per sweep
+    if (sync) {  // few, small graphs left: the whole phase in one launch
+        LevelResult lv;
+        GSP_CUDA(cudaMemsetAsync(li, 0, sizeof(int) * G, s));
+        GSP_CUDA(cudaMemsetAsync(mb.dq_g, 0, sizeof(double) * G, s));
+        GSP_CUDA(cudaEventRecord(e0, s));
+        const bool ran = move_level(g, cl, mb, fp64, rule, tau, o.max_iterations, lv, G, live, li, s);
+        if (ran) {
+            GSP_CUDA(cudaEventRecord(e1, s));
+            GSP_CUDA(cudaMemcpyAsync(h_li.data(), li, sizeof(int) * G, cudaMemcpyDeviceToHost, s));
+            GSP_CUDA(cudaMemcpyAsync(h_live.data(), live, G, cudaMemcpyDeviceToHost, s));
+            GSP_CUDA(cudaStreamSynchronize(s));
+            GSP_CUDA(cudaEventElapsedTime(&r.ms_kernels, e0, e1));
+            r.bytes = sweep_bytes(lv.ctr, g.wt);
+            r.vertices = lv.ctr.vertices;
+            r.edges = lv.ctr.edges;
+        }
+        if (ran) return r;
+    }
     side_streams();
     try {
         for (int it = 0; it < o.max_iterations && nlive; it++) {
@@ -455,7 +474,8 @@ void louvain_batched_run(const DevGraph &g0, uint32_t G, const uint64_t *h_gvo0,
         alloc_pool(mb, cl, s);
         float ms_other = lap();
         mb.dq_g = dq_g;
-        BatchMove mr = batch_move_loop(cur, cl, mb, G, tau, o, h_live, h_li, live, s);
+        BatchMove mr = batch_move_loop(cur, cl, mb, G, tau, o, h_live, h_li, live,
+                                       reinterpret_cast<int *>(k_g), s);
         mb.dq_g = nullptr;
         float ms_move = lap();
         Cp = mb.C;

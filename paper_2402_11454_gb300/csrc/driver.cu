@@ -442,6 +442,21 @@ static MoveLoopResult move_loop_on(const DevGraph &g, const Classes &cl, MoveBuf
     const bool use_graph = graphs_enabled();
     bool use_persist = sync && persistent_enabled();  // small graphs: one launch per sweep
     cudaGraphExec_t exec = nullptr;
+    if (sync && !pr.learned) {  // small graphs: the whole phase in one launch
+        LevelResult lv;
+        GSP_CUDA(cudaEventRecord(e0, s));
+        if (move_level(g, cl, mb, fp64, rule, tau, max_it, lv, 0, nullptr, nullptr, s)) {
+            GSP_CUDA(cudaEventRecord(e1, s));
+            GSP_CUDA(cudaStreamSynchronize(s));
+            GSP_CUDA(cudaEventElapsedTime(&r.ms_kernels, e0, e1));
+            r.iterations = lv.iterations;
+            r.bytes = sweep_bytes(lv.ctr, g.wt);
+            r.vertices = lv.ctr.vertices;
+            r.edges = lv.ctr.edges;
+            r.candidates = lv.ctr.candidates;
+            return r;
+        }
+    }
     side_streams();
     try {
         // Learned pruning: the first sweep of a pass is plain (no vertex has a

@@ -159,6 +159,19 @@ void apply_moves(const DevGraph &g, MoveBuffers &mb, uint32_t n_hint, cudaStream
 bool sweep_persistent(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64, bool rule, int iteration,
                       int max_iterations, cudaStream_t s);
 
+// The whole local-moving phase of a small graph (every sweep until the gain
+// is <= tau or max_it) as one launch of one thread-block cluster, frozen-state
+// waves.  Returns false (launching nothing) when the graph or the run does
+// not qualify; otherwise *out is filled once the stream is synchronised.
+// Batches: G graphs, live (device, in/out) the graphs still iterating, li
+// (device) the sweeps of each; mb.dq_g zero at the call.
+struct LevelResult {
+    int iterations = 0;
+    MoveCounters ctr;
+};
+bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64, bool rule, double tau, int max_it,
+                LevelResult &out, uint32_t G, uint8_t *live, int *li, cudaStream_t s);
+
 // Scratch of one call taken from a caller's device buffer (gsp_opts.workspace)
 // for as long as the object lives; base == NULL leaves the internal workspace
 // in use.  workspace_peak(): most bytes the current workspace held at once

@@ -184,25 +184,32 @@ template <> struct Score<false> {
     using S = float;
     float kif, sd;
     double inv_m;
-    __device__ S score(float kic, double Sc) const { return kic - kif * (float)Sc; }
+    __device__ S score(float kic, double Sc) const { return __fmaf_rn(-kif, (float)Sc, kic); }
     __device__ double gain(S best) const { return (double)(best - sd) * inv_m; }
 };
 
 // m and inv_m = 1/m of the vertex's graph (the float64 score uses m only).
+// The float32 operations are spelled out, so that every kernel that may serve
+// a vertex decides exact ties of s_c and s_d alike: the candidates' scores
+// round once (fused); the score of staying rounds twice, but once for the
+// vertices of the largest degree class (hub), whichever kernel serves them.
 template <bool F64>
-__device__ __forceinline__ Score<F64> make_score(double Ki, double kid, double Sd, double m, double inv_m);
+__device__ __forceinline__ Score<F64> make_score(double Ki, double kid, double Sd, double m, double inv_m,
+                                                 bool hub = false);
 template <>
-__device__ __forceinline__ Score<true> make_score<true>(double Ki, double kid, double Sd, double m, double) {
+__device__ __forceinline__ Score<true> make_score<true>(double Ki, double kid, double Sd, double m, double, bool) {
     Score<true> s;
     s.Ki = Ki; s.Kid = kid; s.Sd = Sd; s.m = m;
     return s;
 }
 template <>
-__device__ __forceinline__ Score<false> make_score<false>(double Ki, double kid, double Sd, double, double inv_m) {
+__device__ __forceinline__ Score<false> make_score<false>(double Ki, double kid, double Sd, double, double inv_m,
+                                                          bool hub) {
     Score<false> s;
     const double inv2m = 0.5 * inv_m;
     s.kif = (float)(Ki * inv2m);
-    s.sd = (float)kid - s.kif * (float)(Sd - Ki);
+    const float rest = (float)(Sd - Ki);
+    s.sd = hub ? __fmaf_rn(-s.kif, rest, (float)kid) : __fsub_rn((float)kid, __fmul_rn(s.kif, rest));
     s.inv_m = inv_m;
     return s;
 }
@@ -227,9 +234,9 @@ __device__ __forceinline__ bool decide_move(const MoveArgs &a, uint32_t i, uint3
         uint32_t sd = ld_state<SYNC>(a.size + d), sc = ld_state<SYNC>(a.size + c);
         if (sd == 1 && sc == 1 && c > d) return false;
     }
-    if (a.no_return_from > 0 && a.left[i] == c) {
+    if (a.no_return_from > 0 && ld_state<SYNC>(a.left + i) == c) {
         const int it = *a.iteration;
-        if (it >= a.no_return_from && a.left_it[i] == it - 1) return false;
+        if (it >= a.no_return_from && ld_state<SYNC>(a.left_it + i) == it - 1) return false;
     }
     if (a.choice) a.choice[i] = c;
     if constexpr (SYNC) {
@@ -302,22 +309,24 @@ __device__ __forceinline__ void record_visit(const MoveArgs &a, uint32_t i, uint
 }
 
 // --------------------------------------------------------------------------
-// Groups of G lanes, one vertex per group, table of up to CAP slots per group
-// (slots carved out of the block's shared buffer).
+// Groups of G lanes, one vertex per group, table of up to CAP slots per group.
+// A warp's tables lie in its own region of shared memory (32 / G tables), so
+// the warps of a block run independently: warp `wbase` of `wstep` takes the
+// list entries wbase, wbase + wstep, ...
 // --------------------------------------------------------------------------
+template <int G, int CAP, typename V> constexpr size_t warp_tables = (size_t)(32 / G) * CAP * (sizeof(uint32_t) + sizeof(V));
+
 template <int G, int CAP, typename WT, bool F64, int SYNC>
-__device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list, uint32_t count, uint32_t lb,
-                           uint32_t nb, unsigned char *smem, LocalCtr &lc) {
+__device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list, uint32_t count, uint32_t wbase,
+                           uint32_t wstep, unsigned char *warp_smem, LocalCtr &lc) {
     using V = typename std::conditional<F64, double, float>::type;
     using SC = Score<F64>;
     using S = typename SC::S;
-    constexpr int NG = 256 / G;
     const int lane = threadIdx.x % G;
-    const int grp = threadIdx.x / G;
     const int leader = (threadIdx.x & 31) & ~(G - 1);
     const unsigned gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << leader);
-    uint32_t *keys = reinterpret_cast<uint32_t *>(smem) + grp * CAP;
-    V *vals = reinterpret_cast<V *>(smem + (size_t)NG * CAP * sizeof(uint32_t)) + grp * CAP;
+    uint32_t *keys = reinterpret_cast<uint32_t *>(warp_smem) + leader / G * CAP;
+    V *vals = reinterpret_cast<V *>(warp_smem + (size_t)(32 / G) * CAP * sizeof(uint32_t)) + leader / G * CAP;
     const WT *w = static_cast<const WT *>(a.w);
     const double m0 = *a.m;
     const double inv0 = 1.0 / m0;
@@ -330,7 +339,6 @@ __device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list,
     // in step.
     constexpr int NGW = 32 / G;  // groups per warp
     const int wl = threadIdx.x & 31, gw = wl / G;
-    const uint32_t wbase = lb * 8 + (threadIdx.x >> 5), wstep = nb * 8;
     for (uint64_t kb = 0; wbase + kb * wstep < count; kb += 32) {
         const uint64_t my = wbase + (kb + wl) * wstep;
         uint32_t vi = 0;
@@ -402,7 +410,7 @@ __device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list,
         __syncwarp(gmask);
         }
     }
-    __syncthreads();  // the block's tables are free for the next body
+    __syncwarp();  // the warp's tables are free for the next body
 }
 
 struct GroupLists {
@@ -411,25 +419,20 @@ struct GroupLists {
     uint32_t bstart[5];  // block ranges of the four classes
 };
 
-constexpr size_t GROUP_SMEM_F64 = 2048 * (sizeof(uint32_t) + sizeof(double));
-constexpr size_t GROUP_SMEM_F32 = 2048 * (sizeof(uint32_t) + sizeof(float));
-
 template <typename WT, bool F64, int SYNC>
 __global__ void __launch_bounds__(256) k_move_groups(MoveArgs a, GroupLists gl) {
-    __shared__ __align__(16) unsigned char smem[F64 ? GROUP_SMEM_F64 : GROUP_SMEM_F32];
-    uint32_t b = blockIdx.x;
+    using V = typename std::conditional<F64, double, float>::type;
+    constexpr size_t WREG = warp_tables<32, 256, V>;  // the largest of the four
+    __shared__ __align__(16) unsigned char smem[8 * WREG];
+    const uint32_t b = blockIdx.x, wid = threadIdx.x >> 5;
+    unsigned char *ws = smem + wid * WREG;
+    const int k = b < gl.bstart[1] ? 0 : b < gl.bstart[2] ? 1 : b < gl.bstart[3] ? 2 : 3;
+    const uint32_t wb = (b - gl.bstart[k]) * 8 + wid, wn = (gl.bstart[k + 1] - gl.bstart[k]) * 8;
     LocalCtr lc;
-    if (b < gl.bstart[1])
-        group_body<4, 16, WT, F64, SYNC>(a, gl.list[0], gl.count[0], b, gl.bstart[1], smem, lc);
-    else if (b < gl.bstart[2])
-        group_body<8, 32, WT, F64, SYNC>(a, gl.list[1], gl.count[1], b - gl.bstart[1], gl.bstart[2] - gl.bstart[1],
-                                         smem, lc);
-    else if (b < gl.bstart[3])
-        group_body<16, 64, WT, F64, SYNC>(a, gl.list[2], gl.count[2], b - gl.bstart[2],
-                                          gl.bstart[3] - gl.bstart[2], smem, lc);
-    else
-        group_body<32, 256, WT, F64, SYNC>(a, gl.list[3], gl.count[3], b - gl.bstart[3],
-                                           gl.bstart[4] - gl.bstart[3], smem, lc);
+    if (k == 0) group_body<4, 16, WT, F64, SYNC>(a, gl.list[0], gl.count[0], wb, wn, ws, lc);
+    else if (k == 1) group_body<8, 32, WT, F64, SYNC>(a, gl.list[1], gl.count[1], wb, wn, ws, lc);
+    else if (k == 2) group_body<16, 64, WT, F64, SYNC>(a, gl.list[2], gl.count[2], wb, wn, ws, lc);
+    else group_body<32, 256, WT, F64, SYNC>(a, gl.list[3], gl.count[3], wb, wn, ws, lc);
     flush_counters(lc, a.ctr);
 }
 
@@ -437,9 +440,12 @@ __global__ void __launch_bounds__(256) k_move_groups(MoveArgs a, GroupLists gl) 
 constexpr int W512_CAP = 1024;
 template <typename WT, bool F64, int SYNC>
 __global__ void __launch_bounds__(256) k_move_w512(MoveArgs a, const uint32_t *__restrict__ list, uint32_t count) {
+    using V = typename std::conditional<F64, double, float>::type;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
+    const uint32_t wid = threadIdx.x >> 5;
     LocalCtr lc;
-    group_body<32, W512_CAP, WT, F64, SYNC>(a, list, count, blockIdx.x, gridDim.x, dyn_smem, lc);
+    group_body<32, W512_CAP, WT, F64, SYNC>(a, list, count, blockIdx.x * 8 + wid, gridDim.x * 8,
+                                            dyn_smem + wid * warp_tables<32, W512_CAP, V>, lc);
     flush_counters(lc, a.ctr);
 }
 
@@ -449,7 +455,7 @@ __global__ void __launch_bounds__(256) k_move_w512(MoveArgs a, const uint32_t *_
 // --------------------------------------------------------------------------
 template <int CAP, typename WT, bool F64, int SYNC>
 __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list, uint32_t count, uint32_t lb,
-                           uint32_t nb, unsigned char *dyn_smem, LocalCtr &lc) {
+                           uint32_t nb, unsigned char *dyn_smem, LocalCtr &lc, uint32_t slots = CAP, bool hub = false) {
     using V = typename std::conditional<F64, double, float>::type;
     using SC = Score<F64>;
     using S = typename SC::S;
@@ -470,16 +476,17 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
     // counters accumulate in the caller's lc
-    __shared__ uint32_t s_todo[256], s_ntodo, s_wcnt[8];
-    for (uint32_t s = threadIdx.x; s < CAP; s += blockDim.x) { keys[s] = EMPTY; vals[s] = V(0); }
-    // The block's entries are lb + k * nb; blockDim.x of them are claimed at
+    constexpr uint32_t CLAIM = 256;
+    __shared__ uint32_t s_todo[CLAIM], s_ntodo, s_wcnt[32];
+    for (uint32_t s = threadIdx.x; s < slots; s += blockDim.x) { keys[s] = EMPTY; vals[s] = V(0); }
+    // The block's entries are lb + k * nb; CLAIM of them are claimed at
     // once (one flag per thread) and the active ones listed in shared memory,
     // so inactive vertices cost no serial round trip.
-    for (uint64_t kb = 0; lb + kb * nb < count; kb += blockDim.x) {
+    for (uint64_t kb = 0; lb + kb * nb < count; kb += CLAIM) {
         const uint64_t my = lb + (kb + threadIdx.x) * nb;
         uint32_t vi = 0;
         int claim = 0;
-        if (my < count) {
+        if (threadIdx.x < CLAIM && my < count) {
             vi = list[my];
             claim = ld_state<SYNC>(a.act + vi);
             if (claim) {
@@ -515,7 +522,8 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
         uint32_t d = s_d;
         uint64_t b = a.off[i], e = a.off[i + 1];
         uint32_t deg = (uint32_t)(e - b);
-        int logcap = ceil_log2(2 * deg);
+        // a degree above CAP / 2 comes only on graphs of fewer than CAP vertices (sweep_level)
+        const int logcap = min(ceil_log2(2 * deg), ceil_log2(CAP));
         V kid = 0;
         constexpr int U = CAP >= 16384 ? 8 : 4;  // hubs: more gathers in flight per thread
         scan_edges<U, SYNC, V>(a.tgt, w, a.C, i, d, b, e, threadIdx.x, blockDim.x, kid,
@@ -527,7 +535,7 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
         for (int t = 0; t < nw; t++) kid += red_k[t];
         double Ki = a.K[i];
         const double m = vertex_m(a, i, m0);
-        SC sc = make_score<F64>(Ki, (double)kid, s_Sd, m, vertex_inv_m(a, i, inv0));
+        SC sc = make_score<F64>(Ki, (double)kid, s_Sd, m, vertex_inv_m(a, i, inv0), hub);
         S best = -INFINITY;
         uint32_t bestc = EMPTY;
         uint32_t nocc = s_nocc;
@@ -563,14 +571,13 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
         __syncthreads();
         if (s_mv) {
             if (threadIdx.x == 0) lc.marked += deg;
-            for (uint64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
+            for (uint64_t p = b + threadIdx.x; a.mark && p < e; p += blockDim.x) {
                 uint32_t j = __ldg(a.tgt + p);
                 if (j != i) a.mark[j] = 1;
             }
         }
     }
     }
-    __syncthreads();
     __syncthreads();  // the block's table is free for the next body
 }
 
@@ -816,12 +823,17 @@ __global__ void __launch_bounds__(256) k_sweep_persistent(MoveArgs a, const uint
         if (!tot) continue;  // the same for every block
         MoveArgs aw = a;
         aw.mv_cnt = mv_cnts + wr;
-        if (cc[CLS_G4]) group_body<4, 16, WT, F64, 2>(aw, list + cb[CLS_G4], cc[CLS_G4], lb, nb, dyn_smem, lc);
-        if (cc[CLS_G8]) group_body<8, 32, WT, F64, 2>(aw, list + cb[CLS_G8], cc[CLS_G8], lb, nb, dyn_smem, lc);
-        if (cc[CLS_G16]) group_body<16, 64, WT, F64, 2>(aw, list + cb[CLS_G16], cc[CLS_G16], lb, nb, dyn_smem, lc);
-        if (cc[CLS_G32]) group_body<32, 256, WT, F64, 2>(aw, list + cb[CLS_G32], cc[CLS_G32], lb, nb, dyn_smem, lc);
-        if (cc[CLS_W512])
-            group_body<32, W512_CAP, WT, F64, 2>(aw, list + cb[CLS_W512], cc[CLS_W512], lb, nb, dyn_smem, lc);
+        {
+            using V = typename std::conditional<F64, double, float>::type;
+            const uint32_t wid = threadIdx.x >> 5, wb = lb * 8 + wid, wn = nb * 8;
+            unsigned char *ws = dyn_smem + wid * warp_tables<32, W512_CAP, V>;
+            group_body<4, 16, WT, F64, 2>(aw, list + cb[CLS_G4], cc[CLS_G4], wb, wn, ws, lc);
+            group_body<8, 32, WT, F64, 2>(aw, list + cb[CLS_G8], cc[CLS_G8], wb, wn, ws, lc);
+            group_body<16, 64, WT, F64, 2>(aw, list + cb[CLS_G16], cc[CLS_G16], wb, wn, ws, lc);
+            group_body<32, 256, WT, F64, 2>(aw, list + cb[CLS_G32], cc[CLS_G32], wb, wn, ws, lc);
+            group_body<32, W512_CAP, WT, F64, 2>(aw, list + cb[CLS_W512], cc[CLS_W512], wb, wn, ws, lc);
+            __syncthreads();  // the block class uses the whole buffer
+        }
         if (cc[CLS_BLOCK])
             block_body<4096, WT, F64, 2>(aw, list + cb[CLS_BLOCK], cc[CLS_BLOCK], lb, nb, dyn_smem, lc);
         if (!grid_sync(bar, nb, a.ctr)) return;
@@ -831,6 +843,406 @@ __global__ void __launch_bounds__(256) k_sweep_persistent(MoveArgs a, const uint
         if (!grid_sync(bar, nb, a.ctr)) return;
     }
     flush_counters(lc, a.ctr);
+}
+
+// --------------------------------------------------------------------------
+// Local moving of a small graph in one launch: every sweep of the phase, all
+// waves and repeats, run by one thread-block cluster.
+//
+// What bounds a small graph (and the later, aggregated levels of every run)
+// is the number of dependent steps, not the work in them: a sweep is W waves
+// (times the repeats of the first iteration), each a decide step and an apply
+// step that must see all of the other's writes; as launches a wave cost 17-25
+// us in five kernels and memsets.  Inside one cluster the steps are parted by
+// the hardware's cluster barrier, and the sweep's gain is tested against tau
+// on the device, so the host neither launches nor waits between sweeps.  The
+// rest is a chain of L2 round trips, kept short:
+//   * a warp handles 32 lanes' worth of vertices of one class (8 of 4 lanes
+//     ... 1 of 32 lanes) as one task; what of a task never changes (vertex,
+//     row bounds, K, the first LEVEL_EPL targets and weights of each lane) is
+//     fetched into registers between the arrival at a barrier and the wait;
+//   * decide: trip 1 reads the flag, C_i and C_j, trip 2 Sigma and the sizes
+//     of all candidates;
+//   * a warp keeps its movers in shared memory and applies them itself after
+//     the barrier: Sigma and size by atomics that nobody waits for, marks
+//     straight into the flags (no vertex is deciding then).
+// A cluster has at most 16 of the 152 SMs, so the host takes this path only
+// while a wave's work fits them (move_level).  Measured (611 vertices, 153
+// wave runs): 5.7 us a run against 21 as launches, of which the visit takes
+// 2.2, each barrier with its release and acquire 0.7-1.3.
+//
+// Batches: per-graph gains and stopping as in the host loop (a graph whose
+// gain of the sweep is <= tau stops, and its vertices become inactive).
+// --------------------------------------------------------------------------
+constexpr int LEVEL_CTAS = 16;       // non-portable cluster size; 8 when 16 do not fit the device
+constexpr int LEVEL_THREADS = 512;
+constexpr int LEVEL_WARPS = LEVEL_THREADS / 32;
+constexpr int LEVEL_EPL = 4;         // edges a lane holds in registers
+constexpr uint32_t LEVEL_TASKS = 6;  // most tasks of a warp in a wave ...
+constexpr uint32_t LEVEL_MOVERS = 8 * LEVEL_TASKS;  // ... of at most 8 vertices each
+constexpr uint32_t LEVEL_BMOVERS = 64;              // most vertices of the block classes per CTA and wave
+// slots of the block classes' table
+template <bool F64> constexpr int LEVEL_CAP = F64 ? 8192 : 16384;
+
+struct LevelArgs {
+    const uint32_t *list, *start;  // class/wave lists (Classes)
+    int W, R;                      // waves; repeats of a wave in the first iteration
+    uint32_t n;
+    double tau;
+    int max_it;
+    double *dq;                    // 3 gains of a sweep, zero at start
+    int *iterations;               // out: sweeps run
+    // batches (G == 0: one graph)
+    uint32_t G;
+    uint8_t *live;
+    int *li;                       // sweeps of each graph
+    uint32_t *nlive;               // 3 counts of the graphs still iterating, zero at start
+};
+
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+struct LevelMover {
+    uint64_t b;
+    double K;
+    uint32_t i, c, d, deg;
+};
+
+template <bool F64> struct LevelSmem {
+    using V = typename std::conditional<F64, double, float>::type;
+    static constexpr size_t tables_bytes =
+        std::max((size_t)LEVEL_WARPS * warp_tables<32, W512_CAP, V>,
+                 (size_t)LEVEL_CAP<F64> * (sizeof(uint32_t) + sizeof(V) + sizeof(uint16_t)));
+    alignas(16) unsigned char tables[tables_bytes];  // per-warp tables, or one table of a block class
+    LevelMover mv[LEVEL_WARPS][LEVEL_MOVERS];
+    uint32_t start[NUM_CLS * MAX_WAVES + 1];
+};
+
+// What a lane holds of its warp's task: the vertex of its group of 2^lg lanes
+// (i == EMPTY: none), and the group's edges lane, lane + G, ...
+template <typename WT> struct LevelTask {
+    uint64_t b;
+    double K, m, inv_m;
+    uint32_t i, deg;
+    int lg;
+    uint32_t j[LEVEL_EPL];
+    WT w[LEVEL_EPL];
+};
+
+// Number of warp tasks of class k with `count` vertices (lanes per vertex:
+// 4, 8, 16, 32, 32 for the classes up to CLS_W512).
+__host__ __device__ constexpr uint32_t level_lg(int k) { return k < 3 ? 2 + k : 5; }
+__host__ __device__ constexpr uint32_t level_tasks(int k, uint32_t count) {
+    return ((count << level_lg(k)) + 31) >> 5;
+}
+
+template <typename WT>
+__device__ __forceinline__ void level_fetch(const MoveArgs &a, const uint32_t *__restrict__ list,
+                                            const uint32_t *start, int W, int wv, uint32_t task, double m0, double inv0,
+                                            LevelTask<WT> &t) {
+    const uint32_t lane = threadIdx.x & 31;
+    t.i = EMPTY;
+    t.deg = 0;
+    t.lg = 5;
+    for (int k = CLS_W512; k >= CLS_G4; k--) {
+        const uint32_t beg = start[k * W + wv], cnt = start[k * W + wv + 1] - beg;
+        const uint32_t nt = level_tasks(k, cnt);
+        if (task >= nt) { task -= nt; continue; }
+        t.lg = (int)level_lg(k);
+        const uint32_t idx = (task << (5 - t.lg)) + (lane >> t.lg);
+        if (idx < cnt) t.i = list[beg + idx];
+        break;
+    }
+    if (t.i == EMPTY) return;
+    t.b = a.off[t.i];
+    t.deg = (uint32_t)(a.off[t.i + 1] - t.b);
+    t.K = a.K[t.i];
+    t.m = vertex_m(a, t.i, m0);
+    t.inv_m = vertex_inv_m(a, t.i, inv0);
+    const uint32_t gl = lane & ((1u << t.lg) - 1u);
+    const WT *w = static_cast<const WT *>(a.w);
+#pragma unroll
+    for (int u = 0; u < LEVEL_EPL; u++) {
+        const uint32_t p = gl + ((uint32_t)u << t.lg);
+        const bool ok = p < t.deg;
+        t.j[u] = ok ? __ldg(a.tgt + t.b + p) : t.i;  // padding counts as a self-loop
+        t.w[u] = ok ? __ldg(w + t.b + p) : WT(0);
+    }
+}
+
+// Decide the vertices of a task; movers are appended to mv[0..nmv).
+template <typename WT, bool F64>
+__device__ __forceinline__ void level_visit(const MoveArgs &a, const LevelTask<WT> &t, int it, unsigned char *ws,
+                                            LevelMover *mv, uint32_t &nmv, LocalCtr &lc) {
+    using V = typename std::conditional<F64, double, float>::type;
+    using SC = Score<F64>;
+    using S = typename SC::S;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t G = 1u << t.lg, gl = lane & (G - 1u);
+    const WT *w = static_cast<const WT *>(a.w);
+    const bool has = t.i != EMPTY;
+    const bool act = has && ldcg(a.act + t.i);
+    uint32_t d = 0, c[LEVEL_EPL], lf = EMPTY;
+    if (has) {
+        d = ldcg(a.C + t.i);
+#pragma unroll
+        for (int u = 0; u < LEVEL_EPL; u++) c[u] = ldcg(a.C + t.j[u]);
+        if (a.no_return_from > 0 && it >= a.no_return_from && ldcg(a.left_it + t.i) == it - 1) lf = ldcg(a.left + t.i);
+    }
+    if (!__any_sync(FULL, act)) return;
+    double Sd = 0.0;
+    uint32_t sd = 0;
+    if (act) {
+        Sd = ldcg(a.Sig + d);
+        sd = ldcg(a.size + d);
+        if (gl == 0) {
+            a.act[t.i] = 0;
+            if (a.deferred) a.deferred[t.i] = 0;
+        }
+    }
+    // the group's table: G4 16 slots, G8 32, G16 64, then 256 and 1024
+    const int logcap = max(1, ceil_log2(2 * t.deg));
+    const uint32_t cap = act ? 1u << logcap : 0u;
+    const uint32_t first = t.lg == 5 ? 0u : (lane >> t.lg) * (4u * G);
+    uint32_t *keys = reinterpret_cast<uint32_t *>(ws) + first;
+    V *vals = reinterpret_cast<V *>(ws + (size_t)W512_CAP * sizeof(uint32_t)) + first;
+    for (uint32_t s = gl; s < cap; s += G) { keys[s] = EMPTY; vals[s] = V(0); }
+    __syncwarp();
+    V kid = 0;
+    if (act) {
+#pragma unroll
+        for (int u = 0; u < LEVEL_EPL; u++) {
+            if (t.j[u] == t.i) continue;
+            if (c[u] == d) kid += (V)t.w[u];
+            else ht_add<V>(keys, vals, logcap, c[u], (V)t.w[u]);
+        }
+        if (t.deg > LEVEL_EPL * G)
+            scan_edges<4, 2, V>(a.tgt, w, a.C, t.i, d, t.b + LEVEL_EPL * G, t.b + t.deg, gl, G, kid,
+                                [&](uint32_t cc, V wv) { ht_add<V>(keys, vals, logcap, cc, wv); });
+    }
+    __syncwarp();
+    for (uint32_t o = G >> 1; o > 0; o >>= 1) kid += __shfl_xor_sync(FULL, kid, o);
+    const SC sc = make_score<F64>(t.K, (double)kid, Sd, t.m, t.inv_m);
+    S best = -INFINITY;
+    uint32_t bestc = EMPTY, bsz = 0, ncand = 0;
+    const bool need_size = a.rule && sd == 1;  // the singleton rule looks at the target's size
+    for (uint32_t s0 = gl; s0 < cap; s0 += 4 * G) {
+        uint32_t cc[4], sz[4];
+        V val[4];
+        double sg[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const uint32_t s = s0 + u * G;
+            cc[u] = s < cap ? keys[s] : EMPTY;
+            val[u] = s < cap ? vals[s] : V(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            sg[u] = cc[u] != EMPTY ? ldcg(a.Sig + cc[u]) : 0.0;
+            sz[u] = cc[u] != EMPTY && need_size ? ldcg(a.size + cc[u]) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (cc[u] == EMPTY) continue;
+            ncand++;
+            const S x = sc.score(val[u], sg[u]);
+            if (better(x, cc[u], best, bestc)) { best = x; bestc = cc[u]; bsz = sz[u]; }
+        }
+    }
+    lc.candidates += ncand;
+    __syncwarp();
+    for (uint32_t o = G >> 1; o > 0; o >>= 1) {
+        const S x = __shfl_xor_sync(FULL, best, o);
+        const uint32_t cx = __shfl_xor_sync(FULL, bestc, o), zx = __shfl_xor_sync(FULL, bsz, o);
+        if (better(x, cx, best, bestc)) { best = x; bestc = cx; bsz = zx; }
+    }
+    bool moves = false;
+    if (act && gl == 0) {
+        lc.vertices++;
+        lc.edges += t.deg;
+        const double gain = bestc == EMPTY ? 0.0 : sc.gain(best);
+        moves = gain > 0.0 && bestc != lf && !(need_size && bsz == 1 && bestc > d);
+        if (moves) {
+            lc.moved++;
+            lc.marked += t.deg;
+            lc.dq += gain;
+            add_graph_gain(a, t.i, gain);
+        }
+    }
+    const unsigned bal = __ballot_sync(FULL, moves);
+    if (moves) mv[nmv + __popc(bal & ((1u << lane) - 1u))] = LevelMover{t.b, t.K, t.i, bestc, d, t.deg};
+    nmv += __popc(bal);
+}
+
+// One thread moves vertex i from d to c after the wave's barrier.
+__device__ __forceinline__ void level_apply(const MoveArgs &a, uint32_t i, uint32_t c, uint32_t d, double Ki, int it) {
+    a.C[i] = c;
+    a.left[i] = d;
+    a.left_it[i] = it;
+    atomicAdd(a.Sig + d, -Ki);
+    atomicAdd(a.Sig + c, Ki);
+    atomicSub(a.size + d, 1u);
+    atomicAdd(a.size + c, 1u);
+}
+
+template <typename WT, bool F64>
+__global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, LevelArgs v) {
+    using V = typename std::conditional<F64, double, float>::type;
+    constexpr int CAP = LEVEL_CAP<F64>;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    LevelSmem<F64> &sm = *reinterpret_cast<LevelSmem<F64> *>(dyn_smem);
+    __shared__ int s_it;
+    __shared__ double s_red[32];
+    __shared__ uint32_t s_bv[LEVEL_BMOVERS], s_bc[LEVEL_BMOVERS], s_bn;
+    const uint32_t lb = blockIdx.x, nb = gridDim.x;
+    const uint32_t tid = lb * LEVEL_THREADS + threadIdx.x, nt = nb * LEVEL_THREADS;
+    const uint32_t wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // warp w of CTA b is number w * nb + b, so that few tasks spread over the CTAs
+    const uint32_t wb = wid * nb + lb, wn = nb * LEVEL_WARPS;
+    unsigned char *ws = sm.tables + wid * warp_tables<32, W512_CAP, V>;
+    LevelMover *mv = sm.mv[wid];
+    const double m0 = *a.m, inv0 = 1.0 / m0;
+    for (int t = threadIdx.x; t <= NUM_CLS * v.W; t += LEVEL_THREADS) sm.start[t] = v.start[t];
+    __syncthreads();
+    // the block classes' movers go to the CTA's list, applied after the barrier
+    MoveArgs ab = a;
+    ab.iteration = &s_it;
+    ab.mv_vtx = s_bv;
+    ab.mv_cmt = s_bc;
+    ab.mv_cnt = &s_bn;
+    ab.mark = nullptr;
+    auto cls = [&](int k, int wv, uint32_t &beg) {
+        beg = sm.start[k * v.W + wv];
+        return sm.start[k * v.W + wv + 1] - beg;
+    };
+    auto next_wave = [&](int wv) {  // the next wave after wv with a vertex, or W
+        for (wv++; wv < v.W; wv++) {
+            uint32_t tot = 0, beg;
+            for (int k = 0; k < NUM_CLS; k++) tot += cls(k, wv, beg);
+            if (tot) break;
+        }
+        return wv;
+    };
+    LocalCtr lc;
+    LevelTask<WT> t0;
+    const int wave0 = next_wave(-1);
+    int fetched = wave0;
+    if (wave0 < v.W) level_fetch(a, v.list, sm.start, v.W, wave0, wb, m0, inv0, t0);
+    int it = 0;
+    for (;; it++) {
+        if (threadIdx.x == 0) s_it = it;
+        // sums of a sweep rotate through three slots: the next sweep's was
+        // last read before this sweep's first barrier
+        const int sum = it % 3;
+        if (tid == 0) {
+            v.dq[(it + 1) % 3] = 0.0;
+            v.nlive[(it + 1) % 3] = 0;
+        }
+        lc.dq = 0.0;
+        const int rep = it == 0 ? v.R : 1;
+        for (int wv = wave0; wv < v.W;) {
+            const int after = next_wave(wv);
+            uint32_t tasks = 0, nblk = 0, beg;
+            for (int k = CLS_G4; k <= CLS_W512; k++) tasks += level_tasks(k, cls(k, wv, beg));
+            for (int k = CLS_BLOCK; k <= CLS_HUGE; k++) nblk += cls(k, wv, beg);
+            for (int r = 0; r < rep; r++) {
+                uint32_t nmv = 0;
+                if (nblk) {  // the same for every CTA; the heaviest first: a whole CTA per vertex
+                    if (threadIdx.x == 0) s_bn = 0;
+                    __syncthreads();
+                    for (int k = CLS_HUGE; k >= CLS_BLOCK; k--) {
+                        const uint32_t cnt = cls(k, wv, beg);
+                        const uint32_t slots = k == CLS_BLOCK ? 4096u : (uint32_t)CAP;
+                        if (cnt) block_body<CAP, WT, F64, 2>(ab, v.list + beg, cnt, lb, nb, sm.tables, lc, slots, k == CLS_HUGE);
+                    }
+                }
+                if (wb < tasks) level_visit<WT, F64>(a, t0, it, ws, mv, nmv, lc);
+                for (uint32_t x = wb + wn; x < tasks; x += wn) {
+                    LevelTask<WT> t;
+                    level_fetch(a, v.list, sm.start, v.W, wv, x, m0, inv0, t);
+                    level_visit<WT, F64>(a, t, it, ws, mv, nmv, lc);
+                }
+                cluster_arrive();  // every vertex of the wave has decided
+                __syncwarp();      // the warp's movers are visible to its lanes
+                if (r + 1 == rep) {
+                    const int nx = after < v.W ? after : wave0;
+                    if (nx != fetched) level_fetch(a, v.list, sm.start, v.W, nx, wb, m0, inv0, t0);
+                    fetched = nx;
+                }
+                cluster_wait();
+                for (uint32_t x = lane; x < nmv; x += 32) {
+                    const LevelMover q = mv[x];
+                    level_apply(a, q.i, q.c, q.d, q.K, it);
+                }
+                // marks: four lanes per mover, the whole warp for the long rows
+                for (uint32_t x = lane >> 2; x < nmv; x += 8) {
+                    const LevelMover q = mv[x];
+                    if (q.deg > 32) continue;
+                    for (uint32_t p = lane & 3; p < q.deg; p += 4) {
+                        const uint32_t j = __ldg(a.tgt + q.b + p);
+                        if (j != q.i) a.act[j] = 1;
+                    }
+                }
+                for (uint32_t x = 0; x < nmv; x++) {
+                    const LevelMover q = mv[x];
+                    if (q.deg <= 32) continue;
+                    for (uint32_t p = lane; p < q.deg; p += 32) {
+                        const uint32_t j = __ldg(a.tgt + q.b + p);
+                        if (j != q.i) a.act[j] = 1;
+                    }
+                }
+                if (nblk) {
+                    __syncthreads();
+                    for (uint32_t x = 0; x < s_bn; x++) {
+                        const uint32_t i = s_bv[x];
+                        const uint64_t b = a.off[i], e = a.off[i + 1];
+                        if (threadIdx.x == 0) level_apply(a, i, s_bc[x], ldcg(a.C + i), a.K[i], it);
+                        for (uint64_t p = b + threadIdx.x; p < e; p += LEVEL_THREADS) {
+                            const uint32_t j = __ldg(a.tgt + p);
+                            if (j != i) a.act[j] = 1;
+                        }
+                    }
+                    __syncthreads();
+                }
+                cluster_arrive();  // the wave's moves and marks are in place
+                cluster_wait();
+            }
+            wv = after;
+        }
+        // the sweep's gain; then every CTA takes the same decision
+        const double dq = block_sum<double>(lc.dq, s_red);
+        if (threadIdx.x == 0 && dq != 0.0) atomicAdd(v.dq + sum, dq);
+        cluster_arrive();
+        cluster_wait();
+        if (!v.G) {
+            if (it + 1 >= v.max_it || __ldcg(v.dq + sum) <= v.tau) break;
+            continue;
+        }
+        uint32_t alive = 0;
+        for (uint32_t g = tid; g < v.G; g += nt) {
+            if (!ldcg(v.live + g)) continue;
+            v.li[g] = it + 1;
+            if (__ldcg(a.dq_g + g) <= v.tau) v.live[g] = 0;
+            else alive = 1;
+            a.dq_g[g] = 0.0;
+        }
+        alive = (uint32_t)__syncthreads_count(alive != 0);
+        if (threadIdx.x == 0 && alive) atomicAdd(v.nlive + sum, alive);
+        cluster_arrive();
+        cluster_wait();
+        if (it + 1 >= v.max_it || !__ldcg(v.nlive + sum)) break;
+        for (uint32_t i = tid; i < v.n; i += nt)
+            if (!ldcg(v.live + a.gid[i])) a.act[i] = 0;
+        cluster_arrive();
+        cluster_wait();
+    }
+    lc.dq = 0.0;  // reported per sweep
+    flush_counters(lc, a.ctr);
+    if (tid == 0) *v.iterations = it + 1;
 }
 
 // --------------------------------------------------------------------------
@@ -936,7 +1348,7 @@ __global__ void __launch_bounds__(256) k_hub_score(MoveArgs a, HubArgs h) {
         const uint32_t *occ = h.occ + h.pool_off[t];
         uint64_t k1 = min(k0 + HUB_CHUNK, (uint64_t)h.occ_n[t]);
         SC sc = make_score<F64>(a.K[i], (double)kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
-                                vertex_inv_m(a, i, inv0));
+                                vertex_inv_m(a, i, inv0), true);
         S best = -INFINITY;
         uint32_t bestc = EMPTY;
         // U entries per thread per round; each level of the gather chain
@@ -1017,7 +1429,7 @@ __global__ void k_hub_decide(MoveArgs a, HubArgs h) {
             double Ki = a.K[i];
             uint64_t deg = a.off[i + 1] - a.off[i];
             const double m = vertex_m(a, i, m0);
-            SC sc = make_score<F64>(Ki, (double)kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, inv0));
+            SC sc = make_score<F64>(Ki, (double)kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, inv0), true);
             double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
             int mv = 0;
             if (gain > 0.0) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
@@ -1422,6 +1834,90 @@ bool sweep_persistent(const DevGraph &g, const Classes &cl, MoveBuffers &mb, boo
                                        : launch_persistent<float, false>(a, cl, g.n, mb, iteration, s);
     return fp64 ? launch_persistent<double, true>(a, cl, g.n, mb, iteration, s)
                 : launch_persistent<double, false>(a, cl, g.n, mb, iteration, s);
+}
+
+template <typename WT, bool F64>
+static bool launch_level(const MoveArgs &a, const LevelArgs &v, int ctas_needed, cudaStream_t s) {
+    constexpr size_t smem = sizeof(LevelSmem<F64>);
+    static int ctas[64] = {0};  // CTAs of the cluster, per device (-1: cannot run)
+    int dev = 0;
+    GSP_CUDA(cudaGetDevice(&dev));
+    dev &= 63;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(LEVEL_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const auto fn = k_move_level<WT, F64>;
+    if (!ctas[dev]) {
+        GSP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        GSP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        int found = -1;
+        for (int c = LEVEL_CTAS; c >= 8 && found < 0; c /= 2) {
+            at[0].val.clusterDim.x = c;
+            cfg.gridDim = dim3(c);
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) found = c;
+            else cudaGetLastError();
+        }
+        ctas[dev] = found;
+    }
+    if (ctas[dev] < ctas_needed) return false;
+    at[0].val.clusterDim.x = ctas[dev];
+    cfg.gridDim = dim3(ctas[dev]);
+    GSP_CUDA(cudaLaunchKernelEx(&cfg, fn, a, v));
+    count_launch();
+    return true;
+}
+
+// Most stored entries of a graph that one cluster moves.  Measured on GB300,
+// whole local-moving phase (gsp_local_move), launches against cluster:
+// planted 2 K vertices / 30 K entries 3.36 against 1.07 ms, 10 K / 151 K 4.02
+// against 1.30, 20 K / 995 K 2.54 against 1.94, 60 K / 906 K 4.44 against 3.68,
+// 300^2 grid 2.84 against 1.48; R-MAT 3 K / 75 K 3.96 against 1.90, 60 K / 879 K
+// 5.03 against 4.39, 12 K / 1.32 M 5.70 against 5.98.  The float64 mode's
+// divisions need more SMs sooner: planted 10 K / 151 K 5.16 against 3.15, R-MAT
+// 9 K / 252 K 10.7 against 7.4, planted 20 K / 542 K 4.30 against 5.46.
+constexpr uint64_t LEVEL_MAX_EDGES = 1u << 20, LEVEL_MAX_EDGES_F64 = 1u << 18;
+
+bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64, bool rule, double tau, int max_it,
+                LevelResult &out, uint32_t G, uint8_t *live, int *li, cudaStream_t s) {
+    if (g.nnz > (fp64 ? LEVEL_MAX_EDGES_F64 : LEVEL_MAX_EDGES) || mb.feat_kept || mb.choice || !cl.dstart) return false;
+    // a vertex's communities must fit the block classes' table
+    const uint32_t cap = fp64 ? LEVEL_CAP<true> : LEVEL_CAP<false>;
+    if (g.n > cap * 3 / 4 && (cl.cls_count(CLS_HUGE) || (fp64 && cl.cls_count(CLS_BIG)))) return false;
+    // a wave must fit the warps' task and mover lists, and the CTAs' lists of block-class movers
+    int need = 1;
+    for (int wv = 0; wv < cl.W; wv++) {
+        uint64_t tasks = 0, blk = 0;
+        for (int k = CLS_G4; k <= CLS_W512; k++) tasks += level_tasks(k, cl.count(k, wv));
+        // a CTA takes its share of each block class, rounded up
+        for (int k = CLS_BLOCK; k <= CLS_HUGE; k++) blk += cl.count(k, wv);
+        const uint64_t c = std::max((tasks + LEVEL_TASKS * LEVEL_WARPS - 1) / (LEVEL_TASKS * LEVEL_WARPS),
+                                    (blk + LEVEL_BMOVERS - 4) / (LEVEL_BMOVERS - 3));
+        if (c > LEVEL_CTAS) return false;
+        need = std::max(need, (int)c);
+    }
+    MoveArgs a = make_move_args(g, mb, true, rule, 0, max_it);
+    struct Scratch { double dq[3]; uint32_t nlive[3]; int iterations; };
+    static_assert(sizeof(Scratch) <= sizeof(uint32_t) * MAX_WAVES * MAX_REPEATS, "the persistent sweep's counters hold it");
+    Scratch *d = reinterpret_cast<Scratch *>(mb.mv_cnts);
+    GSP_CUDA(cudaMemsetAsync(d, 0, sizeof(Scratch), s));
+    GSP_CUDA(cudaMemsetAsync(mb.ctr, 0, sizeof(MoveCounters), s));
+    const LevelArgs v{cl.list, cl.dstart, cl.W, std::min(std::max(mb.repeats, 1), MAX_REPEATS), g.n, tau, max_it,
+                      d->dq, &d->iterations, G, live, li, d->nlive};
+    bool ran;
+    if (g.wt == GSP_W_F32) ran = fp64 ? launch_level<float, true>(a, v, need, s) : launch_level<float, false>(a, v, need, s);
+    else ran = fp64 ? launch_level<double, true>(a, v, need, s) : launch_level<double, false>(a, v, need, s);
+    if (ran) {
+        GSP_CUDA(cudaMemcpyAsync(&out.iterations, &d->iterations, sizeof(int), cudaMemcpyDeviceToHost, s));
+        GSP_CUDA(cudaMemcpyAsync(&out.ctr, mb.ctr, sizeof(MoveCounters), cudaMemcpyDeviceToHost, s));
+    }
+    return ran;
 }
 
 void move_wave(const DevGraph &g, const Classes &cl, MoveBuffers &mb, int wave, bool sync, bool fp64, bool rule,
