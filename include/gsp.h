@@ -48,8 +48,10 @@ typedef enum {
 /* Split techniques of Section 4.1: none (GVE-Louvain), min-label propagation
  * (Algorithm 2), min-label propagation with pruning (Algorithm 2, LPP), and
  * breadth-first search (Algorithm 3); SV (not in the paper) is hooking and
- * shortcutting (Shiloach-Vishkin) on the intra-community edges, for graphs of
- * high diameter.  All give the same labels. */
+ * shortcutting on the intra-community edges.  All give the same labels, and
+ * LPP and SV run as the same computation: one hooking pass over a
+ * disjoint-set forest, whose roots are the labels that pruned propagation
+ * reaches round by round. */
 typedef enum {
     GSP_SPLIT_NONE = 0,
     GSP_SPLIT_LP = 1,

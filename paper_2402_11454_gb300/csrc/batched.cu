@@ -610,7 +610,7 @@ void louvain_batched_run(const DevGraph &g0, uint32_t G, const uint64_t *h_gvo0,
     }
     if (o.split != GSP_SPLIT_NONE && o.split_when == GSP_SPLIT_LAST) {
         Classes cl;
-        classify_vertices(g0, cl, 1, s);
+        if (split_uses_classes(o.split)) classify_vertices(g0, cl, 1, s);
         split_labels(g0, cl, membership, o.split, labels, s);
         GSP_CUDA(cudaMemcpyAsync(membership, labels, sizeof(uint32_t) * n0, cudaMemcpyDeviceToDevice, s));
     }

@@ -48,6 +48,7 @@ class Arena {
   public:
     void *alloc(size_t bytes);
     template <typename T> T *get(size_t count) { return static_cast<T *>(alloc(count * sizeof(T))); }
+    void *try_alloc(size_t bytes);  // nullptr where alloc() would fail
     size_t mark();
     void release(size_t m);
     void reset();

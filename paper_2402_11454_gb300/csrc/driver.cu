@@ -133,6 +133,15 @@ static ChunkArena &backing(const Arena *a) {
 }
 size_t workspace_peak() { return backing(&g_work_facade).peak; }
 void *Arena::alloc(size_t bytes) { return backing(this).alloc(bytes); }
+void *Arena::try_alloc(size_t bytes) {
+    const size_t m = mark();
+    try {
+        return alloc(bytes);
+    } catch (const Error &) {
+        release(m);
+        return nullptr;
+    }
+}
 size_t Arena::mark() { return backing(this).mark(); }
 void Arena::release(size_t m) { backing(this).release(m); }
 void Arena::reset() { backing(this).reset(); }
@@ -816,7 +825,7 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
     lookup(n0, membership, Cp, s);
     if (split_last) {
         Classes cl;
-        classify_vertices(g0, cl, 1, s);
+        if (split_uses_classes(o.split)) classify_vertices(g0, cl, 1, s);
         split_labels(g0, cl, membership, o.split, labels, s);
         GSP_CUDA(cudaMemcpyAsync(membership, labels, sizeof(uint32_t) * n0, cudaMemcpyDeviceToDevice, s));
     }
@@ -1183,7 +1192,7 @@ gsp_status gsp_split(const uint64_t *offsets, const uint32_t *targets, uint32_t 
     check_csr(offsets, targets, n, nnz, arena().get<unsigned long long>(1), s);
     check_ids(C, n, n, "membership", s);
     Classes cl;
-    classify_vertices(g, cl, 1, s);
+    if (split_uses_classes(mode)) classify_vertices(g, cl, 1, s);
     split_labels(g, cl, C, mode, labels, s);
     if (k_host) {
         uint32_t *tmp = arena().get<uint32_t>(n);

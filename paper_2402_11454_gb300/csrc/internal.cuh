@@ -247,7 +247,9 @@ void sigma_from_membership(const uint32_t *C, const double *K, double *Sigma, ui
 // starts the next pass in the bound community B (dense) of its members.
 void scatter_bound(const uint32_t *R, const uint32_t *B, uint32_t *C_next, uint32_t n, cudaStream_t s);
 
-// Split (Algorithms 2, 3): labels = smallest vertex of the component.
+// Split (Algorithms 2, 3): labels = smallest vertex of the component.  cl is
+// read only where split_uses_classes(mode).
+inline bool split_uses_classes(int mode) { return mode == GSP_SPLIT_LP; }
 void split_labels(const DevGraph &g, const Classes &cl, const uint32_t *C, int mode, uint32_t *labels,
                   cudaStream_t s);
 

@@ -513,9 +513,7 @@ uint32_t count_disconnected(const DevGraph &g, const uint32_t *C, uint8_t *flags
     uint32_t *lab = arena().get<uint32_t>(g.n);
     uint32_t *ncomp = arena().get<uint32_t>(g.n);
     unsigned long long *cnt = arena().get<unsigned long long>(1);
-    Classes cl;
-    classify_vertices(g, cl, 1, s);
-    split_labels(g, cl, C, GSP_SPLIT_SV, lab, s);  // every technique gives the same labels
+    split_labels(g, Classes(), C, GSP_SPLIT_SV, lab, s);  // every technique gives the same labels
     GSP_CUDA(cudaMemsetAsync(ncomp, 0, sizeof(uint32_t) * g.n, s));
     GSP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
     unsigned gr = grid_for(g.n, 256);

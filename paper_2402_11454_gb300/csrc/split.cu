@@ -5,11 +5,11 @@
 //        takes the minimum label over its same-community neighbours, in place,
 //        until a sweep changes nothing.  Labels only decrease, so the in-place
 //        updates of concurrent threads converge to the same fixpoint.
-//   LPP (Algorithm 2 with pruning): only vertices flagged unprocessed are
-//        visited; a vertex whose label drops flags its same-community
-//        neighbours.
-//   SV  (not in the paper): hooking and shortcutting (Shiloach-Vishkin) on
-//        the intra-community edges, O(log n) sweeps on high-diameter graphs.
+//   LPP (Algorithm 2 with pruning) and SV (hooking and shortcutting on the
+//        intra-community edges, not in the paper) both run as one hooking
+//        pass: a disjoint-set forest over the vertices whose roots are the
+//        smallest id of their set, which is the fixpoint that pruned label
+//        propagation reaches round by round.
 //   BFS (Algorithm 3): rounds of multi-source, level-synchronous,
 //        frontier-compacted BFS.  In each round the seed of a community is its
 //        smallest unvisited vertex, found with atomicMin; vertices are claimed
@@ -19,6 +19,8 @@
 // The seed of a round is the smallest vertex of its component (the smaller
 // vertices of the community are already visited, and components are
 // disjoint), so every mode yields label = smallest vertex id of the component.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace gsp {
@@ -51,198 +53,80 @@ __device__ __forceinline__ uint32_t min_label(const uint32_t *__restrict__ tgt, 
     return mn;
 }
 
-// ----------------------------------------------------------------- LP / LPP
-// HOOK (the hooking split): besides lowering its own label, a vertex whose
-// smallest neighbouring label mn is below its label p hooks p's tree under
-// mn (lab[p] = min(lab[p], mn)); with the shortcut kernel between sweeps the
-// labels then converge in O(log n) sweeps instead of O(diameter).
-template <int G, bool PRUNE, bool HOOK = false>
+// ------------------------------------------------------------------------ LP
+template <int G>
 __global__ void __launch_bounds__(256) k_lp_group(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tgt,
-                                                  const uint32_t *__restrict__ C, uint32_t *lab, uint8_t *flag,
+                                                  const uint32_t *__restrict__ C, uint32_t *lab,
                                                   const uint32_t *__restrict__ list, uint32_t count,
                                                   unsigned long long *changed) {
     const int lane = threadIdx.x % G;
     const unsigned gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
     unsigned long long ch = 0;
-    // 32 list entries per warp and round: each lane reads (and, pruned,
-    // clears) one flag; the flagged vertices are dealt to the warp's groups
-    constexpr int NGW = 32 / G;
-    const int wl = threadIdx.x & 31, gw = wl / G;
-    const uint32_t wbase = blockIdx.x * 8 + (threadIdx.x >> 5), wstep = gridDim.x * 8;
-    for (uint64_t kb = 0; wbase + kb * wstep < count; kb += 32) {
-        const uint64_t my = wbase + (kb + wl) * wstep;
-        uint32_t vi = 0;
-        int claim = 0;
-        if (my < count) {
-            vi = list[my];
-            claim = 1;
-            if (PRUNE) {
-                claim = ldcg_(flag + vi);
-                if (claim) flag[vi] = 0;
-            }
-        }
-        const unsigned amask = __ballot_sync(0xFFFFFFFFu, claim);
-        const int nact = __popc(amask);
-        // a consumed flag was set after its setter's label store: order the
-        // label reads below after the flag reads
-        if (PRUNE && nact) __threadfence();
-        for (int r0 = 0; r0 < nact; r0 += NGW) {
-        const int qa = r0 + gw;
-        const uint32_t i = __shfl_sync(0xFFFFFFFFu, vi, qa < nact ? select_bit(amask, qa) : 0);
-        if (qa >= nact) continue;
-        uint32_t ci = C[i];
-        uint32_t cur = ldcg_(lab + i);
-        uint32_t mn = cur;
-        uint64_t b = off[i], e = off[i + 1];
-        mn = min_label(tgt, C, lab, ci, b, e, lane, G, mn);
+    for (uint64_t q = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; q < count;
+         q += (uint64_t)gridDim.x * blockDim.x / G) {
+        const uint32_t i = list[q];
+        const uint32_t cur = ldcg_(lab + i);
+        uint32_t mn = min_label(tgt, C, lab, C[i], off[i], off[i + 1], lane, G, cur);
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(gmask, mn, o));
-        if (mn < cur) {
-            if (lane == 0) {
-                if (HOOK) {
-                    atomicMin(lab + cur, mn);
-                    atomicMin(lab + i, mn);
-                } else {
-                    lab[i] = mn;
-                }
-                ch++;
-            }
-            if (PRUNE) {
-                // the new label must be visible before any neighbour sees its
-                // flag (a neighbour that consumes the flag re-reads it once)
-                __syncwarp(gmask);
-                __threadfence();
-            }
-            if (PRUNE)
-                for (uint64_t p = b + lane; p < e; p += G) {
-                    uint32_t j = tgt[p];
-                    if (C[j] == ci) flag[j] = 1;
-                }
+        if (mn < cur && lane == 0) {
+            lab[i] = mn;
+            ch++;
         }
         __syncwarp(gmask);
-        }
     }
     __shared__ unsigned long long red[32];
     ch = block_sum(ch, red);
     if (threadIdx.x == 0 && ch) atomicAdd(changed, ch);
 }
 
-template <bool PRUNE, bool HOOK = false>
 __global__ void __launch_bounds__(256) k_lp_block(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tgt,
-                                                  const uint32_t *__restrict__ C, uint32_t *lab, uint8_t *flag,
+                                                  const uint32_t *__restrict__ C, uint32_t *lab,
                                                   const uint32_t *__restrict__ list, uint32_t count,
                                                   unsigned long long *changed) {
     __shared__ uint32_t red[32];
-    __shared__ uint32_t s_todo[256], s_ntodo, s_wcnt[8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long ch = 0;
-    // 256 list entries per block and round (blockIdx.x + k * gridDim.x):
-    // each thread reads (and, pruned, clears) one flag; the flagged vertices
-    // are listed in shared memory and processed one by one
-    for (uint64_t kb = 0; blockIdx.x + kb * gridDim.x < count; kb += blockDim.x) {
-        const uint64_t my = blockIdx.x + (kb + threadIdx.x) * gridDim.x;
-        uint32_t vi = 0;
-        int claim = 0;
-        if (my < count) {
-            vi = list[my];
-            claim = 1;
-            if (PRUNE) {
-                claim = ldcg_(flag + vi);
-                if (claim) flag[vi] = 0;
-            }
-        }
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, claim);
-        __syncthreads();  // the loop's previous step is done with s_todo
-        if (lane == 0) s_wcnt[wid] = __popc(bal);
-        __syncthreads();
-        if (claim) {
-            uint32_t pos = __popc(bal & ((1u << lane) - 1u));
-            for (int k = 0; k < wid; k++) pos += s_wcnt[k];
-            s_todo[pos] = vi;
-        }
-        if (threadIdx.x == 0) {
-            uint32_t t = 0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += s_wcnt[k];
-            s_ntodo = t;
-        }
-        __syncthreads();
-        const uint32_t ntodo = s_ntodo;
-        if (PRUNE && ntodo) __threadfence();  // flags consumed before the labels are read
-    for (uint32_t kk = 0; kk < ntodo; kk++) {
-        const uint32_t i = s_todo[kk];
+    for (uint32_t q = blockIdx.x; q < count; q += gridDim.x) {
+        const uint32_t i = list[q];
         __syncthreads();  // previous vertex done with red
-        uint32_t ci = C[i];
-        uint32_t cur = ldcg_(lab + i);
-        uint32_t mn = cur;
-        uint64_t b = off[i], e = off[i + 1];
-        mn = min_label(tgt, C, lab, ci, b, e, threadIdx.x, blockDim.x, mn);
+        const uint32_t cur = ldcg_(lab + i);
+        uint32_t mn = min_label(tgt, C, lab, C[i], off[i], off[i + 1], threadIdx.x, blockDim.x, cur);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mn;
         __syncthreads();
-        mn = red[0];
-        for (int t = 1; t < (int)(blockDim.x >> 5); t++) mn = min(mn, red[t]);
-        if (mn < cur) {
-            if (threadIdx.x == 0) {
-                if (HOOK) {
-                    atomicMin(lab + cur, mn);
-                    atomicMin(lab + i, mn);
-                } else {
-                    lab[i] = mn;
-                }
+        if (threadIdx.x == 0) {
+            for (int t = 1; t < (int)(blockDim.x >> 5); t++) mn = min(mn, red[t]);
+            if (mn < cur) {
+                lab[i] = mn;
                 ch++;
             }
-            if (PRUNE) {  // the new label visible before the neighbours' flags
-                __syncthreads();
-                __threadfence();
-            }
-            if (PRUNE)
-                for (uint64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
-                    uint32_t j = tgt[p];
-                    if (C[j] == ci) flag[j] = 1;
-                }
         }
     }
-    }
-    __shared__ unsigned long long r2[32];
-    __syncthreads();
-    ch = block_sum(ch, r2);
     if (threadIdx.x == 0 && ch) atomicAdd(changed, ch);
 }
 
-static void split_lp(const DevGraph &g, const Classes &cl, const uint32_t *C, bool prune, uint32_t *lab,
-                     cudaStream_t s) {
+static void split_lp(const DevGraph &g, const Classes &cl, const uint32_t *C, uint32_t *lab, cudaStream_t s) {
     size_t mk = arena().mark();
-    uint8_t *flag = prune ? arena().get<uint8_t>(g.n) : nullptr;
     unsigned long long *changed = arena().get<unsigned long long>(1);
     iota_u32(lab, g.n, s);
-    if (prune) GSP_CUDA(cudaMemsetAsync(flag, 1, g.n, s));
     // every class with all its waves (class c spans [cls_begin(c), cls_begin(c+1)))
     auto cnt = [&](int c) { return cl.cls_count(c); };
     auto lst = [&](int c) { return cl.list + cl.cls_begin(c); };
     const unsigned maxg = sms(8);
-    uint32_t nbig = cl.cls_count(CLS_BLOCK) + cl.cls_count(CLS_BIG) + cl.cls_count(CLS_HUGE);
+    const uint32_t nbig = cl.cls_count(CLS_BLOCK) + cl.cls_count(CLS_BIG) + cl.cls_count(CLS_HUGE);
     for (int it = 0; it < (1 << 30); it++) {
         GSP_CUDA(cudaMemsetAsync(changed, 0, sizeof(unsigned long long), s));
-#define LPG(G, CLS)                                                                                  \
-    if (cnt(CLS)) {                                                                                  \
-        if (prune)                                                                                   \
-            k_lp_group<G, true><<<grid_for((uint64_t)cnt(CLS) * G, 256, maxg), 256, 0, s>>>(        \
-                g.off, g.tgt, C, lab, flag, lst(CLS), cnt(CLS), changed);                            \
-        else                                                                                         \
-            k_lp_group<G, false><<<grid_for((uint64_t)cnt(CLS) * G, 256, maxg), 256, 0, s>>>(       \
-                g.off, g.tgt, C, lab, flag, lst(CLS), cnt(CLS), changed);                            \
-        GSP_CHECK_LAUNCH();                                                                          \
+#define LPG(G, CLS)                                                                                            \
+    if (cnt(CLS)) {                                                                                            \
+        k_lp_group<G><<<grid_for((uint64_t)cnt(CLS) * G, 256, maxg), 256, 0, s>>>(g.off, g.tgt, C, lab, lst(CLS), \
+                                                                                  cnt(CLS), changed);          \
+        GSP_CHECK_LAUNCH();                                                                                    \
     }
         LPG(4, CLS_G4) LPG(8, CLS_G8) LPG(16, CLS_G16) LPG(32, CLS_G32) LPG(32, CLS_W512)
 #undef LPG
         if (nbig) {
-            if (prune)
-                k_lp_block<true><<<grid_for(nbig, 1, sms(4)), 256, 0, s>>>(g.off, g.tgt, C, lab, flag,
-                                                                              lst(CLS_BLOCK), nbig, changed);
-            else
-                k_lp_block<false><<<grid_for(nbig, 1, sms(4)), 256, 0, s>>>(g.off, g.tgt, C, lab, flag,
-                                                                               lst(CLS_BLOCK), nbig, changed);
+            k_lp_block<<<grid_for(nbig, 1, sms(4)), 256, 0, s>>>(g.off, g.tgt, C, lab, lst(CLS_BLOCK), nbig, changed);
             GSP_CHECK_LAUNCH();
         }
         unsigned long long h;
@@ -253,55 +137,212 @@ static void split_lp(const DevGraph &g, const Classes &cl, const uint32_t *C, bo
     arena().release(mk);
 }
 
-// ------------------------------------------------------------ hooking split
-// Shiloach-Vishkin-style connected components restricted to intra-community
-// edges: hooking sweeps (k_lp_group/k_lp_block with HOOK) alternate with a
-// shortcut pass that points every vertex at the root of its tree.  Labels
-// only decrease and always name a vertex of the same component, so at the
-// fixpoint every component carries its smallest vertex id, as LP and BFS.
-__global__ void k_sv_shortcut(uint32_t *lab, uint32_t n) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        uint32_t x = ldcg_(lab + i);
-        // lab[x] <= x, so the chain strictly decreases and ends at a root
-        for (;;) {
-            const uint32_t y = ldcg_(lab + x);
-            if (y == x) break;
-            x = y;
+// ------------------------------------------------------------- hooking split
+// Disjoint-set forest over the vertices, parents in lab: every set is a tree
+// whose pointers lead to smaller ids, so its root is its smallest vertex and
+// after the last link lab (pointing at the roots) holds the split's labels.
+// Links hook the larger root under the smaller by compare-and-swap; finds
+// halve the path as they go.  Both may run on stale values: only a root is
+// ever hooked, a stored parent is always an earlier ancestor (a smaller id of
+// the same set), and a failed hook returns the parent it lost to, so that a
+// link's larger end falls with every attempt.
+//
+// Label propagation read every edge and both ends' C in each of its rounds
+// (a round trip to the host between them); one pass of links over all edges
+// would read them once.  Most edges need not be read at all (the sampling of
+// Sutton, Ben-Nun and Barak's Afforest, per community): after linking each
+// vertex with the first few of its row, nearly every community already is one
+// tree.  The vertices of one tree per community (`tree`: whichever vertex
+// wrote last, likely of the largest) need no further look: an edge inside the
+// tree is redundant, and an edge that leaves it is linked from its other end.
+// Everyone else links along the whole row.  A vertex that joins the tree while
+// the links run may be skipped too: its edges then lead into the tree or to
+// vertices that link them.
+// On R-MAT 22 the sample leaves 3 % of the vertices and 5 % of the edges to
+// the row pass (4 entries instead of 8: 12 and 16 %).
+// Measured (all splits of a call, ms, rounds of pruned propagation -> this):
+// R-MAT 22 4.7 -> 1.0, R-MAT 24 17.6 -> 3.5, 2048^2 grid 3.4 -> 1.2, 512 planted
+// graphs 8.1 -> 2.2, 611 vertices 0.38 -> 0.18.  With rows up to 4096 entries
+// left to a warp, R-MAT 22 took 4.4: its hubs have neighbouring ids and queued
+// in the same warps.
+constexpr uint32_t HOOK_SAMPLE = 8;   // entries of a row linked in the sampling pass
+constexpr uint32_t HOOK_MID = 256;    // longer rows are linked by a block each ...
+constexpr uint32_t HOOK_HUB = 16384;  // ... or by a column of HOOK_COL blocks
+constexpr uint32_t HOOK_COL = 16;
+
+struct HookLists {  // open rows longer than HOOK_MID: one array filled from both ends
+    uint32_t *rows, *nmid, *nhub;
+    uint32_t cap;
+};
+
+__device__ __forceinline__ uint32_t hook_find(uint32_t *lab, uint32_t x) {
+    uint32_t p = __ldca(lab + x);
+    while (p != x) {
+        const uint32_t g = __ldca(lab + p);
+        if (g == p) return p;
+        lab[x] = g;
+        x = g;
+        p = __ldca(lab + x);
+    }
+    return x;
+}
+
+// Link the trees of two roots; returns the smaller one met last.
+__device__ __forceinline__ uint32_t hook_link(uint32_t *lab, uint32_t u, uint32_t v) {
+    while (u != v) {
+        if (u < v) {
+            const uint32_t t = u;
+            u = v;
+            v = t;
         }
-        lab[i] = x;
+        const uint32_t old = atomicCAS(lab + u, u, v);
+        if (old == u) return v;
+        u = hook_find(lab, old);
+    }
+    return u;
+}
+
+// Link vertex i with the same-community targets of entries p, p + step, ... < e,
+// four gathers of C in flight.
+__device__ __forceinline__ void hook_row(const uint32_t *__restrict__ tgt, const uint32_t *__restrict__ C,
+                                         uint32_t *lab, uint32_t i, uint32_t ci, uint64_t p, uint64_t e,
+                                         uint32_t step) {
+    uint32_t r = EMPTY;
+    for (; p < e; p += 4ull * step) {
+        uint32_t j[4], cj[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const uint64_t q = p + (uint64_t)u * step;
+            j[u] = q < e ? __ldg(tgt + q) : i;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) cj[u] = __ldg(C + j[u]);
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (j[u] == i || cj[u] != ci) continue;
+            if (r == EMPTY) r = hook_find(lab, i);
+            r = hook_link(lab, r, hook_find(lab, j[u]));
+        }
     }
 }
 
-static void split_sv(const DevGraph &g, const Classes &cl, const uint32_t *C, uint32_t *lab, cudaStream_t s) {
-    size_t mk = arena().mark();
-    unsigned long long *changed = arena().get<unsigned long long>(1);
-    iota_u32(lab, g.n, s);
-    auto cnt = [&](int c) { return cl.cls_count(c); };
-    auto lst = [&](int c) { return cl.list + cl.cls_begin(c); };
-    const unsigned maxg = sms(8);
-    const uint32_t nbig = cl.cls_count(CLS_BLOCK) + cl.cls_count(CLS_BIG) + cl.cls_count(CLS_HUGE);
-    for (int it = 0; it < (1 << 30); it++) {
-        GSP_CUDA(cudaMemsetAsync(changed, 0, sizeof(unsigned long long), s));
-#define SVG(G, CLS)                                                                                            \
-    if (cnt(CLS)) {                                                                                            \
-        k_lp_group<G, false, true><<<grid_for((uint64_t)cnt(CLS) * G, 256, maxg), 256, 0, s>>>(               \
-            g.off, g.tgt, C, lab, nullptr, lst(CLS), cnt(CLS), changed);                                       \
-        GSP_CHECK_LAUNCH();                                                                                    \
-    }
-        SVG(4, CLS_G4) SVG(8, CLS_G8) SVG(16, CLS_G16) SVG(32, CLS_G32) SVG(32, CLS_W512)
-#undef SVG
-        if (nbig) {
-            k_lp_block<false, true><<<grid_for(nbig, 1, sms(4)), 256, 0, s>>>(g.off, g.tgt, C, lab, nullptr,
-                                                                               lst(CLS_BLOCK), nbig, changed);
-            GSP_CHECK_LAUNCH();
+__global__ void __launch_bounds__(256) k_hook_sample(const uint64_t *__restrict__ off,
+                                                     const uint32_t *__restrict__ tgt,
+                                                     const uint32_t *__restrict__ C, uint32_t n, uint32_t *lab) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint64_t b = off[i];
+        const uint32_t k = (uint32_t)min(off[i + 1] - b, (uint64_t)HOOK_SAMPLE), ci = C[i];
+        uint32_t j[HOOK_SAMPLE], cj[HOOK_SAMPLE];
+#pragma unroll
+        for (uint32_t u = 0; u < HOOK_SAMPLE; u++) j[u] = u < k ? __ldg(tgt + b + u) : i;
+#pragma unroll
+        for (uint32_t u = 0; u < HOOK_SAMPLE; u++) cj[u] = __ldg(C + j[u]);
+        uint32_t r = EMPTY;
+#pragma unroll
+        for (uint32_t u = 0; u < HOOK_SAMPLE; u++) {
+            if (j[u] == i || cj[u] != ci) continue;
+            if (r == EMPTY) r = hook_find(lab, i);
+            r = hook_link(lab, r, hook_find(lab, j[u]));
         }
-        k_sv_shortcut<<<grid_for(g.n, 256), 256, 0, s>>>(lab, g.n);
-        GSP_CHECK_LAUNCH();
-        unsigned long long h;
-        GSP_CUDA(cudaMemcpyAsync(&h, changed, sizeof(h), cudaMemcpyDeviceToHost, s));
-        GSP_CUDA(cudaStreamSynchronize(s));
-        if (h == 0) break;
     }
+}
+
+// Point every vertex at its root; tree (optional): a root of each community.
+// Read-only finds: a halving store could land on a vertex already finished.
+__global__ void __launch_bounds__(256) k_hook_compress(const uint32_t *__restrict__ C, uint32_t n, uint32_t *lab,
+                                                       uint32_t *tree) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        uint32_t r = __ldca(lab + i);
+        for (uint32_t p; (p = __ldca(lab + r)) != r;) r = p;
+        lab[i] = r;
+        if (tree) tree[C[i]] = r;
+    }
+}
+
+// Link the rows of the vertices outside their community's tree (of all
+// vertices when there is no room for the trees and lists: h.rows null): a
+// warp reads 32 vertices' state at once and takes the open ones in turn.
+// Long rows are listed, so that neighbouring hubs do not queue in one warp.
+__global__ void __launch_bounds__(256) k_hook_rows(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tgt,
+                                                   const uint32_t *__restrict__ C, uint32_t n, uint32_t *lab,
+                                                   const uint32_t *__restrict__ tree, HookLists h) {
+    const uint32_t FULL = 0xFFFFFFFFu, lane = threadIdx.x & 31;
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (uint64_t v0 = (uint64_t)warp * 32; v0 < n; v0 += (uint64_t)nwarps * 32) {
+        const uint32_t v = (uint32_t)v0 + lane;
+        uint64_t b = 0, e = 0;
+        uint32_t c = 0;
+        bool open = false;
+        if (v < n) {
+            c = C[v];
+            open = !h.rows || ldcg_(lab + v) != tree[c];
+            if (open) {
+                b = off[v] + HOOK_SAMPLE;  // the sampled entries are linked already
+                e = off[v + 1];
+                open = b < e;
+                if (open && h.rows && e - b > HOOK_MID) {
+                    if (e - b > HOOK_HUB) h.rows[h.cap - 1 - atomicAdd(h.nhub, 1u)] = v;
+                    else h.rows[atomicAdd(h.nmid, 1u)] = v;
+                    open = false;
+                }
+            }
+        }
+        for (unsigned todo = __ballot_sync(FULL, open); todo; todo &= todo - 1) {
+            const int src = __ffs((int)todo) - 1;
+            const uint32_t i = (uint32_t)v0 + src, ci = __shfl_sync(FULL, c, src);
+            const uint64_t bi = __shfl_sync(FULL, b, src), ei = __shfl_sync(FULL, e, src);
+            hook_row(tgt, C, lab, i, ci, bi + lane, ei, 32);
+            __syncwarp();
+        }
+    }
+}
+
+// The listed rows: block columns (x) take the longest rows in turn, their
+// HOOK_COL blocks interleaved slices of each; then every block takes one of
+// the others at a time.
+__global__ void __launch_bounds__(256) k_hook_long(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tgt,
+                                                   const uint32_t *__restrict__ C, uint32_t *lab, HookLists h) {
+    const uint32_t nhub = *h.nhub, nmid = *h.nmid;
+    for (uint32_t t = blockIdx.x; t < nhub; t += gridDim.x) {
+        const uint32_t i = h.rows[h.cap - 1 - t];
+        hook_row(tgt, C, lab, i, C[i], off[i] + HOOK_SAMPLE + blockIdx.y * blockDim.x + threadIdx.x, off[i + 1],
+                 HOOK_COL * blockDim.x);
+    }
+    for (uint32_t t = blockIdx.y * gridDim.x + blockIdx.x; t < nmid; t += gridDim.x * HOOK_COL) {
+        const uint32_t i = h.rows[t];
+        hook_row(tgt, C, lab, i, C[i], off[i] + HOOK_SAMPLE + threadIdx.x, off[i + 1], blockDim.x);
+    }
+}
+
+static void split_hook(const DevGraph &g, const uint32_t *C, uint32_t *lab, cudaStream_t s) {
+    size_t mk = arena().mark();
+    // trees, lists of long rows and their counts; without room for them in a
+    // caller's workspace every row is linked by its warp
+    HookLists h{};
+    h.cap = (uint32_t)std::min<uint64_t>(g.n, g.nnz / HOOK_MID) + 1;
+    uint32_t *tree = static_cast<uint32_t *>(arena().try_alloc(sizeof(uint32_t) * ((size_t)g.n + h.cap + 2)));
+    if (tree) {
+        h.rows = tree + g.n;
+        h.nmid = h.rows + h.cap;
+        h.nhub = h.nmid + 1;
+        GSP_CUDA(cudaMemsetAsync(h.nmid, 0, 2 * sizeof(uint32_t), s));
+    }
+    iota_u32(lab, g.n, s);
+    const unsigned gr = grid_for(g.n, 256);
+    k_hook_sample<<<gr, 256, 0, s>>>(g.off, g.tgt, C, g.n, lab);
+    GSP_CHECK_LAUNCH();
+    if (tree) {
+        k_hook_compress<<<gr, 256, 0, s>>>(C, g.n, lab, tree);
+        GSP_CHECK_LAUNCH();
+    }
+    k_hook_rows<<<gr, 256, 0, s>>>(g.off, g.tgt, C, g.n, lab, tree, h);
+    GSP_CHECK_LAUNCH();
+    if (tree && h.cap > 1) {
+        k_hook_long<<<dim3(sm_count(), HOOK_COL), 256, 0, s>>>(g.off, g.tgt, C, lab, h);
+        GSP_CHECK_LAUNCH();
+    }
+    k_hook_compress<<<gr, 256, 0, s>>>(C, g.n, lab, nullptr);
+    GSP_CHECK_LAUNCH();
     arena().release(mk);
 }
 
@@ -496,8 +537,8 @@ static void split_bfs(const DevGraph &g, const uint32_t *C, uint32_t *lab, cudaS
 void split_labels(const DevGraph &g, const Classes &cl, const uint32_t *C, int mode, uint32_t *labels,
                   cudaStream_t s) {
     if (mode == GSP_SPLIT_BFS) split_bfs(g, C, labels, s);
-    else if (mode == GSP_SPLIT_SV) split_sv(g, cl, C, labels, s);
-    else split_lp(g, cl, C, mode == GSP_SPLIT_LPP, labels, s);
+    else if (mode == GSP_SPLIT_LP) split_lp(g, cl, C, labels, s);
+    else split_hook(g, C, labels, s);
 }
 
 }  // namespace gsp
