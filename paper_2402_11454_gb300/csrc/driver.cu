@@ -581,7 +581,7 @@ void alloc_move_state(MoveBuffers &mb, uint32_t n) {
     mb.left = arena().get<uint32_t>(n);
     mb.left_it = arena().get<int>(n);
     mb.it_dev = arena().get<int>(1);
-    mb.m_dev = arena().get<double>(1);
+    mb.m_dev = arena().get<double>(2);
     mb.ctr = arena().get<MoveCounters>(1);
 }
 
@@ -1056,7 +1056,8 @@ gsp_status gsp_move_sweep(const uint64_t *offsets, const uint32_t *targets, cons
     mb.choice = choice;
     GSP_CUDA(cudaMemcpyAsync(mb.C, C, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
     GSP_CUDA(cudaMemcpyAsync(mb.Sigma, Sigma, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    GSP_CUDA(cudaMemcpyAsync(mb.m_dev, &m, sizeof(double), cudaMemcpyHostToDevice, s));
+    const double m_pair[2] = {m, 1.0 / m};
+    GSP_CUDA(cudaMemcpyAsync(mb.m_dev, m_pair, sizeof(m_pair), cudaMemcpyHostToDevice, s));
     GSP_CUDA(cudaMemcpyAsync(choice, C, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
     GSP_CUDA(cudaMemsetAsync(mb.size, 0, sizeof(uint32_t) * n, s));
     k_community_sizes<<<grid_for(n, 256), 256, 0, s>>>(C, n, mb.size);
@@ -1104,7 +1105,8 @@ gsp_status gsp_local_move(const uint64_t *offsets, const uint32_t *targets, cons
     mb.repeats = wave_repeats;
     mb.no_return_from = no_return_from;
     reset_left(mb, n, s);
-    GSP_CUDA(cudaMemcpyAsync(mb.m_dev, &m, sizeof(double), cudaMemcpyHostToDevice, s));
+    const double m_pair[2] = {m, 1.0 / m};
+    GSP_CUDA(cudaMemcpyAsync(mb.m_dev, m_pair, sizeof(m_pair), cudaMemcpyHostToDevice, s));
     GSP_CUDA(cudaMemcpyAsync(mb.C, C, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
     GSP_CUDA(cudaMemcpyAsync(mb.Sigma, Sigma, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     GSP_CUDA(cudaMemsetAsync(mb.size, 0, sizeof(uint32_t) * n, s));
@@ -1170,7 +1172,7 @@ gsp_status gsp_refine(const uint64_t *offsets, const uint32_t *targets, const vo
     check_csr(offsets, targets, n, nnz, arena().get<unsigned long long>(1), s);
     check_ids(B, n, n, "bound membership", s);
     double *K = arena().get<double>(n);
-    double *m_dev = arena().get<double>(1);
+    double *m_dev = arena().get<double>(2);
     double m = vertex_weights(g, K, m_dev, s, exact_lsb(g, s));
     Classes cl;
     classify_vertices(g, cl, effective_waves(waves, true), s);

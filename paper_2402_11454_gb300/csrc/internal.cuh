@@ -98,7 +98,7 @@ struct MoveBuffers {
     uint8_t *act = nullptr;      // unprocessed flags
     uint8_t *mark = nullptr;     // re-marks of a frozen-state wave (merged into act after it)
     const double *K = nullptr;
-    double *m_dev = nullptr;     // device copy of m
+    double *m_dev = nullptr;     // device copy of m and 1/m
     const uint32_t *gid = nullptr;   // batches: graph of each vertex
     const double *m_g = nullptr;     // batches: m of each graph
     const double *minv_g = nullptr;  // batches: 1/m of each graph
@@ -271,7 +271,7 @@ uint64_t aggregate(const DevGraph &g, const uint32_t *Cd, uint32_t k, uint64_t *
 // for every pass of a run.
 int exact_lsb(const DevGraph &g, cudaStream_t s);
 
-// K and m (m also written to *m_dev when non-null); returns m.  lsb: the
+// K and m (m and 1/m also written to m_dev[0..1] when non-null); returns m.  lsb: the
 // graph's exact_lsb (INT_MIN: float64 sums).
 double vertex_weights(const DevGraph &g, double *K, double *m_dev, cudaStream_t s, int lsb = INT_MIN);
 double modularity(const DevGraph &g, const uint32_t *C, cudaStream_t s, int lsb = INT_MIN);

@@ -282,7 +282,10 @@ static void row_sums_any(const DevGraph &g, const uint32_t *C, double *K, double
     else row_sums<float, double>(g, C, K, Sig, acc, INT_MIN, s);
 }
 
-__global__ void k_half(const double *acc, double *m_dev) { *m_dev = acc[0] / 2.0; }
+__global__ void k_half(const double *acc, double *m_dev) {
+    m_dev[0] = acc[0] / 2.0;
+    m_dev[1] = 1.0 / m_dev[0];
+}
 
 double vertex_weights(const DevGraph &g, double *K, double *m_dev, cudaStream_t s, int lsb) {
     size_t mk = arena().mark();

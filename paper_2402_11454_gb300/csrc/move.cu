@@ -44,7 +44,7 @@ struct MoveArgs {
     uint32_t *size;
     uint8_t *act;
     uint8_t *mark;  // re-marking target: a separate array merged after a frozen-state wave, act in place
-    const double *m;
+    const double *m;  // m and 1/m
     // batches of independent graphs: graph of each vertex, m of each graph,
     // per-graph summed gains (null for a single graph)
     const uint32_t *gid;
@@ -127,27 +127,89 @@ __device__ __forceinline__ void scan_edges(const uint32_t *__restrict__ tgt, con
     }
 }
 
+// Open-addressing table of a vertex's K_{i->c} in shared memory, linear probing,
+// 2^logcap slots, at least twice the vertex's degree.  It is empty between
+// vertices: add() tells the thread that claimed a slot which one, that thread
+// alone scores it once every edge is in, and empties it.  So nobody reads or
+// clears the two to four slots per edge that stay free, and there is no shared
+// list of occupied slots.  Float32 values share a 64-bit word with their key: a
+// community seen for the first time (in a pass's first sweep nearly every one)
+// is claimed and given its weight by one compare-and-swap, and key and value
+// are read and cleared in one access.  Float64 values lie beside the keys.
+template <typename V> struct Table;
+template <> struct Table<float> {
+    unsigned long long *t;
+    static constexpr size_t slot_bytes = 8;
+    static constexpr unsigned long long FREE = ~0ull;
+    // slots [first, ...) of a region of `total` slots at base
+    __device__ Table(unsigned char *base, uint32_t, uint32_t first)
+        : t(reinterpret_cast<unsigned long long *>(base) + first) {}
+    __device__ void clear(uint32_t s) { t[s] = FREE; }
+    __device__ uint32_t get(uint32_t s, float &v) const {
+        const unsigned long long e = t[s];
+        v = __uint_as_float((uint32_t)e);
+        return (uint32_t)(e >> 32);
+    }
+    __device__ uint32_t add(int logcap, uint32_t c, float w) {  // the slot claimed, or EMPTY
+        const uint32_t mask = (1u << logcap) - 1u;
+        uint32_t h = logcap ? (hash32(c) >> (32 - logcap)) : 0u;
+        const unsigned long long e = ((unsigned long long)c << 32) | __float_as_uint(w);
+        for (uint32_t probe = 0; probe <= mask; probe++) {
+            unsigned long long old = *(volatile unsigned long long *)(t + h);
+            if (old == FREE) old = atomicCAS(t + h, FREE, e);
+            if (old == FREE) return h;
+            if ((uint32_t)(old >> 32) == c) {
+                atomicAdd(reinterpret_cast<float *>(t + h), w);
+                return EMPTY;
+            }
+            h = (h + 1) & mask;
+        }
+        return EMPTY;
+    }
+};
+template <> struct Table<double> {
+    uint32_t *keys;
+    double *vals;
+    static constexpr size_t slot_bytes = 12;
+    __device__ Table(unsigned char *base, uint32_t total, uint32_t first)
+        : keys(reinterpret_cast<uint32_t *>(base) + first),
+          vals(reinterpret_cast<double *>(base + (size_t)total * sizeof(uint32_t)) + first) {}
+    __device__ void clear(uint32_t s) {
+        keys[s] = EMPTY;
+        vals[s] = 0.0;
+    }
+    __device__ uint32_t get(uint32_t s, double &v) const {
+        v = vals[s];
+        return keys[s];
+    }
+    __device__ uint32_t add(int logcap, uint32_t c, double w) {
+        uint32_t slot;
+        return ht_add_slot<double>(keys, vals, logcap, c, w, &slot) == 1 ? slot : EMPTY;
+    }
+};
+
 template <typename S> __device__ __forceinline__ bool better(S s1, uint32_t c1, S s2, uint32_t c2) {
     return s1 > s2 || (s1 == s2 && c1 < c2);
 }
 
-// Score the entries of a table: slots s = lane, lane + step, ... < cap (or
-// the listed slots occ[...] when occ is given).  U entries per round, with
-// the gathers of Sigma_c issued together.
-template <int U, int SYNC, typename SC, typename S, typename V>
-__device__ __forceinline__ void score_table(const uint32_t *keys, const V *vals, const uint16_t *occ, uint32_t cap,
-                                            uint32_t lane, uint32_t step, const double *Sig, const SC &sc, S &best,
-                                            uint32_t &bestc, uint32_t &ncand) {
-    for (uint32_t s0 = lane; s0 < cap; s0 += U * step) {
+// Score the slots listed in slot[] (EMPTY: none) and empty them, four gathers
+// of Sigma_c in flight.
+template <int N, int SYNC, typename SC, typename S, typename V>
+__device__ __forceinline__ void score_slots(Table<V> &tab, const uint32_t *slot, const double *Sig, const SC &sc,
+                                            S &best, uint32_t &bestc, uint32_t &ncand) {
+    constexpr int U = N < 4 ? N : 4;
+#pragma unroll
+    for (int s0 = 0; s0 < N; s0 += U) {
         uint32_t c[U];
         V v[U];
         double sg[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
-            uint32_t s = s0 + u * step;
-            uint32_t slot = s < cap ? (occ ? (uint32_t)occ[s] : s) : 0;
-            c[u] = s < cap ? keys[slot] : EMPTY;
-            v[u] = s < cap ? vals[slot] : V(0);
+            c[u] = EMPTY;
+            if (slot[s0 + u] != EMPTY) {
+                c[u] = tab.get(slot[s0 + u], v[u]);
+                tab.clear(slot[s0 + u]);
+            }
         }
 #pragma unroll
         for (int u = 0; u < U; u++) sg[u] = c[u] != EMPTY ? ld_state<SYNC>(Sig + c[u]) : 0.0;
@@ -161,6 +223,23 @@ __device__ __forceinline__ void score_table(const uint32_t *keys, const V *vals,
     }
 }
 
+// The same over a whole table of cap slots, this thread's lane, lane + step, ...
+template <int SYNC, typename SC, typename S, typename V>
+__device__ __forceinline__ void score_table(Table<V> &tab, uint32_t cap, uint32_t lane, uint32_t step,
+                                            const double *Sig, const SC &sc, S &best, uint32_t &bestc,
+                                            uint32_t &ncand) {
+    for (uint32_t s0 = lane; s0 < cap; s0 += 4 * step) {
+        uint32_t slot[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const uint32_t s = s0 + u * step;
+            V v;
+            slot[u] = s < cap && tab.get(s, v) != EMPTY ? s : EMPTY;
+        }
+        score_slots<4, SYNC>(tab, slot, Sig, sc, best, bestc, ncand);
+    }
+}
+
 // Equation 2, evaluated in the order written, with no contraction.
 __device__ __forceinline__ double eq2(double Kic, double Kid, double Ki, double Sc, double Sd, double m) {
     double t1 = __ddiv_rn(__dsub_rn(Kic, Kid), m);
@@ -169,12 +248,26 @@ __device__ __forceinline__ double eq2(double Kic, double Kid, double Ki, double 
     return __dsub_rn(t1, __ddiv_rn(t2, den));
 }
 
+// (float)x, rounded to nearest even, in integer operations.  Float64
+// instructions, conversions included, issue at a fraction of the integer rate
+// on this GPU, and the conversion of Sigma_c is the one a score needs.
+// Values outside float32's normal range take the instruction.
+__device__ __forceinline__ float f32_of(double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const uint32_t hi = (uint32_t)(u >> 32), mag = hi & 0x7FFFFFFFu;
+    if (mag - 0x38100000u >= 0x0FE00000u) return (mag | (uint32_t)u) ? (float)x : __uint_as_float(hi);
+    // 29 bits of the mantissa go; add half an ulp, less one bit when the kept part is even
+    const unsigned long long r = (u & 0x7FFFFFFFFFFFFFFFull) + 0x0FFFFFFFull + ((u >> 29) & 1ull);
+    return __uint_as_float(((uint32_t)(r >> 29) - (896u << 23)) | (hi & 0x80000000u));
+}
+
 // Per-vertex scoring context.
 template <bool F64> struct Score;
 template <> struct Score<true> {
     using S = double;
     double Ki, Kid, Sd, m;
     __device__ S score(double kic, double Sc) const { return eq2(kic, Kid, Ki, Sc, Sd, m); }
+    __device__ bool gains(S best) const { return best > 0.0; }
     __device__ double gain(S best) const { return best; }  // in units of Q
 };
 // Float64 is a narrow pipe on this GPU: the mixed-precision scores take 1/m
@@ -184,7 +277,8 @@ template <> struct Score<false> {
     using S = float;
     float kif, sd;
     double inv_m;
-    __device__ S score(float kic, double Sc) const { return __fmaf_rn(-kif, (float)Sc, kic); }
+    __device__ S score(float kic, double Sc) const { return __fmaf_rn(-kif, f32_of(Sc), kic); }
+    __device__ bool gains(S best) const { return best - sd > 0.0f; }  // gain(best) > 0
     __device__ double gain(S best) const { return (double)(best - sd) * inv_m; }
 };
 
@@ -194,8 +288,8 @@ template <> struct Score<false> {
 // round once (fused); the score of staying rounds twice, but once for the
 // vertices of the largest degree class (hub), whichever kernel serves them.
 template <bool F64>
-__device__ __forceinline__ Score<F64> make_score(double Ki, double kid, double Sd, double m, double inv_m,
-                                                 bool hub = false);
+__device__ __forceinline__ Score<F64> make_score(double Ki, typename std::conditional<F64, double, float>::type kid,
+                                                 double Sd, double m, double inv_m, bool hub = false);
 template <>
 __device__ __forceinline__ Score<true> make_score<true>(double Ki, double kid, double Sd, double m, double, bool) {
     Score<true> s;
@@ -203,13 +297,13 @@ __device__ __forceinline__ Score<true> make_score<true>(double Ki, double kid, d
     return s;
 }
 template <>
-__device__ __forceinline__ Score<false> make_score<false>(double Ki, double kid, double Sd, double, double inv_m,
+__device__ __forceinline__ Score<false> make_score<false>(double Ki, float kid, double Sd, double, double inv_m,
                                                           bool hub) {
     Score<false> s;
     const double inv2m = 0.5 * inv_m;
-    s.kif = (float)(Ki * inv2m);
-    const float rest = (float)(Sd - Ki);
-    s.sd = hub ? __fmaf_rn(-s.kif, rest, (float)kid) : __fsub_rn((float)kid, __fmul_rn(s.kif, rest));
+    s.kif = f32_of(Ki * inv2m);
+    const float rest = f32_of(Sd - Ki);
+    s.sd = hub ? __fmaf_rn(-s.kif, rest, kid) : __fsub_rn(kid, __fmul_rn(s.kif, rest));
     s.inv_m = inv_m;
     return s;
 }
@@ -223,6 +317,17 @@ __device__ __forceinline__ double vertex_inv_m(const MoveArgs &a, uint32_t i, do
 }
 __device__ __forceinline__ void add_graph_gain(const MoveArgs &a, uint32_t i, double gain) {
     if (a.dq_g) atomicAdd(a.dq_g + a.gid[i], gain);
+}
+
+// In place: i moves from d to c now.
+__device__ __forceinline__ void apply_now(const MoveArgs &a, uint32_t i, uint32_t d, uint32_t c, double Ki) {
+    a.left[i] = d;
+    a.left_it[i] = *a.iteration;
+    a.C[i] = c;
+    atomicAdd(a.Sig + d, -Ki);
+    atomicAdd(a.Sig + c, Ki);
+    atomicSub(a.size + d, 1u);
+    atomicAdd(a.size + c, 1u);
 }
 
 // Decide the move of i toward c (one thread).  Frozen-state: record it in the
@@ -244,38 +349,54 @@ __device__ __forceinline__ bool decide_move(const MoveArgs &a, uint32_t i, uint3
         a.mv_vtx[slot] = i;
         a.mv_cmt[slot] = c;
     } else {
-        a.left[i] = d;
-        a.left_it[i] = *a.iteration;
-        a.C[i] = c;
-        atomicAdd(a.Sig + d, -Ki);
-        atomicAdd(a.Sig + c, Ki);
-        atomicSub(a.size + d, 1u);
-        atomicAdd(a.size + c, 1u);
+        apply_now(a, i, d, c, Ki);
     }
     return true;
 }
 
-struct LocalCtr {
+struct LocalCtr {  // of one thread (a thread visits fewer than 2^32 edges in a launch's sums)
     double dq = 0;
-    unsigned long long moved = 0, vertices = 0, edges = 0, candidates = 0, marked = 0;
+    uint32_t moved = 0, vertices = 0, candidates = 0;
+    unsigned long long edges = 0, marked = 0;
 };
 
+// Warp sums by the reduction instruction, a float64 sum only where something
+// moved, and one shared atomic per warp and counter (six block-wide sums of
+// shuffles took twelve barriers).
 __device__ void flush_counters(const LocalCtr &l, MoveCounters *g) {
-    __shared__ double sd[32];
-    __shared__ unsigned long long su[32];
-    double dq = block_sum<double>(l.dq, sd);
-    unsigned long long mv = block_sum<unsigned long long>(l.moved, su);
-    unsigned long long vx = block_sum<unsigned long long>(l.vertices, su);
-    unsigned long long ed = block_sum<unsigned long long>(l.edges, su);
-    unsigned long long ca = block_sum<unsigned long long>(l.candidates, su);
-    unsigned long long mk = block_sum<unsigned long long>(l.marked, su);
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    __shared__ unsigned long long s_cnt[5];
+    __shared__ double s_dq;
+    if (threadIdx.x < 5) s_cnt[threadIdx.x] = 0;
+    if (threadIdx.x == 5) s_dq = 0.0;
+    __syncthreads();
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    const uint32_t n3[3] = {l.moved, l.vertices, l.candidates};
+    const unsigned long long e2[2] = {l.edges, l.marked};
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const uint32_t t = __reduce_add_sync(FULL, n3[k]);
+        if (lane0 && t) atomicAdd(&s_cnt[k], (unsigned long long)t);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        // 64-bit sums in two halves: the low 26 bits of 32 lanes stay below 2^32
+        const uint32_t lo = __reduce_add_sync(FULL, (uint32_t)(e2[k] & 0x3FFFFFFu));
+        const uint32_t hi = __reduce_add_sync(FULL, (uint32_t)(e2[k] >> 26));
+        if (lane0 && (lo | hi)) atomicAdd(&s_cnt[3 + k], ((unsigned long long)hi << 26) + lo);
+    }
+    if (__any_sync(FULL, l.dq != 0.0)) {
+        const double dq = warp_sum(l.dq);
+        if (lane0) atomicAdd(&s_dq, dq);
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (dq != 0.0) atomicAdd(&g->dq, dq);
-        if (mv) atomicAdd(&g->moved, mv);
-        if (vx) atomicAdd(&g->vertices, vx);
-        if (ed) atomicAdd(&g->edges, ed);
-        if (ca) atomicAdd(&g->candidates, ca);
-        if (mk) atomicAdd(&g->marked, mk);
+        if (s_dq != 0.0) atomicAdd(&g->dq, s_dq);
+        if (s_cnt[0]) atomicAdd(&g->moved, s_cnt[0]);
+        if (s_cnt[1]) atomicAdd(&g->vertices, s_cnt[1]);
+        if (s_cnt[2]) atomicAdd(&g->candidates, s_cnt[2]);
+        if (s_cnt[3]) atomicAdd(&g->edges, s_cnt[3]);
+        if (s_cnt[4]) atomicAdd(&g->marked, s_cnt[4]);
     }
 }
 
@@ -309,36 +430,172 @@ __device__ __forceinline__ void record_visit(const MoveArgs &a, uint32_t i, uint
 }
 
 // --------------------------------------------------------------------------
-// Groups of G lanes, one vertex per group, table of up to CAP slots per group.
-// A warp's tables lie in its own region of shared memory (32 / G tables), so
-// the warps of a block run independently: warp `wbase` of `wstep` takes the
-// list entries wbase, wbase + wstep, ...
+// One warp, 32 / 2^lg vertices at a time: 2^lg lanes per vertex.
+//
+// The warp goes through the steps of a visit together, groups without a
+// vertex idling along.  What bounds a visit is its chain of gathers (flag ->
+// row and C_i -> targets -> C_j -> Sigma_c) and what it issues between them:
+// Sigma of the first EPL edges' communities is gathered while the table fills,
+// movers of a round share one reservation in the move list, the row is read
+// once (its targets stay in registers for the marks of a mover), and nothing
+// on the way is a float64 instruction that an integer or float32 one can
+// replace (this part issues float64 at 1/64 of the float32 rate; one division
+// 1/m per thread was a third of the group kernel's time).
+// A full wave of R-MAT 21 alone, before -> after: degrees <= 128 78 -> 61 us,
+// 129-512 49 -> 36, 513-2048 85 -> 57.
 // --------------------------------------------------------------------------
-template <int G, int CAP, typename V> constexpr size_t warp_tables = (size_t)(32 / G) * CAP * (sizeof(uint32_t) + sizeof(V));
+template <int EPL, typename WT> struct LaneEdges {
+    uint32_t j[EPL];
+    WT w[EPL];
+    // edges gl, gl + G, ... of a row of deg entries at b; padding counts as a self-loop
+    __device__ __forceinline__ void load(const uint32_t *__restrict__ tgt, const WT *__restrict__ wt, uint32_t i,
+                                         uint64_t b, uint32_t deg, uint32_t gl, int lg) {
+#pragma unroll
+        for (int u = 0; u < EPL; u++) {
+            const uint32_t p = gl + ((uint32_t)u << lg);
+            const bool ok = p < deg;
+            j[u] = ok ? __ldg(tgt + b + p) : i;
+            w[u] = ok ? __ldg(wt + b + p) : WT(0);
+        }
+    }
+};
+
+template <typename V> struct Decision {  // of the group's vertex, the same in all its lanes
+    uint32_t to = EMPTY;  // community to move to (EMPTY: stay)
+    double gain = 0.0;
+    V kid = 0;
+};
+
+// Decide vertex i (act: the group has one and it is unprocessed) of community
+// d, whose lanes hold c[] = C of their first EPL edges' targets; rows of up to
+// CH * EPL * G edges.  tab: the group's table of 2^logcap slots, empty before
+// and after; all of it is used whatever the degree, since free slots cost
+// nothing and make the probes shorter.
+template <int EPL, int CH, int SYNC, typename WT, bool F64, typename V>
+__device__ __forceinline__ Decision<V> decide_warp(const MoveArgs &a, int lg, bool act, uint32_t i, uint32_t d,
+                                                   uint64_t b, uint32_t deg, double Ki, double m, double inv_m,
+                                                   const LaneEdges<EPL, WT> &ed, const uint32_t (&c)[EPL], int it,
+                                                   Table<V> tab, int logcap, LocalCtr &lc) {
+    using SC = Score<F64>;
+    using S = typename SC::S;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const uint32_t G = 1u << lg, gl = threadIdx.x & (G - 1u);
+    const WT *w = static_cast<const WT *>(a.w);
+    double Sd = 0.0, sg[EPL];
+    uint32_t sd = 0, lf = EMPTY;
+    if (act) {
+        // Sigma of the first edges' communities while the table fills
+#pragma unroll
+        for (int u = 0; u < EPL; u++) sg[u] = c[u] != d ? ld_state<SYNC>(a.Sig + c[u]) : 0.0;
+        Sd = ld_state<SYNC>(a.Sig + d);
+        if (a.rule) sd = ld_state<SYNC>(a.size + d);
+        if (a.no_return_from > 0 && it >= a.no_return_from && ld_state<SYNC>(a.left_it + i) == it - 1)
+            lf = ld_state<SYNC>(a.left + i);
+    }
+    uint32_t slot[EPL * CH];
+#pragma unroll
+    for (int u = 0; u < EPL * CH; u++) slot[u] = EMPTY;
+    V kid = 0;
+    if (act) {
+#pragma unroll
+        for (int u = 0; u < EPL; u++) {
+            if (ed.j[u] == i) continue;
+            if (c[u] == d) kid += (V)ed.w[u];
+            else slot[u] = tab.add(logcap, c[u], (V)ed.w[u]);
+        }
+    }
+    if constexpr (CH > 1) {
+#pragma unroll
+        for (int h = 1; h < CH; h++) {
+            const uint32_t p0 = h * EPL * G;
+            if (!act || deg <= p0) continue;
+            LaneEdges<EPL, WT> more;
+            more.load(a.tgt, w, i, b + p0, deg - p0, gl, lg);
+            uint32_t cm[EPL];
+#pragma unroll
+            for (int u = 0; u < EPL; u++) cm[u] = more.j[u] != i ? ld_state<SYNC>(a.C + more.j[u]) : d;
+#pragma unroll
+            for (int u = 0; u < EPL; u++) {
+                if (more.j[u] == i) continue;
+                if (cm[u] == d) kid += (V)more.w[u];
+                else slot[h * EPL + u] = tab.add(logcap, cm[u], (V)more.w[u]);
+            }
+        }
+    }
+    __syncwarp();  // every edge is in
+    for (uint32_t o = G >> 1; o > 0; o >>= 1) kid += __shfl_xor_sync(FULL, kid, o);
+    const SC sc = make_score<F64>(Ki, kid, Sd, m, inv_m);
+    S best = -INFINITY;
+    uint32_t bestc = EMPTY, ncand = 0;
+#pragma unroll
+    for (int u = 0; u < EPL; u++) {
+        if (slot[u] == EMPTY) continue;
+        V v;
+        const uint32_t cu = tab.get(slot[u], v);
+        tab.clear(slot[u]);
+        ncand++;
+        const S x = sc.score(v, sg[u]);
+        if (better(x, cu, best, bestc)) { best = x; bestc = cu; }
+    }
+    if constexpr (CH > 1) {
+        if (act && deg > EPL * G)
+            score_slots<EPL * (CH - 1), SYNC>(tab, slot + EPL, a.Sig, sc, best, bestc, ncand);
+    }
+    lc.candidates += ncand;
+    const bool need_size = sd == 1;  // the singleton rule looks at the target's size
+    uint32_t bsz = need_size && bestc != EMPTY ? ld_state<SYNC>(a.size + bestc) : 0u;
+    __syncwarp();  // the table is empty
+    for (uint32_t o = G >> 1; o > 0; o >>= 1) {
+        const S x = __shfl_xor_sync(FULL, best, o);
+        const uint32_t cx = __shfl_xor_sync(FULL, bestc, o), zx = __shfl_xor_sync(FULL, bsz, o);
+        if (better(x, cx, best, bestc)) { best = x; bestc = cx; bsz = zx; }
+    }
+    Decision<V> r;
+    r.kid = kid;
+    if (act) {
+        // a vertex alone in its community moves to another singleton only
+        // toward a lower id, and nobody back to the community just left
+        if (bestc != EMPTY && sc.gains(best) && bestc != lf && !(need_size && bsz == 1 && bestc > d)) r.to = bestc;
+        if (r.to != EMPTY || (a.feat_kept && bestc != EMPTY)) r.gain = sc.gain(best);
+        if (gl == 0) {
+            lc.vertices++;
+            lc.edges += deg;
+            if (r.to != EMPTY) {
+                lc.moved++;
+                lc.marked += deg;
+                lc.dq += r.gain;
+                add_graph_gain(a, i, r.gain);
+            }
+        }
+    }
+    return r;
+}
+
+// A class of at most CAP / 2 edges per vertex, G lanes each; a warp's tables
+// (32 / G of CAP slots) lie in its own region of shared memory, so the warps of
+// a block run independently: warp `wbase` of `wstep` takes the list entries
+// wbase, wbase + wstep, ...
+template <int G, int CAP, typename V> constexpr size_t warp_tables = (size_t)(32 / G) * CAP * Table<V>::slot_bytes;
 
 template <int G, int CAP, typename WT, bool F64, int SYNC>
 __device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list, uint32_t count, uint32_t wbase,
                            uint32_t wstep, unsigned char *warp_smem, LocalCtr &lc) {
     using V = typename std::conditional<F64, double, float>::type;
-    using SC = Score<F64>;
-    using S = typename SC::S;
-    const int lane = threadIdx.x % G;
-    const int leader = (threadIdx.x & 31) & ~(G - 1);
-    const unsigned gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << leader);
-    uint32_t *keys = reinterpret_cast<uint32_t *>(warp_smem) + leader / G * CAP;
-    V *vals = reinterpret_cast<V *>(warp_smem + (size_t)(32 / G) * CAP * sizeof(uint32_t)) + leader / G * CAP;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr int LG = G == 4 ? 2 : G == 8 ? 3 : G == 16 ? 4 : 5;
+    constexpr int NGW = 32 / G;                  // vertices of a warp at a time
+    constexpr int EPL = CAP <= 4 * G ? 2 : 4;    // edges a lane holds ...
+    constexpr int CH = CAP / 2 / (EPL * G);      // ... and rounds of them in the longest row
+    const int wl = threadIdx.x & 31, gl = wl % G, gw = wl / G;
+    Table<V> tab(warp_smem, NGW * CAP, gw * CAP);
+    for (int t = gl; t < CAP; t += G) tab.clear(t);
     const WT *w = static_cast<const WT *>(a.w);
-    const double m0 = *a.m;
-    const double inv0 = 1.0 / m0;
-    // counters accumulate in the caller's lc
-    // The warp's list entries are wbase, wbase + wstep, ...; 32 of them are
-    // claimed at once (each lane reads one flag and marks its vertex
-    // processed), and the active ones are dealt to the warp's groups round
-    // by round, so that the inactive vertices of later sweeps cost one
-    // parallel round of loads per 32 entries and the groups of a warp stay
-    // in step.
-    constexpr int NGW = 32 / G;  // groups per warp
-    const int wl = threadIdx.x & 31, gw = wl / G;
+    const double m0 = *a.m, inv0 = a.m[1];
+    const int it = *a.iteration;
+    // 32 of the warp's entries are claimed at once (each lane reads one flag
+    // and marks its vertex processed), and the active ones are dealt to the
+    // groups round by round, so that the inactive vertices of later sweeps
+    // cost one parallel round of loads per 32 entries.
     for (uint64_t kb = 0; wbase + kb * wstep < count; kb += 32) {
         const uint64_t my = wbase + (kb + wl) * wstep;
         uint32_t vi = 0;
@@ -351,63 +608,61 @@ __device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list,
                 if (a.deferred) a.deferred[vi] = 0;
             }
         }
-        const unsigned amask = __ballot_sync(0xFFFFFFFFu, claim);
+        const unsigned amask = __ballot_sync(FULL, claim);
         const int nact = __popc(amask);
         for (int r0 = 0; r0 < nact; r0 += NGW) {
-        const int q = r0 + gw;  // this group's active entry in the round
-        const uint32_t i = __shfl_sync(0xFFFFFFFFu, vi, q < nact ? select_bit(amask, q) : 0);
-        if (q >= nact) continue;
-        uint32_t d = ld_state<SYNC>(a.C + i);
-        uint64_t b = a.off[i], e = a.off[i + 1];
-        uint32_t deg = (uint32_t)(e - b);
-        int logcap = ceil_log2(2 * deg);
-        if (logcap < 1) logcap = 1;
-        uint32_t cap = 1u << logcap;
-        for (uint32_t s = lane; s < cap; s += G) { keys[s] = EMPTY; vals[s] = V(0); }
-        __syncwarp(gmask);
-        V kid = 0;
-        scan_edges<(CAP >= 1024 ? 4 : 2), SYNC, V>(a.tgt, w, a.C, i, d, b, e, lane, G, kid,
-                                                    [&](uint32_t c, V wv) { ht_add<V>(keys, vals, logcap, c, wv); });
-        __syncwarp(gmask);
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) kid += __shfl_xor_sync(gmask, kid, o);
-        double Ki = a.K[i];
-        double Sd = ld_state<SYNC>(a.Sig + d);
-        Sd = __shfl_sync(gmask, Sd, leader);
-        const double m = vertex_m(a, i, m0);
-        SC sc = make_score<F64>(Ki, (double)kid, Sd, m, vertex_inv_m(a, i, inv0));
-        S best = -INFINITY;
-        uint32_t bestc = EMPTY;
-        uint32_t ncand = 0;
-        score_table<(CAP >= 1024 ? 4 : 2), SYNC>(keys, vals, (const uint16_t *)nullptr, cap, lane, G, a.Sig, sc, best,
-                                                  bestc, ncand);
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) {
-            S v2 = __shfl_xor_sync(gmask, best, o);
-            uint32_t c2 = __shfl_xor_sync(gmask, bestc, o);
-            if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
-        }
-        lc.candidates += ncand;
-        double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
-        int mv = 0;
-        if (lane == 0) {
-            lc.vertices++;
-            lc.edges += deg;
-            if (gain > 0.0) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
-            if (mv) { lc.moved++; lc.dq += gain; add_graph_gain(a, i, gain); }
-            record_visit(a, i, deg, Ki, (double)kid, gain, m, mv);
-        }
-        // movers re-mark their neighbours (frozen-state waves write a separate
-        // array merged after the wave, so that the wave never sees its marks)
-        mv = __shfl_sync(gmask, mv, leader);
-        if (mv) {
-            if (lane == 0) lc.marked += deg;
-            for (uint64_t p = b + lane; p < e; p += G) {
-                uint32_t j = __ldg(a.tgt + p);
-                if (j != i) a.mark[j] = 1;
+            const int q = r0 + gw;  // this group's active entry in the round
+            const bool act = q < nact;
+            const uint32_t i = __shfl_sync(FULL, vi, act ? select_bit(amask, q) : 0);
+            uint64_t b = 0;
+            uint32_t deg = 0, d = 0, c[EPL];
+            double Ki = 0.0, m = m0, inv_m = inv0;
+            LaneEdges<EPL, WT> ed;
+            if (act) {
+                d = ld_state<SYNC>(a.C + i);
+                b = a.off[i];
+                deg = (uint32_t)(a.off[i + 1] - b);
+                Ki = a.K[i];
+                m = vertex_m(a, i, m0);
+                inv_m = vertex_inv_m(a, i, inv0);
             }
-        }
-        __syncwarp(gmask);
+            ed.load(a.tgt, w, i, b, deg, gl, LG);
+#pragma unroll
+            for (int u = 0; u < EPL; u++) c[u] = ed.j[u] != i ? ld_state<SYNC>(a.C + ed.j[u]) : d;
+            const Decision<V> r = decide_warp<EPL, CH, SYNC, WT, F64, V>(a, LG, act, i, d, b, deg, Ki, m, inv_m, ed, c,
+                                                                         it, tab, ceil_log2(CAP), lc);
+            const bool moves = r.to != EMPTY;
+            if (act && gl == 0) {
+                if (moves && a.choice) a.choice[i] = r.to;
+                record_visit(a, i, deg, Ki, (double)r.kid, r.gain, m, moves);
+            }
+            const unsigned movers = __ballot_sync(FULL, moves && gl == 0);
+            if (!movers) continue;
+            if constexpr (SYNC) {  // one reservation in the move list per round
+                uint32_t base = 0;
+                if (wl == 0) base = atomicAdd(a.mv_cnt, (uint32_t)__popc(movers));
+                base = __shfl_sync(FULL, base, 0);
+                if (moves && gl == 0) {
+                    const uint32_t slot = base + __popc(movers & ((1u << wl) - 1u));
+                    a.mv_vtx[slot] = i;
+                    a.mv_cmt[slot] = r.to;
+                }
+            } else if (moves && gl == 0) {
+                apply_now(a, i, d, r.to, Ki);
+            }
+            // movers re-mark their neighbours (frozen-state waves write a
+            // separate array merged after the wave, so that the wave never
+            // sees its marks)
+            if (moves) {
+#pragma unroll
+                for (int u = 0; u < EPL; u++)
+                    if (ed.j[u] != i) a.mark[ed.j[u]] = 1;
+                for (uint64_t p = b + EPL * G + gl; p < b + deg; p += G) {
+                    const uint32_t j = __ldg(a.tgt + p);
+                    if (j != i) a.mark[j] = 1;
+                }
+            }
+            __syncwarp();
         }
     }
     __syncwarp();  // the warp's tables are free for the next body
@@ -420,7 +675,7 @@ struct GroupLists {
 };
 
 template <typename WT, bool F64, int SYNC>
-__global__ void __launch_bounds__(256) k_move_groups(MoveArgs a, GroupLists gl) {
+__global__ void __launch_bounds__(256, F64 ? 3 : 4) k_move_groups(MoveArgs a, GroupLists gl) {
     using V = typename std::conditional<F64, double, float>::type;
     constexpr size_t WREG = warp_tables<32, 256, V>;  // the largest of the four
     __shared__ __align__(16) unsigned char smem[8 * WREG];
@@ -439,7 +694,7 @@ __global__ void __launch_bounds__(256) k_move_groups(MoveArgs a, GroupLists gl) 
 // Degrees 129..512: one warp per vertex, 1024-slot table per warp.
 constexpr int W512_CAP = 1024;
 template <typename WT, bool F64, int SYNC>
-__global__ void __launch_bounds__(256) k_move_w512(MoveArgs a, const uint32_t *__restrict__ list, uint32_t count) {
+__global__ void __launch_bounds__(256, F64 ? 2 : 3) k_move_w512(MoveArgs a, const uint32_t *__restrict__ list, uint32_t count) {
     using V = typename std::conditional<F64, double, float>::type;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     const uint32_t wid = threadIdx.x >> 5;
@@ -450,35 +705,35 @@ __global__ void __launch_bounds__(256) k_move_w512(MoveArgs a, const uint32_t *_
 }
 
 // --------------------------------------------------------------------------
-// One block per vertex; table in shared memory (CAP > 0) or in the global
-// pool (CAP == 0, slots at pool_off[idx]).
+// One block per vertex, table of up to CAP slots in shared memory.  Two block
+// barriers a vertex: after the edges are inserted, and after their slots are
+// scored and emptied; warp 0 decides while the others start the next vertex.
+// A thread holds the slots of U edges; with more edges than the block's threads
+// hold the table is read through instead.
 // --------------------------------------------------------------------------
-template <int CAP, typename WT, bool F64, int SYNC>
+template <int CAP, int U, typename WT, bool F64, int SYNC>
 __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list, uint32_t count, uint32_t lb,
                            uint32_t nb, unsigned char *dyn_smem, LocalCtr &lc, uint32_t slots = CAP, bool hub = false) {
     using V = typename std::conditional<F64, double, float>::type;
     using SC = Score<F64>;
     using S = typename SC::S;
-    // table: keys, values and the list of occupied slots (scoring and
-    // clearing touch only those)
-    uint32_t *keys = reinterpret_cast<uint32_t *>(dyn_smem);
-    V *vals = reinterpret_cast<V *>(dyn_smem + (size_t)CAP * sizeof(uint32_t));
-    uint16_t *occ = reinterpret_cast<uint16_t *>(dyn_smem + (size_t)CAP * (sizeof(uint32_t) + sizeof(V)));
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr uint32_t CLAIM = 256;
+    // all of the table is used whatever the degree; a degree above CAP / 2 comes
+    // only on graphs of fewer than CAP vertices (move_level)
+    const int logcap = ceil_log2(slots);
+    Table<V> tab(dyn_smem, CAP, 0);
     __shared__ S red_s[32];
     __shared__ uint32_t red_c[32];
     __shared__ V red_k[32];
-    __shared__ int s_mv;
-    __shared__ uint32_t s_d, s_nocc;
-    __shared__ double s_Sd;
+    __shared__ uint32_t s_todo[CLAIM], s_ntodo, s_wcnt[32];
+    __shared__ uint8_t s_moved[CLAIM];
     const WT *w = static_cast<const WT *>(a.w);
     const double m0 = *a.m;
-    const double inv0 = 1.0 / m0;
+    const double inv0 = a.m[1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
-    // counters accumulate in the caller's lc
-    constexpr uint32_t CLAIM = 256;
-    __shared__ uint32_t s_todo[CLAIM], s_ntodo, s_wcnt[32];
-    for (uint32_t s = threadIdx.x; s < slots; s += blockDim.x) { keys[s] = EMPTY; vals[s] = V(0); }
+    for (uint32_t s = threadIdx.x; s < slots; s += blockDim.x) tab.clear(s);
     // The block's entries are lb + k * nb; CLAIM of them are claimed at
     // once (one flag per thread) and the active ones listed in shared memory,
     // so inactive vertices cost no serial round trip.
@@ -494,7 +749,7 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
                 if (a.deferred) a.deferred[vi] = 0;
             }
         }
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, claim);
+        const unsigned bal = __ballot_sync(FULL, claim);
         __syncthreads();  // the loop's previous step is done with s_todo
         if (lane == 0) s_wcnt[wid] = __popc(bal);
         __syncthreads();
@@ -510,82 +765,96 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
         }
         __syncthreads();
         const uint32_t ntodo = s_ntodo;
-    for (uint32_t kk = 0; kk < ntodo; kk++) {
-        const uint32_t i = s_todo[kk];
-        __syncthreads();  // previous vertex done with the table and reductions
-        if (threadIdx.x == 0) {
-            s_nocc = 0;
-            s_d = ld_state<SYNC>(a.C + i);
-            s_Sd = ld_state<SYNC>(a.Sig + s_d);
-        }
-        __syncthreads();
-        uint32_t d = s_d;
-        uint64_t b = a.off[i], e = a.off[i + 1];
-        uint32_t deg = (uint32_t)(e - b);
-        // a degree above CAP / 2 comes only on graphs of fewer than CAP vertices (sweep_level)
-        const int logcap = min(ceil_log2(2 * deg), ceil_log2(CAP));
-        V kid = 0;
-        constexpr int U = CAP >= 16384 ? 8 : 4;  // hubs: more gathers in flight per thread
-        scan_edges<U, SYNC, V>(a.tgt, w, a.C, i, d, b, e, threadIdx.x, blockDim.x, kid,
-                               [&](uint32_t c, V wv) { smem_add<V>(keys, vals, logcap, occ, &s_nocc, c, wv); });
-        kid = warp_sum(kid);
-        if (lane == 0) red_k[wid] = kid;
-        __syncthreads();
-        kid = 0;
-        for (int t = 0; t < nw; t++) kid += red_k[t];
-        double Ki = a.K[i];
-        const double m = vertex_m(a, i, m0);
-        SC sc = make_score<F64>(Ki, (double)kid, s_Sd, m, vertex_inv_m(a, i, inv0), hub);
-        S best = -INFINITY;
-        uint32_t bestc = EMPTY;
-        uint32_t nocc = s_nocc;
-        uint32_t ncand = 0;
-        score_table<U, SYNC>(keys, vals, occ, nocc, threadIdx.x, blockDim.x, a.Sig, sc, best, bestc, ncand);
-        __syncthreads();  // every slot scored before the table is emptied
-        for (uint32_t k = threadIdx.x; k < nocc; k += blockDim.x) {
-            uint32_t slot = occ[k];
-            keys[slot] = EMPTY;  // leave the table empty for the next vertex
-            vals[slot] = V(0);
-        }
-        if (threadIdx.x == 0) lc.candidates += nocc;
+        for (uint32_t kk = 0; kk < ntodo; kk++) {
+            const uint32_t i = s_todo[kk];
+            const uint32_t d = ld_state<SYNC>(a.C + i);
+            const uint64_t b = a.off[i], e = a.off[i + 1];
+            const double Ki = a.K[i];
+            const double Sd = ld_state<SYNC>(a.Sig + d);
+            const uint32_t deg = (uint32_t)(e - b);
+            const bool held = deg <= U * blockDim.x;  // every claimed slot is in its thread's registers
+            uint32_t slot[U];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            S v2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-            uint32_t c2 = __shfl_xor_sync(0xFFFFFFFFu, bestc, o);
-            if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
+            for (int u = 0; u < U; u++) slot[u] = EMPTY;
+            V kid = 0;
+            for (uint64_t p0 = b + threadIdx.x; p0 < e; p0 += (uint64_t)U * blockDim.x) {
+                uint32_t j[U], c[U];
+                V wv[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const uint64_t p = p0 + (uint64_t)u * blockDim.x;
+                    j[u] = p < e ? __ldg(a.tgt + p) : i;
+                    wv[u] = p < e ? (V)__ldg(w + p) : V(0);
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) c[u] = j[u] != i ? ld_state<SYNC>(a.C + j[u]) : EMPTY;
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (c[u] == EMPTY) continue;
+                    if (c[u] == d) kid += wv[u];
+                    else slot[u] = tab.add(logcap, c[u], wv[u]);
+                }
+            }
+            kid = warp_sum(kid);
+            if (lane == 0) red_k[wid] = kid;
+            __syncthreads();  // every edge inserted
+            kid = warp_sum(lane < nw ? red_k[lane] : V(0));
+            const double m = vertex_m(a, i, m0);
+            const SC sc = make_score<F64>(Ki, kid, Sd, m, vertex_inv_m(a, i, inv0), hub);
+            S best = -INFINITY;
+            uint32_t bestc = EMPTY, ncand = 0;
+            if (held) score_slots<U, SYNC>(tab, slot, a.Sig, sc, best, bestc, ncand);
+            else score_table<SYNC>(tab, slots, threadIdx.x, blockDim.x, a.Sig, sc, best, bestc, ncand);
+            lc.candidates += ncand;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const S v2 = __shfl_xor_sync(FULL, best, o);
+                const uint32_t c2 = __shfl_xor_sync(FULL, bestc, o);
+                if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
+            }
+            if (lane == 0) { red_s[wid] = best; red_c[wid] = bestc; }
+            __syncthreads();  // every slot scored and emptied
+            if (wid != 0) continue;
+            best = lane < nw ? red_s[lane] : (S)-INFINITY;
+            bestc = lane < nw ? red_c[lane] : EMPTY;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const S v2 = __shfl_xor_sync(FULL, best, o);
+                const uint32_t c2 = __shfl_xor_sync(FULL, bestc, o);
+                if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
+            }
+            if (lane == 0) {
+                const double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
+                int mv = 0;
+                if (bestc != EMPTY && sc.gains(best)) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
+                lc.vertices++;
+                lc.edges += deg;
+                if (mv) { lc.moved++; lc.marked += deg; lc.dq += gain; add_graph_gain(a, i, gain); }
+                record_visit(a, i, deg, Ki, (double)kid, gain, m, mv);
+                s_moved[kk] = (uint8_t)mv;
+            }
+            __syncwarp();
         }
-        if (lane == 0) { red_s[wid] = best; red_c[wid] = bestc; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int t = 1; t < nw; t++)
-                if (better(red_s[t], red_c[t], best, bestc)) { best = red_s[t]; bestc = red_c[t]; }
-            double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
-            int mv = 0;
-            if (gain > 0.0) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
-            lc.vertices++;
-            lc.edges += deg;
-            if (mv) { lc.moved++; lc.dq += gain; add_graph_gain(a, i, gain); }
-            record_visit(a, i, deg, Ki, (double)kid, gain, m, mv);
-            s_mv = mv;
-        }
-        __syncthreads();
-        if (s_mv) {
-            if (threadIdx.x == 0) lc.marked += deg;
-            for (uint64_t p = b + threadIdx.x; a.mark && p < e; p += blockDim.x) {
-                uint32_t j = __ldg(a.tgt + p);
+        __syncthreads();  // the decisions of the claimed vertices are in
+        if (!a.mark) continue;
+        for (uint32_t kk = 0; kk < ntodo; kk++) {
+            if (!s_moved[kk]) continue;
+            const uint32_t i = s_todo[kk];
+            const uint64_t e = a.off[i + 1];
+            for (uint64_t p = a.off[i] + threadIdx.x; p < e; p += blockDim.x) {
+                const uint32_t j = __ldg(a.tgt + p);
                 if (j != i) a.mark[j] = 1;
             }
         }
     }
-    }
     __syncthreads();  // the block's table is free for the next body
 }
 
-template <int CAP, typename WT, bool F64, int SYNC>
-__global__ void __launch_bounds__(256) k_move_block(MoveArgs a, const uint32_t *__restrict__ list, uint32_t count) {
+template <int CAP, int THREADS, typename WT, bool F64, int SYNC>
+__global__ void __launch_bounds__(THREADS, F64 ? 1 : 1024 / THREADS) k_move_block(MoveArgs a, const uint32_t *__restrict__ list, uint32_t count) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     LocalCtr lc;
-    block_body<CAP, WT, F64, SYNC>(a, list, count, blockIdx.x, gridDim.x, dyn_smem, lc);
+    block_body<CAP, 8, WT, F64, SYNC>(a, list, count, blockIdx.x, gridDim.x, dyn_smem, lc);
     flush_counters(lc, a.ctr);
 }
 
@@ -614,25 +883,23 @@ __device__ __forceinline__ double signed_units_val(unsigned long long u, int lsb
                  : Acc<unsigned long long>::val((unsigned long long)v, lsb);
 }
 
-__device__ __forceinline__ void apply_delta(uint32_t *keys, double *ds, int *dn, uint32_t c, double k, int n,
-                                            double *Sig, uint32_t *size, int lsb) {
+// n = -1 or 1 member of weight k leaves or joins c; u: k in units.
+__device__ __forceinline__ void apply_delta(uint32_t *keys, double *ds, int *dn, uint32_t c, double k,
+                                            unsigned long long u, int n, double *Sig, uint32_t *size, int lsb) {
     uint32_t mask = (1u << APPLY_SLOG) - 1u;
     uint32_t h = hash32(c) >> (32 - APPLY_SLOG);
     for (uint32_t probe = 0; probe < 64; probe++) {
-        uint32_t old = atomicCAS(&keys[h], EMPTY, c);
+        uint32_t old = *(volatile uint32_t *)&keys[h];
+        if (old == EMPTY) old = atomicCAS(&keys[h], EMPTY, c);
         if (old == EMPTY || old == c) {
-            if (lsb != INT_MIN) {
-                const unsigned long long u = units_of(k < 0.0 ? -k : k, lsb);
-                atomicAdd(reinterpret_cast<unsigned long long *>(ds) + h, k < 0.0 ? 0ull - u : u);
-            } else {
-                atomicAdd(&ds[h], k);
-            }
+            if (lsb != INT_MIN) atomicAdd(reinterpret_cast<unsigned long long *>(ds) + h, n < 0 ? 0ull - u : u);
+            else atomicAdd(&ds[h], n < 0 ? -k : k);
             atomicAdd(&dn[h], n);
             return;
         }
         h = (h + 1) & mask;
     }
-    atomicAdd(Sig + c, k);  // crowded table: apply directly
+    atomicAdd(Sig + c, n < 0 ? -k : k);  // crowded table: apply directly
     atomicAdd(size + c, (uint32_t)n);
 }
 
@@ -669,8 +936,9 @@ __global__ void __launch_bounds__(256) k_apply_moves(const uint32_t *__restrict_
         C[i] = c;
         left[i] = d;
         left_it[i] = iteration;
-        apply_delta(skeys, sds, sdn, d, -Ki, -1, Sig, size, lsb);
-        apply_delta(skeys, sds, sdn, c, Ki, 1, Sig, size, lsb);
+        const unsigned long long u = lsb != INT_MIN ? units_of(Ki, lsb) : 0ull;
+        apply_delta(skeys, sds, sdn, d, Ki, u, -1, Sig, size, lsb);
+        apply_delta(skeys, sds, sdn, c, Ki, u, 1, Sig, size, lsb);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < (1 << APPLY_SLOG); t += blockDim.x) flush_delta(skeys, sds, sdn, t, Sig, size, lsb);
@@ -775,8 +1043,9 @@ __device__ void apply_body_l2(const uint32_t *mv_vtx, const uint32_t *mv_cmt, co
         C[i] = c;
         left[i] = d;
         left_it[i] = iteration;
-        apply_delta(skeys, sds, sdn, d, -Ki, -1, Sig, size, lsb);
-        apply_delta(skeys, sds, sdn, c, Ki, 1, Sig, size, lsb);
+        const unsigned long long u = lsb != INT_MIN ? units_of(Ki, lsb) : 0ull;
+        apply_delta(skeys, sds, sdn, d, Ki, u, -1, Sig, size, lsb);
+        apply_delta(skeys, sds, sdn, c, Ki, u, 1, Sig, size, lsb);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < (1 << APPLY_SLOG); t += blockDim.x) flush_delta(skeys, sds, sdn, t, Sig, size, lsb);
@@ -835,7 +1104,7 @@ __global__ void __launch_bounds__(256) k_sweep_persistent(MoveArgs a, const uint
             __syncthreads();  // the block class uses the whole buffer
         }
         if (cc[CLS_BLOCK])
-            block_body<4096, WT, F64, 2>(aw, list + cb[CLS_BLOCK], cc[CLS_BLOCK], lb, nb, dyn_smem, lc);
+            block_body<4096, 8, WT, F64, 2>(aw, list + cb[CLS_BLOCK], cc[CLS_BLOCK], lb, nb, dyn_smem, lc);
         if (!grid_sync(bar, nb, a.ctr)) return;
         apply_body_l2(a.mv_vtx, a.mv_cmt, mv_cnts + wr, a.K, a.C, a.Sig, a.size, lb, nb, dyn_smem, a.lsb, a.left,
                       a.left_it, *a.iteration);
@@ -881,8 +1150,7 @@ constexpr int LEVEL_EPL = 4;         // edges a lane holds in registers
 constexpr uint32_t LEVEL_TASKS = 6;  // most tasks of a warp in a wave ...
 constexpr uint32_t LEVEL_MOVERS = 8 * LEVEL_TASKS;  // ... of at most 8 vertices each
 constexpr uint32_t LEVEL_BMOVERS = 64;              // most vertices of the block classes per CTA and wave
-// slots of the block classes' table
-template <bool F64> constexpr int LEVEL_CAP = F64 ? 8192 : 16384;
+constexpr int LEVEL_CAP = 16384;  // slots of the block classes' table
 
 struct LevelArgs {
     const uint32_t *list, *start;  // class/wave lists (Classes)
@@ -915,7 +1183,7 @@ template <bool F64> struct LevelSmem {
     using V = typename std::conditional<F64, double, float>::type;
     static constexpr size_t tables_bytes =
         std::max((size_t)LEVEL_WARPS * warp_tables<32, W512_CAP, V>,
-                 (size_t)LEVEL_CAP<F64> * (sizeof(uint32_t) + sizeof(V) + sizeof(uint16_t)));
+                 (size_t)LEVEL_CAP * Table<V>::slot_bytes);
     alignas(16) unsigned char tables[tables_bytes];  // per-warp tables, or one table of a block class
     LevelMover mv[LEVEL_WARPS][LEVEL_MOVERS];
     uint32_t start[NUM_CLS * MAX_WAVES + 1];
@@ -928,8 +1196,7 @@ template <typename WT> struct LevelTask {
     double K, m, inv_m;
     uint32_t i, deg;
     int lg;
-    uint32_t j[LEVEL_EPL];
-    WT w[LEVEL_EPL];
+    LaneEdges<LEVEL_EPL, WT> ed;
 };
 
 // Number of warp tasks of class k with `count` vertices (lanes per vertex:
@@ -962,15 +1229,7 @@ __device__ __forceinline__ void level_fetch(const MoveArgs &a, const uint32_t *_
     t.K = a.K[t.i];
     t.m = vertex_m(a, t.i, m0);
     t.inv_m = vertex_inv_m(a, t.i, inv0);
-    const uint32_t gl = lane & ((1u << t.lg) - 1u);
-    const WT *w = static_cast<const WT *>(a.w);
-#pragma unroll
-    for (int u = 0; u < LEVEL_EPL; u++) {
-        const uint32_t p = gl + ((uint32_t)u << t.lg);
-        const bool ok = p < t.deg;
-        t.j[u] = ok ? __ldg(a.tgt + t.b + p) : t.i;  // padding counts as a self-loop
-        t.w[u] = ok ? __ldg(w + t.b + p) : WT(0);
-    }
+    t.ed.load(a.tgt, static_cast<const WT *>(a.w), t.i, t.b, t.deg, lane & ((1u << t.lg) - 1u), t.lg);
 }
 
 // Decide the vertices of a task; movers are appended to mv[0..nmv).
@@ -978,103 +1237,28 @@ template <typename WT, bool F64>
 __device__ __forceinline__ void level_visit(const MoveArgs &a, const LevelTask<WT> &t, int it, unsigned char *ws,
                                             LevelMover *mv, uint32_t &nmv, LocalCtr &lc) {
     using V = typename std::conditional<F64, double, float>::type;
-    using SC = Score<F64>;
-    using S = typename SC::S;
     constexpr unsigned FULL = 0xFFFFFFFFu;
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t G = 1u << t.lg, gl = lane & (G - 1u);
-    const WT *w = static_cast<const WT *>(a.w);
+    const uint32_t lane = threadIdx.x & 31, gl = lane & ((1u << t.lg) - 1u);
     const bool has = t.i != EMPTY;
     const bool act = has && ldcg(a.act + t.i);
-    uint32_t d = 0, c[LEVEL_EPL], lf = EMPTY;
+    uint32_t d = 0, c[LEVEL_EPL];
     if (has) {
         d = ldcg(a.C + t.i);
 #pragma unroll
-        for (int u = 0; u < LEVEL_EPL; u++) c[u] = ldcg(a.C + t.j[u]);
-        if (a.no_return_from > 0 && it >= a.no_return_from && ldcg(a.left_it + t.i) == it - 1) lf = ldcg(a.left + t.i);
+        for (int u = 0; u < LEVEL_EPL; u++) c[u] = ldcg(a.C + t.ed.j[u]);
     }
     if (!__any_sync(FULL, act)) return;
-    double Sd = 0.0;
-    uint32_t sd = 0;
-    if (act) {
-        Sd = ldcg(a.Sig + d);
-        sd = ldcg(a.size + d);
-        if (gl == 0) {
-            a.act[t.i] = 0;
-            if (a.deferred) a.deferred[t.i] = 0;
-        }
-    }
-    // the group's table: G4 16 slots, G8 32, G16 64, then 256 and 1024
-    const int logcap = max(1, ceil_log2(2 * t.deg));
-    const uint32_t cap = act ? 1u << logcap : 0u;
-    const uint32_t first = t.lg == 5 ? 0u : (lane >> t.lg) * (4u * G);
-    uint32_t *keys = reinterpret_cast<uint32_t *>(ws) + first;
-    V *vals = reinterpret_cast<V *>(ws + (size_t)W512_CAP * sizeof(uint32_t)) + first;
-    for (uint32_t s = gl; s < cap; s += G) { keys[s] = EMPTY; vals[s] = V(0); }
-    __syncwarp();
-    V kid = 0;
-    if (act) {
-#pragma unroll
-        for (int u = 0; u < LEVEL_EPL; u++) {
-            if (t.j[u] == t.i) continue;
-            if (c[u] == d) kid += (V)t.w[u];
-            else ht_add<V>(keys, vals, logcap, c[u], (V)t.w[u]);
-        }
-        if (t.deg > LEVEL_EPL * G)
-            scan_edges<4, 2, V>(a.tgt, w, a.C, t.i, d, t.b + LEVEL_EPL * G, t.b + t.deg, gl, G, kid,
-                                [&](uint32_t cc, V wv) { ht_add<V>(keys, vals, logcap, cc, wv); });
-    }
-    __syncwarp();
-    for (uint32_t o = G >> 1; o > 0; o >>= 1) kid += __shfl_xor_sync(FULL, kid, o);
-    const SC sc = make_score<F64>(t.K, (double)kid, Sd, t.m, t.inv_m);
-    S best = -INFINITY;
-    uint32_t bestc = EMPTY, bsz = 0, ncand = 0;
-    const bool need_size = a.rule && sd == 1;  // the singleton rule looks at the target's size
-    for (uint32_t s0 = gl; s0 < cap; s0 += 4 * G) {
-        uint32_t cc[4], sz[4];
-        V val[4];
-        double sg[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const uint32_t s = s0 + u * G;
-            cc[u] = s < cap ? keys[s] : EMPTY;
-            val[u] = s < cap ? vals[s] : V(0);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            sg[u] = cc[u] != EMPTY ? ldcg(a.Sig + cc[u]) : 0.0;
-            sz[u] = cc[u] != EMPTY && need_size ? ldcg(a.size + cc[u]) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            if (cc[u] == EMPTY) continue;
-            ncand++;
-            const S x = sc.score(val[u], sg[u]);
-            if (better(x, cc[u], best, bestc)) { best = x; bestc = cc[u]; bsz = sz[u]; }
-        }
-    }
-    lc.candidates += ncand;
-    __syncwarp();
-    for (uint32_t o = G >> 1; o > 0; o >>= 1) {
-        const S x = __shfl_xor_sync(FULL, best, o);
-        const uint32_t cx = __shfl_xor_sync(FULL, bestc, o), zx = __shfl_xor_sync(FULL, bsz, o);
-        if (better(x, cx, best, bestc)) { best = x; bestc = cx; bsz = zx; }
-    }
-    bool moves = false;
     if (act && gl == 0) {
-        lc.vertices++;
-        lc.edges += t.deg;
-        const double gain = bestc == EMPTY ? 0.0 : sc.gain(best);
-        moves = gain > 0.0 && bestc != lf && !(need_size && bsz == 1 && bestc > d);
-        if (moves) {
-            lc.moved++;
-            lc.marked += t.deg;
-            lc.dq += gain;
-            add_graph_gain(a, t.i, gain);
-        }
+        a.act[t.i] = 0;
+        if (a.deferred) a.deferred[t.i] = 0;
     }
+    // the group's table: 16, 32 or 64 slots, then 256 and 1024
+    const Table<V> tab(ws, W512_CAP, t.lg == 5 ? 0u : (lane >> t.lg) * (4u << t.lg));
+    const Decision<V> r = decide_warp<LEVEL_EPL, 4, 2, WT, F64, V>(a, t.lg, act, t.i, d, t.b, t.deg, t.K, t.m, t.inv_m,
+                                                                t.ed, c, it, tab, t.lg == 5 ? ceil_log2(W512_CAP) : t.lg + 2, lc);
+    const bool moves = r.to != EMPTY && gl == 0;
     const unsigned bal = __ballot_sync(FULL, moves);
-    if (moves) mv[nmv + __popc(bal & ((1u << lane) - 1u))] = LevelMover{t.b, t.K, t.i, bestc, d, t.deg};
+    if (moves) mv[nmv + __popc(bal & ((1u << lane) - 1u))] = LevelMover{t.b, t.K, t.i, r.to, d, t.deg};
     nmv += __popc(bal);
 }
 
@@ -1092,7 +1276,7 @@ __device__ __forceinline__ void level_apply(const MoveArgs &a, uint32_t i, uint3
 template <typename WT, bool F64>
 __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, LevelArgs v) {
     using V = typename std::conditional<F64, double, float>::type;
-    constexpr int CAP = LEVEL_CAP<F64>;
+    constexpr int CAP = LEVEL_CAP;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     LevelSmem<F64> &sm = *reinterpret_cast<LevelSmem<F64> *>(dyn_smem);
     __shared__ int s_it;
@@ -1105,8 +1289,13 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
     const uint32_t wb = wid * nb + lb, wn = nb * LEVEL_WARPS;
     unsigned char *ws = sm.tables + wid * warp_tables<32, W512_CAP, V>;
     LevelMover *mv = sm.mv[wid];
-    const double m0 = *a.m, inv0 = 1.0 / m0;
+    const double m0 = *a.m, inv0 = a.m[1];
     for (int t = threadIdx.x; t <= NUM_CLS * v.W; t += LEVEL_THREADS) sm.start[t] = v.start[t];
+    auto clear_tables = [&]() {
+        Table<V> tab(ws, W512_CAP, 0);
+        for (int t = lane; t < W512_CAP; t += 32) tab.clear(t);
+    };
+    clear_tables();
     __syncthreads();
     // the block classes' movers go to the CTA's list, applied after the barrier
     MoveArgs ab = a;
@@ -1157,8 +1346,9 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
                     for (int k = CLS_HUGE; k >= CLS_BLOCK; k--) {
                         const uint32_t cnt = cls(k, wv, beg);
                         const uint32_t slots = k == CLS_BLOCK ? 4096u : (uint32_t)CAP;
-                        if (cnt) block_body<CAP, WT, F64, 2>(ab, v.list + beg, cnt, lb, nb, sm.tables, lc, slots, k == CLS_HUGE);
+                        if (cnt) block_body<CAP, 4, WT, F64, 2>(ab, v.list + beg, cnt, lb, nb, sm.tables, lc, slots, k == CLS_HUGE);
                     }
+                    clear_tables();
                 }
                 if (wb < tasks) level_visit<WT, F64>(a, t0, it, ws, mv, nmv, lc);
                 for (uint32_t x = wb + wn; x < tasks; x += wn) {
@@ -1335,7 +1525,7 @@ __global__ void __launch_bounds__(256) k_hub_score(MoveArgs a, HubArgs h) {
     const V *kidv = static_cast<const V *>(h.kid);
     S *bs = static_cast<S *>(h.best_s);
     const double m0 = *a.m;
-    const double inv0 = 1.0 / m0;
+    const double inv0 = a.m[1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t base = h.tasks[0], total = h.tasks[h.nh] - base;
     for (uint64_t task = blockIdx.x; task < total; task += gridDim.x) {
@@ -1347,7 +1537,7 @@ __global__ void __launch_bounds__(256) k_hub_score(MoveArgs a, HubArgs h) {
         V *vals = static_cast<V *>(h.vals) + h.pool_off[t];
         const uint32_t *occ = h.occ + h.pool_off[t];
         uint64_t k1 = min(k0 + HUB_CHUNK, (uint64_t)h.occ_n[t]);
-        SC sc = make_score<F64>(a.K[i], (double)kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
+        SC sc = make_score<F64>(a.K[i], kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
                                 vertex_inv_m(a, i, inv0), true);
         S best = -INFINITY;
         uint32_t bestc = EMPTY;
@@ -1403,7 +1593,7 @@ __global__ void k_hub_decide(MoveArgs a, HubArgs h) {
     const V *kidv = static_cast<const V *>(h.kid);
     const S *bs = static_cast<const S *>(h.best_s);
     const double m0 = *a.m;
-    const double inv0 = 1.0 / m0;
+    const double inv0 = a.m[1];
     const int lane = threadIdx.x & 31;
     uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1429,10 +1619,10 @@ __global__ void k_hub_decide(MoveArgs a, HubArgs h) {
             double Ki = a.K[i];
             uint64_t deg = a.off[i + 1] - a.off[i];
             const double m = vertex_m(a, i, m0);
-            SC sc = make_score<F64>(Ki, (double)kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, inv0), true);
+            SC sc = make_score<F64>(Ki, kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, inv0), true);
             double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
             int mv = 0;
-            if (gain > 0.0) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
+            if (bestc != EMPTY && sc.gains(best)) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
             lc.vertices++;
             lc.edges += deg;
             lc.candidates += h.occ_n[t];
@@ -1659,32 +1849,32 @@ static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, uint32_t
     }
     uint32_t nb = cl.count(CLS_BLOCK, wave);
     if (nb) {
-        constexpr int CAP = 4096;
-        constexpr size_t smem = (size_t)CAP * (sizeof(uint32_t) + sizeof(V) + sizeof(uint16_t));
+        constexpr int CAP = 4096, THREADS = 256;
+        constexpr size_t smem = CAP * Table<V>::slot_bytes;
+        const auto fn = k_move_block<CAP, THREADS, WT, F64, SYNC>;
         static bool attr = false;
         if (!attr) {
-            GSP_CUDA(cudaFuncSetAttribute(k_move_block<CAP, WT, F64, SYNC>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            GSP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             attr = true;
         }
-        k_move_block<CAP, WT, F64, SYNC><<<grid_for(nb, 1, (uint32_t)(sm * tn.block)), 256, smem, on(1)>>>(
-            a, cl.list + cl.begin(CLS_BLOCK, wave), nb);
+        fn<<<grid_for(nb, 1, (uint32_t)(sm * tn.block)), THREADS, smem, on(1)>>>(a, cl.list + cl.begin(CLS_BLOCK, wave),
+                                                                                nb);
         GSP_CHECK_LAUNCH();
     }
     uint32_t ng = cl.count(CLS_BIG, wave);
     if (ng) {
         // 2049..8192 edges: one block per vertex with a 16384-slot shared
-        // table (at most 2 x 8192 distinct keys), one block per SM
-        constexpr int CAP = 16384;
-        constexpr size_t smem = (size_t)CAP * (sizeof(uint32_t) + sizeof(V) + sizeof(uint16_t));
+        // table (twice the most edges); the table leaves room for one block
+        // per SM, so the block is as large as the registers allow
+        constexpr int CAP = 16384, THREADS = F64 ? 512 : 1024;
+        constexpr size_t smem = CAP * Table<V>::slot_bytes;
+        const auto fn = k_move_block<CAP, THREADS, WT, F64, SYNC>;
         static bool attr = false;
         if (!attr) {
-            GSP_CUDA(cudaFuncSetAttribute(k_move_block<CAP, WT, F64, SYNC>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            GSP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             attr = true;
         }
-        k_move_block<CAP, WT, F64, SYNC><<<grid_for(ng, 1, (uint32_t)sm), 256, smem, on(3)>>>(
-            a, cl.list + cl.begin(CLS_BIG, wave), ng);
+        fn<<<grid_for(ng, 1, (uint32_t)sm), THREADS, smem, on(3)>>>(a, cl.list + cl.begin(CLS_BIG, wave), ng);
         GSP_CHECK_LAUNCH();
     }
     uint32_t nh = cl.count(CLS_HUGE, wave);
@@ -1792,8 +1982,7 @@ template <typename WT, bool F64>
 static bool launch_persistent(const MoveArgs &a, const Classes &cl, uint32_t n, MoveBuffers &mb, int iteration,
                               cudaStream_t s) {
     using V = typename std::conditional<F64, double, float>::type;
-    constexpr size_t smem = std::max(std::max((size_t)8 * W512_CAP * (sizeof(uint32_t) + sizeof(V)),
-                                              (size_t)4096 * (sizeof(uint32_t) + sizeof(V) + sizeof(uint16_t))),
+    constexpr size_t smem = std::max(std::max(8 * warp_tables<32, W512_CAP, V>, 4096 * Table<V>::slot_bytes),
                                      (size_t)(sizeof(uint32_t) + sizeof(double) + sizeof(int)) << APPLY_SLOG);
     static int per_sm[64] = {0};  // resident blocks per SM, per device (-1: cannot run)
     int dev = 0;
@@ -1888,8 +2077,7 @@ bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64
                 LevelResult &out, uint32_t G, uint8_t *live, int *li, cudaStream_t s) {
     if (g.nnz > (fp64 ? LEVEL_MAX_EDGES_F64 : LEVEL_MAX_EDGES) || mb.feat_kept || mb.choice || !cl.dstart) return false;
     // a vertex's communities must fit the block classes' table
-    const uint32_t cap = fp64 ? LEVEL_CAP<true> : LEVEL_CAP<false>;
-    if (g.n > cap * 3 / 4 && (cl.cls_count(CLS_HUGE) || (fp64 && cl.cls_count(CLS_BIG)))) return false;
+    if (g.n > LEVEL_CAP * 3 / 4 && cl.cls_count(CLS_HUGE)) return false;
     // a wave must fit the warps' task and mover lists, and the CTAs' lists of block-class movers
     int need = 1;
     for (int wv = 0; wv < cl.W; wv++) {

@@ -157,7 +157,7 @@ static cudaStream_t tune_prologue(const DevGraph &g, const uint64_t *offsets, co
     cudaStream_t s = capture_stream();
     size_t mk = arena().mark();
     double *K = arena().get<double>(g.n);
-    double *m_dev = arena().get<double>(1);
+    double *m_dev = arena().get<double>(2);
     const double m = vertex_weights(g, K, m_dev, s);
     arena().release(mk);
     GSP_REQUIRE(m > 0.0, "gsp_autotune: the graph has no edges");

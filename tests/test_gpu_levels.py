@@ -81,3 +81,17 @@ def test_cluster_path_equals_launches(gsp, kw):
         Cs, qs, _ = gsp.louvain(*dev(*g), **kw)
         assert np.array_equal(C[int(gvo[i]):int(gvo[i + 1])], Cs.cpu().numpy()), f"graph {i}"
         assert q[i] == pytest.approx(qs, rel=1e-12, abs=1e-15), f"graph {i}"
+
+
+@pytest.mark.parametrize("exp", [-100, -21, 20, 90])
+@pytest.mark.parametrize("graph", ["rmat", "wide"])
+def test_mixed_scores_do_not_depend_on_the_weights_scale(gsp, graph, exp):
+    """Scaling every weight by a power of two scales the float32 scores
+    exactly, so every decision stays the same whatever the exponents of Sigma
+    (its conversion to float32 works on the bits)."""
+    off, tgt, w = SMALL[-1] if graph == "rmat" else SMALL[1]
+    C, q, st = gsp.louvain(*dev(off, tgt, w))
+    Cs, qs, sts = gsp.louvain(*dev(off, tgt, np.ldexp(w, exp)))
+    assert torch.equal(C, Cs)
+    assert sts["iterations"] == st["iterations"]
+    assert qs == pytest.approx(q, rel=1e-12)
