@@ -471,7 +471,7 @@ void louvain_batched_run(const DevGraph &g0, uint32_t G, const uint64_t *h_gvo0,
         GSP_CUDA(cudaMemsetAsync(mb.mark, 0, nv, s));
         Classes cl;
         classify_vertices(cur, cl, W, s, gid, gvo);
-        alloc_pool(mb, cl, s);
+        alloc_pool(mb, cl, o.precision == GSP_PREC_FP64, s);
         float ms_other = lap();
         mb.dq_g = dq_g;
         BatchMove mr = batch_move_loop(cur, cl, mb, G, tau, o, h_live, h_li, live,

@@ -626,15 +626,16 @@ static double max_value(const double *x, uint32_t n, cudaStream_t s) {
     return v;
 }
 
-// Hub hashtables: keys (u32), values (8 bytes) and an occupied-slot list
-// (u32) per slot.  The tables start empty; each sweep's scoring empties them.
-void alloc_pool(MoveBuffers &mb, const Classes &cl, cudaStream_t s) {
+// Hub hashtables, empty: 64-bit slots of key and float32 value (all bits set
+// when free), or, in the float64 mode, the keys and behind them the values.
+// A wave's scoring leaves them empty, so the waves share them.
+void alloc_pool(MoveBuffers &mb, const Classes &cl, bool fp64, cudaStream_t s) {
     mb.pool = nullptr;
     if (!cl.pool_slots) return;
-    size_t sa = align_up(cl.pool_slots, 64);
-    mb.pool = arena().alloc(sa * 16);
-    GSP_CUDA(cudaMemsetAsync(mb.pool, 0xFF, sa * sizeof(uint32_t), s));
-    GSP_CUDA(cudaMemsetAsync(static_cast<uint32_t *>(mb.pool) + sa, 0, sa * sizeof(double), s));
+    const size_t sa = align_up(cl.wave_pool_slots(), 64), keys = sa * (fp64 ? sizeof(uint32_t) : sizeof(uint64_t));
+    mb.pool = arena().alloc(keys + (fp64 ? sa * sizeof(double) : 0));
+    GSP_CUDA(cudaMemsetAsync(mb.pool, 0xFF, keys, s));
+    if (fp64) GSP_CUDA(cudaMemsetAsync(static_cast<char *>(mb.pool) + keys, 0, sa * sizeof(double), s));
 }
 
 // --------------------------------------------------------- GSP-Louvain run
@@ -750,7 +751,7 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
         }
         Classes cl;
         classify_vertices(cur, cl, W, s);
-        alloc_pool(mb, cl, s);
+        alloc_pool(mb, cl, fp64, s);
         float ms_other = t.lap();
         MoveLoopResult mr{0, 0, 0, 0, 0, 0.0, 0.0f};
         if (m > 0.0) mr = move_loop(cur, cl, mb, tau, o.max_iterations, sync, fp64, o.singleton_rule != 0, pr, s);
@@ -1069,7 +1070,7 @@ gsp_status gsp_move_sweep(const uint64_t *offsets, const uint32_t *targets, cons
     GSP_CUDA(cudaMemsetAsync(mb.mark, 0, n, s));
     Classes cl;
     classify_vertices(g, cl, 1, s);
-    alloc_pool(mb, cl, s);
+    alloc_pool(mb, cl, precision == GSP_PREC_FP64, s);
     set_iteration(mb, 0, s);
     move_wave(g, cl, mb, 0, true, precision == GSP_PREC_FP64, singleton_rule != 0, false, 0, 1, s);
     MoveCounters h;
@@ -1116,7 +1117,7 @@ gsp_status gsp_local_move(const uint64_t *offsets, const uint32_t *targets, cons
     GSP_CUDA(cudaMemsetAsync(mb.mark, 0, n, s));
     Classes cl;
     classify_vertices(g, cl, effective_waves(waves, sync), s);
-    alloc_pool(mb, cl, s);
+    alloc_pool(mb, cl, precision == GSP_PREC_FP64, s);
     PruneCtx pr;
     MoveLoopResult r = move_loop(g, cl, mb, tolerance, max_iterations, sync, precision == GSP_PREC_FP64,
                                  singleton_rule != 0, pr, s);

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <climits>
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -61,7 +62,14 @@ struct Classes {
     uint64_t pool_slots = 0;
     uint64_t *hub_tasks = nullptr;  // huge class: prefix of edge-chunk counts (count+1)
     std::vector<uint64_t> host_hub_tasks;
-    uint32_t *hub_occ_n = nullptr;  // huge class: occupied-slot count of each hub table
+    // slots of the hub tables of the wave that needs the most
+    uint64_t wave_pool_slots() const {
+        uint64_t most = 0;
+        for (int w = 0; w < W && pool_slots; w++)
+            most = std::max(most, host_pool_off[begin(CLS_HUGE, w) + count(CLS_HUGE, w) - cls_begin(CLS_HUGE)] -
+                                      host_pool_off[begin(CLS_HUGE, w) - cls_begin(CLS_HUGE)]);
+        return most;
+    }
     uint32_t begin(int cls, int wave) const { return start[cls * W + wave]; }
     uint32_t count(int cls, int wave) const { return start[cls * W + wave + 1] - start[cls * W + wave]; }
     uint32_t cls_begin(int cls) const { return start[cls * W]; }
@@ -202,7 +210,7 @@ void reset_left(MoveBuffers &mb, uint32_t n, cudaStream_t s);
 // before each sweep's launches or graph replay (a captured graph keeps the
 // kernel arguments of its capture).
 void set_iteration(MoveBuffers &mb, int iteration, cudaStream_t s);
-void alloc_pool(MoveBuffers &mb, const Classes &cl, cudaStream_t s);
+void alloc_pool(MoveBuffers &mb, const Classes &cl, bool fp64, cudaStream_t s);
 double sweep_bytes(const MoveCounters &h, int wt);
 cudaEvent_t pool_event();
 void reset_event_pool();

@@ -144,6 +144,31 @@ template <> struct Table<float> {
     // slots [first, ...) of a region of `total` slots at base
     __device__ Table(unsigned char *base, uint32_t, uint32_t first)
         : t(reinterpret_cast<unsigned long long *>(base) + first) {}
+    __device__ explicit Table(unsigned long long *global) : t(global) {}
+    // Add N distinct communities (EMPTY: none) to a table of cap slots in global
+    // memory, all first probes in flight together.
+    template <int N> __device__ void publish(uint32_t cap, const uint32_t (&c)[N], const float (&v)[N]) {
+        unsigned long long old[N];
+#pragma unroll
+        for (int u = 0; u < N; u++)
+            if (c[u] != EMPTY)
+                old[u] = atomicCAS(t + __umulhi(hash32(c[u]), cap), FREE,
+                                   ((unsigned long long)c[u] << 32) | __float_as_uint(v[u]));
+#pragma unroll
+        for (int u = 0; u < N; u++) {
+            if (c[u] == EMPTY || old[u] == FREE) continue;
+            uint32_t h = __umulhi(hash32(c[u]), cap);
+            for (uint32_t probe = 0; probe < cap; probe++) {
+                if ((uint32_t)(old[u] >> 32) == c[u]) {
+                    atomicAdd(reinterpret_cast<float *>(t + h), v[u]);
+                    break;
+                }
+                if (++h == cap) h = 0;
+                old[u] = atomicCAS(t + h, FREE, ((unsigned long long)c[u] << 32) | __float_as_uint(v[u]));
+                if (old[u] == FREE) break;
+            }
+        }
+    }
     __device__ void clear(uint32_t s) { t[s] = FREE; }
     __device__ uint32_t get(uint32_t s, float &v) const {
         const unsigned long long e = t[s];
@@ -174,6 +199,22 @@ template <> struct Table<double> {
     __device__ Table(unsigned char *base, uint32_t total, uint32_t first)
         : keys(reinterpret_cast<uint32_t *>(base) + first),
           vals(reinterpret_cast<double *>(base + (size_t)total * sizeof(uint32_t)) + first) {}
+    __device__ Table(uint32_t *gkeys, double *gvals) : keys(gkeys), vals(gvals) {}
+    template <int N> __device__ void publish(uint32_t cap, const uint32_t (&c)[N], const double (&v)[N]) {
+#pragma unroll
+        for (int u = 0; u < N; u++) {
+            if (c[u] == EMPTY) continue;
+            uint32_t h = __umulhi(hash32(c[u]), cap);
+            for (uint32_t probe = 0; probe < cap; probe++) {
+                const uint32_t old = atomicCAS(keys + h, EMPTY, c[u]);
+                if (old == EMPTY || old == c[u]) {
+                    atomicAdd(vals + h, v[u]);
+                    break;
+                }
+                if (++h == cap) h = 0;
+            }
+        }
+    }
     __device__ void clear(uint32_t s) {
         keys[s] = EMPTY;
         vals[s] = 0.0;
@@ -1436,37 +1477,53 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
 }
 
 // --------------------------------------------------------------------------
-// Hub vertices (degree > 2048), processed by the whole grid:
+// Hub vertices (degree > 8192), processed by the whole grid:
 //   prepare: read and clear each hub's flag, snapshot its community;
 //   insert:  the hub's edges are cut into HUB_CHUNK-edge tasks; a block
-//            combines a task's communities in a shared-memory table, then
-//            publishes the distinct ones to the hub's global table (new keys
-//            append their slot to the hub's occupied list);
-//   score:   all threads stride over the occupied list (and reset the slots
-//            for the next sweep); per-block best per hub;
-//   decide:  one warp per hub reduces the block bests and decides the move.
+//            combines a task's communities in a shared table, then its threads
+//            publish the slots they claimed to the hub's global table;
+//   score:   the hub's tasks read its table through, each its share of the
+//            slots, score what is there and empty it; the block that ends last
+//            for a hub reduces the tasks' bests and decides;
+//   mark:    all blocks re-mark the movers' neighbours (k_mark_big).
+// The tables are empty between waves, so nothing is cleared ahead and every
+// wave uses the same memory.  Reading a table through moves 16-32 bytes an edge
+// in whole lines (tables of 1.5 slots an edge instead of 2-4 moved less and were
+// slower, R-MAT 24 98 -> 104 ms: longer probes); the list of occupied slots that it replaces was appended to
+// behind a counter per block and cost a sector per entry to follow.
+// The chain of a wave went from three memsets and five kernels to four kernels.
 // --------------------------------------------------------------------------
-constexpr int HUB_SLOG = 11;  // shared table of 2 * HUB_CHUNK slots
+constexpr int HUB_SLOG = 11;     // shared table of 2 * HUB_CHUNK slots
+constexpr int HUB_THREADS = 512;  // 4 blocks of 32 registers a thread per SM: all its warps
+constexpr int HUB_EPT = HUB_CHUNK / HUB_THREADS;  // edges of a task per thread
 
 struct HubArgs {
     const uint32_t *hubs;
     uint32_t nh;
-    const uint64_t *pool_off;  // per hub
+    const uint64_t *pool_off;  // per hub (nh + 1 entries): slots of its table
     const uint64_t *tasks;     // per hub: prefix of chunk counts (nh + 1 entries, tasks[0] = base)
-    uint32_t *keys;
-    void *vals;
-    uint32_t *occ;
-    uint32_t *occ_n;    // per hub
+    void *keys, *vals;         // the pool: 64-bit slots (float32) or keys and values (float64)
     void *kid;          // per hub, V
     uint8_t *go;        // per hub
     uint32_t *d;        // per hub
+    uint32_t *done;     // per hub: tasks scored
     void *best_s;       // per task, S
     uint32_t *best_c;   // per task
     uint32_t *big, *nbig;
 };
 
-template <int SYNC>
+template <typename V> __device__ __forceinline__ Table<V> hub_table(const HubArgs &h, uint32_t t);
+template <> __device__ __forceinline__ Table<float> hub_table<float>(const HubArgs &h, uint32_t t) {
+    return Table<float>(static_cast<unsigned long long *>(h.keys) + (h.pool_off[t] - h.pool_off[0]));
+}
+template <> __device__ __forceinline__ Table<double> hub_table<double>(const HubArgs &h, uint32_t t) {
+    const uint64_t o = h.pool_off[t] - h.pool_off[0];
+    return Table<double>(static_cast<uint32_t *>(h.keys) + o, static_cast<double *>(h.vals) + o);
+}
+
+template <typename V, int SYNC>
 __global__ void k_hub_prepare(MoveArgs a, HubArgs h) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *h.nbig = 0;
     for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < h.nh; t += gridDim.x * blockDim.x) {
         uint32_t i = h.hubs[t];
         uint8_t go = ld_state<SYNC>(a.act + i);
@@ -1476,165 +1533,183 @@ __global__ void k_hub_prepare(MoveArgs a, HubArgs h) {
         }
         h.go[t] = go;
         h.d[t] = ld_state<SYNC>(a.C + i);
+        h.done[t] = 0;
+        static_cast<V *>(h.kid)[t] = V(0);
     }
 }
 
 template <typename WT, bool F64, int SYNC>
-__global__ void __launch_bounds__(256) k_hub_insert(MoveArgs a, HubArgs h) {
+__global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_insert(MoveArgs a, HubArgs h) {
     using V = typename std::conditional<F64, double, float>::type;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    uint32_t *skeys = reinterpret_cast<uint32_t *>(dyn_smem);
-    V *svals = reinterpret_cast<V *>(dyn_smem + sizeof(uint32_t) * (1u << HUB_SLOG));
-    uint16_t *socc = reinterpret_cast<uint16_t *>(dyn_smem + (sizeof(uint32_t) + sizeof(V)) * (1u << HUB_SLOG));
-    __shared__ V red[32];
-    __shared__ uint32_t s_nocc;
+    Table<V> tab(dyn_smem, 1u << HUB_SLOG, 0);
     const WT *w = static_cast<const WT *>(a.w);
     V *kidv = static_cast<V *>(h.kid);
-    for (uint32_t s = threadIdx.x; s < (1u << HUB_SLOG); s += blockDim.x) { skeys[s] = EMPTY; svals[s] = V(0); }
-    if (threadIdx.x == 0) s_nocc = 0;
+    for (uint32_t s = threadIdx.x; s < (1u << HUB_SLOG); s += HUB_THREADS) tab.clear(s);
+    __syncthreads();
     const uint64_t base = h.tasks[0], total = h.tasks[h.nh] - base;
     for (uint64_t task = blockIdx.x; task < total; task += gridDim.x) {
-        uint32_t t = task_item(h.tasks, h.nh, task + base);
+        const uint32_t t = task_item(h.tasks, h.nh, task + base);
         if (!h.go[t]) continue;
-        uint64_t chunk = task + base - h.tasks[t];
-        uint32_t i = h.hubs[t], d = h.d[t];
-        uint64_t e1 = a.off[i + 1];
-        uint64_t b = a.off[i] + chunk * HUB_CHUNK;
-        uint64_t e = min(b + HUB_CHUNK, e1);
-        V kid = 0;
-        scan_edges<4, SYNC, V>(a.tgt, w, a.C, i, d, b, e, threadIdx.x, blockDim.x, kid,
-                               [&](uint32_t c, V wv) { smem_add<V>(skeys, svals, HUB_SLOG, socc, &s_nocc, c, wv); });
-        kid = block_sum<V>(kid, red);
-        if (threadIdx.x == 0 && kid != V(0)) atomicAdd(kidv + t, kid);
-        int glog = ceil_log2((uint32_t)(2 * (e1 - a.off[i])));
-        publish_block_table<V>(skeys, svals, socc, &s_nocc, h.keys + h.pool_off[t],
-                               static_cast<V *>(h.vals) + h.pool_off[t], glog, h.occ + h.pool_off[t], h.occ_n + t);
+        const uint32_t i = h.hubs[t], d = h.d[t];
+        const uint64_t b0 = a.off[i], e1 = a.off[i + 1];
+        const uint64_t b = b0 + (task + base - h.tasks[t]) * HUB_CHUNK;
+        const uint64_t e = min(b + HUB_CHUNK, e1);
+        uint32_t j[HUB_EPT], c[HUB_EPT], slot[HUB_EPT];
+        V wv[HUB_EPT], kid = 0;
+#pragma unroll
+        for (int u = 0; u < HUB_EPT; u++) {
+            const uint64_t p = b + u * HUB_THREADS + threadIdx.x;
+            j[u] = p < e ? __ldg(a.tgt + p) : i;
+            wv[u] = p < e ? (V)__ldg(w + p) : V(0);
+        }
+#pragma unroll
+        for (int u = 0; u < HUB_EPT; u++) c[u] = j[u] != i ? ld_state<SYNC>(a.C + j[u]) : EMPTY;
+#pragma unroll
+        for (int u = 0; u < HUB_EPT; u++) {
+            slot[u] = EMPTY;
+            if (c[u] == EMPTY) continue;
+            if (c[u] == d) kid += wv[u];
+            else slot[u] = tab.add(HUB_SLOG, c[u], wv[u]);
+        }
+        kid = warp_sum(kid);
+        if ((threadIdx.x & 31) == 0 && kid != V(0)) atomicAdd(kidv + t, kid);
+        __syncthreads();  // the task is combined
+        V val[HUB_EPT];
+#pragma unroll
+        for (int u = 0; u < HUB_EPT; u++) {
+            c[u] = EMPTY;
+            if (slot[u] == EMPTY) continue;
+            c[u] = tab.get(slot[u], val[u]);
+            tab.clear(slot[u]);
+        }
+        __syncthreads();  // the shared table is empty
+        hub_table<V>(h, t).template publish<HUB_EPT>((uint32_t)(h.pool_off[t + 1] - h.pool_off[t]), c, val);
     }
 }
 
-// Scoring uses the insert's task split: task k of a hub scores occupied
-// entries [k*HUB_CHUNK, (k+1)*HUB_CHUNK) (a hub has at most one distinct
-// community per edge) and leaves its best in best[task].
+// The move of hub t, its tasks' bests all written: one warp.
+template <bool F64, int SYNC>
+__device__ void hub_decide(const MoveArgs &a, const HubArgs &h, uint32_t t, LocalCtr &lc) {
+    using V = typename std::conditional<F64, double, float>::type;
+    using SC = Score<F64>;
+    using S = typename SC::S;
+    const int lane = threadIdx.x & 31;
+    const V *kidv = static_cast<const V *>(h.kid);
+    const S *bs = static_cast<const S *>(h.best_s);
+    const uint64_t base = h.tasks[0];
+    const uint32_t i = h.hubs[t], d = h.d[t];
+    S best = -INFINITY;
+    uint32_t bestc = EMPTY;
+    for (uint64_t k = h.tasks[t] - base + lane; k < h.tasks[t + 1] - base; k += 32) {
+        const S v = __ldcg(bs + k);
+        const uint32_t c = __ldcg(h.best_c + k);
+        if (c != EMPTY && better(v, c, best, bestc)) { best = v; bestc = c; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        S v2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        uint32_t c2 = __shfl_xor_sync(0xFFFFFFFFu, bestc, o);
+        if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
+    }
+    if (lane != 0) return;
+    const double Ki = a.K[i];
+    const uint64_t deg = a.off[i + 1] - a.off[i];
+    const double m = vertex_m(a, i, a.m[0]);
+    const SC sc = make_score<F64>(Ki, kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, a.m[1]), true);
+    const double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
+    int mv = 0;
+    if (bestc != EMPTY && sc.gains(best)) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
+    lc.vertices++;
+    lc.edges += deg;
+    if (mv) {  // neighbours are re-marked by k_mark_big
+        lc.moved++;
+        lc.dq += gain;
+        add_graph_gain(a, i, gain);
+        lc.marked += deg;
+        h.big[atomicAdd(h.nbig, 1u)] = i;
+    }
+    record_visit(a, i, (uint32_t)deg, Ki, (double)kidv[t], gain, m, mv);
+}
+
+// Scoring uses the insert's task split: task k of a hub's n tasks takes the
+// slots [cap k / n, cap (k + 1) / n) of its table and leaves its best in
+// best[task].
 template <typename WT, bool F64, int SYNC>
-__global__ void __launch_bounds__(256) k_hub_score(MoveArgs a, HubArgs h) {
+__global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_score(MoveArgs a, HubArgs h) {
     using V = typename std::conditional<F64, double, float>::type;
     using SC = Score<F64>;
     using S = typename SC::S;
     __shared__ S red_s[32];
     __shared__ uint32_t red_c[32];
+    __shared__ uint32_t s_last;
     const V *kidv = static_cast<const V *>(h.kid);
     S *bs = static_cast<S *>(h.best_s);
-    const double m0 = *a.m;
-    const double inv0 = a.m[1];
+    const double m0 = a.m[0], inv0 = a.m[1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t base = h.tasks[0], total = h.tasks[h.nh] - base;
+    LocalCtr lc;
     for (uint64_t task = blockIdx.x; task < total; task += gridDim.x) {
-        uint32_t t = task_item(h.tasks, h.nh, task + base);
+        const uint32_t t = task_item(h.tasks, h.nh, task + base);
         if (!h.go[t]) continue;
-        uint64_t k0 = (task + base - h.tasks[t]) * HUB_CHUNK;
-        uint32_t i = h.hubs[t], d = h.d[t];
-        uint32_t *keys = h.keys + h.pool_off[t];
-        V *vals = static_cast<V *>(h.vals) + h.pool_off[t];
-        const uint32_t *occ = h.occ + h.pool_off[t];
-        uint64_t k1 = min(k0 + HUB_CHUNK, (uint64_t)h.occ_n[t]);
-        SC sc = make_score<F64>(a.K[i], kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
-                                vertex_inv_m(a, i, inv0), true);
+        const uint64_t n = h.tasks[t + 1] - h.tasks[t], k = task + base - h.tasks[t];
+        const uint32_t i = h.hubs[t], d = h.d[t];
+        const uint64_t cap = h.pool_off[t + 1] - h.pool_off[t];
+        const uint32_t s0 = (uint32_t)(cap * k / n), s1 = (uint32_t)(cap * (k + 1) / n);
+        Table<V> tab = hub_table<V>(h, t);
+        const SC sc = make_score<F64>(a.K[i], kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
+                                      vertex_inv_m(a, i, inv0), true);
         S best = -INFINITY;
-        uint32_t bestc = EMPTY;
-        // U entries per thread per round; each level of the gather chain
-        // (occupied list -> slot -> Sigma) is issued for all U at once
-        constexpr int U = 8;
-        for (uint64_t kb = k0 + threadIdx.x; kb < k1; kb += (uint64_t)U * blockDim.x) {
-            uint32_t slot[U], c[U];
+        uint32_t bestc = EMPTY, ncand = 0;
+        // U slots per thread per round, their gathers of Sigma issued at once
+        constexpr int U = 4;
+        for (uint32_t sb = s0 + threadIdx.x; sb < s1; sb += U * HUB_THREADS) {
+            uint32_t c[U];
             V val[U];
             double sg[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                uint64_t k = kb + (uint64_t)u * blockDim.x;
-                slot[u] = k < k1 ? occ[k] : EMPTY;
+                const uint32_t s = sb + u * HUB_THREADS;
+                c[u] = s < s1 ? tab.get(s, val[u]) : EMPTY;
             }
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                c[u] = slot[u] != EMPTY ? keys[slot[u]] : EMPTY;
-                val[u] = slot[u] != EMPTY ? vals[slot[u]] : V(0);
+                sg[u] = 0.0;
+                if (c[u] == EMPTY) continue;
+                tab.clear(sb + u * HUB_THREADS);
+                sg[u] = ld_state<SYNC>(a.Sig + c[u]);
             }
-#pragma unroll
-            for (int u = 0; u < U; u++) sg[u] = c[u] != EMPTY ? ld_state<SYNC>(a.Sig + c[u]) : 0.0;
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 if (c[u] == EMPTY) continue;
-                S v = sc.score(val[u], sg[u]);
+                ncand++;
+                const S v = sc.score(val[u], sg[u]);
                 if (better(v, c[u], best, bestc)) { best = v; bestc = c[u]; }
             }
         }
+        lc.candidates += ncand;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             S v2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
             uint32_t c2 = __shfl_xor_sync(0xFFFFFFFFu, bestc, o);
             if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
         }
-        __syncthreads();
+        __syncthreads();  // the previous task's reduction is over
         if (lane == 0) { red_s[wid] = best; red_c[wid] = bestc; }
         __syncthreads();
         if (threadIdx.x == 0) {
-            for (int k = 1; k < (int)(blockDim.x >> 5); k++)
-                if (better(red_s[k], red_c[k], best, bestc)) { best = red_s[k]; bestc = red_c[k]; }
+            for (int x = 1; x < HUB_THREADS / 32; x++)
+                if (better(red_s[x], red_c[x], best, bestc)) { best = red_s[x]; bestc = red_c[x]; }
             bs[task] = best;
             h.best_c[task] = bestc;
+            __threadfence();  // the best is visible before its task counts as done
+            s_last = atomicAdd(h.done + t, 1u) == (uint32_t)n - 1;
         }
-    }
-}
-
-template <bool F64, int SYNC>
-__global__ void k_hub_decide(MoveArgs a, HubArgs h) {
-    using V = typename std::conditional<F64, double, float>::type;
-    using SC = Score<F64>;
-    using S = typename SC::S;
-    const V *kidv = static_cast<const V *>(h.kid);
-    const S *bs = static_cast<const S *>(h.best_s);
-    const double m0 = *a.m;
-    const double inv0 = a.m[1];
-    const int lane = threadIdx.x & 31;
-    uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint64_t base = h.tasks[0];
-    LocalCtr lc;
-    for (uint32_t t = warp; t < h.nh; t += nwarps) {
-        if (!h.go[t]) continue;
-        uint32_t i = h.hubs[t], d = h.d[t];
-        S best = -INFINITY;
-        uint32_t bestc = EMPTY;
-        for (uint64_t k = h.tasks[t] - base + lane; k < h.tasks[t + 1] - base; k += 32) {
-            S v = bs[k];
-            uint32_t c = h.best_c[k];
-            if (c != EMPTY && better(v, c, best, bestc)) { best = v; bestc = c; }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            S v2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-            uint32_t c2 = __shfl_xor_sync(0xFFFFFFFFu, bestc, o);
-            if (better(v2, c2, best, bestc)) { best = v2; bestc = c2; }
-        }
-        if (lane == 0) {
-            double Ki = a.K[i];
-            uint64_t deg = a.off[i + 1] - a.off[i];
-            const double m = vertex_m(a, i, m0);
-            SC sc = make_score<F64>(Ki, kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, inv0), true);
-            double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
-            int mv = 0;
-            if (bestc != EMPTY && sc.gains(best)) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
-            lc.vertices++;
-            lc.edges += deg;
-            lc.candidates += h.occ_n[t];
-            h.occ_n[t] = 0;
-            if (mv) {  // neighbours are re-marked by k_mark_big
-                lc.moved++;
-                lc.dq += gain;
-                add_graph_gain(a, i, gain);
-                lc.marked += deg;
-                h.big[atomicAdd(h.nbig, 1u)] = i;
-            }
-            record_visit(a, i, (uint32_t)deg, Ki, (double)kidv[t], gain, m, mv);
+        __syncthreads();
+        if (s_last && wid == 0) {
+            __threadfence();
+            hub_decide<F64, SYNC>(a, h, t, lc);
+            __syncwarp();
         }
     }
     flush_counters(lc, a.ctr);
@@ -1769,8 +1844,6 @@ void classify_vertices(const DevGraph &g, Classes &cl, int waves, cudaStream_t s
         GSP_CUDA(cudaMemcpyAsync(cl.host_hub_tasks.data(), cl.hub_tasks, sizeof(uint64_t) * (nh + 1),
                                  cudaMemcpyDeviceToHost, s));
         GSP_CUDA(cudaStreamSynchronize(s));
-        cl.hub_occ_n = arena().get<uint32_t>(nh);
-        GSP_CUDA(cudaMemsetAsync(cl.hub_occ_n, 0, sizeof(uint32_t) * nh, s));
     }
 }
 
@@ -1802,8 +1875,8 @@ SideStreams &side_streams() {
 // class on side stream 3, the group classes on the main stream; all join
 // before the wave's moves are applied.
 template <typename WT, bool F64, int SYNC>
-static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, uint32_t *pool_keys, void *pool_vals,
-                        uint32_t *pool_occ, uint32_t *big, uint32_t *nbig, cudaStream_t main) {
+static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, void *pool, uint32_t *big, uint32_t *nbig,
+                        cudaStream_t main) {
     using V = typename std::conditional<F64, double, float>::type;
     SideStreams &ss = side_streams();
     const int f = ss.next;
@@ -1888,40 +1961,27 @@ static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, uint32_t
         h.nh = nh;
         h.pool_off = cl.pool_off + rel;
         h.tasks = cl.hub_tasks + rel;
-        h.keys = pool_keys;
-        h.vals = pool_vals;
-        h.occ = pool_occ;
-        h.occ_n = cl.hub_occ_n + rel;
+        h.keys = pool;
+        h.vals = F64 ? static_cast<uint32_t *>(pool) + align_up(cl.wave_pool_slots(), 64) : nullptr;
         h.kid = arena().alloc(sizeof(V) * nh);
         h.go = arena().get<uint8_t>(nh);
         h.d = arena().get<uint32_t>(nh);
+        h.done = arena().get<uint32_t>(nh);
         uint64_t ntasks = cl.host_hub_tasks[rel + nh] - cl.host_hub_tasks[rel];
         h.best_s = arena().alloc(sizeof(S) * ntasks);
         h.best_c = arena().get<uint32_t>(ntasks);
         h.big = big;
         h.nbig = nbig;
-        // this wave's tables: one contiguous slice of the pool, cleared with
-        // coalesced memsets
-        uint64_t first = cl.host_pool_off[rel], last = cl.host_pool_off[rel + nh];
-        GSP_CUDA(cudaMemsetAsync(pool_keys + first, 0xFF, sizeof(uint32_t) * (last - first), s));
-        GSP_CUDA(cudaMemsetAsync(static_cast<V *>(pool_vals) + first, 0, sizeof(V) * (last - first), s));
-        GSP_CUDA(cudaMemsetAsync(h.kid, 0, sizeof(V) * nh, s));
-        k_hub_prepare<SYNC><<<grid_for(nh, 256), 256, 0, s>>>(a, h);
+        k_hub_prepare<V, SYNC><<<grid_for(nh, 256), 256, 0, s>>>(a, h);
         GSP_CHECK_LAUNCH();
-        constexpr size_t hsmem = (sizeof(uint32_t) + sizeof(V) + sizeof(uint16_t)) << HUB_SLOG;
-        static bool attr = false;
-        if (!attr) {
-            GSP_CUDA(cudaFuncSetAttribute(k_hub_insert<WT, F64, SYNC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)hsmem));
-            attr = true;
-        }
+        constexpr size_t hsmem = Table<V>::slot_bytes << HUB_SLOG;
         // one block per task at most: small waves launch only what they use
         const unsigned hub_grid = (unsigned)std::min<uint64_t>(ntasks, (uint64_t)sm * tn.hub);
-        k_hub_insert<WT, F64, SYNC><<<hub_grid, 256, hsmem, s>>>(a, h);
+        k_hub_insert<WT, F64, SYNC><<<hub_grid, HUB_THREADS, hsmem, s>>>(a, h);
         GSP_CHECK_LAUNCH();
-        k_hub_score<WT, F64, SYNC><<<hub_grid, 256, 0, s>>>(a, h);
+        k_hub_score<WT, F64, SYNC><<<hub_grid, HUB_THREADS, 0, s>>>(a, h);
         GSP_CHECK_LAUNCH();
-        k_hub_decide<F64, SYNC><<<grid_for((uint64_t)nh * 32, 256), 256, 0, s>>>(a, h);
+        k_mark_big<<<dim3(sm, 16), 256, 0, s>>>(a.off, a.tgt, big, nbig, a.mark);
         GSP_CHECK_LAUNCH();
         arena().release(mk);
     }
@@ -2112,14 +2172,8 @@ void move_wave(const DevGraph &g, const Classes &cl, MoveBuffers &mb, int wave, 
                bool learned, int iteration, int max_iterations, cudaStream_t s) {
     (void)learned;
     MoveArgs a = make_move_args(g, mb, sync, rule, iteration, max_iterations);
-    // pool layout: keys (u32), values (8 bytes per slot), occupied-slot list (u32)
-    uint32_t *pool_keys = static_cast<uint32_t *>(mb.pool);
-    const size_t sa = align_up(cl.pool_slots, 64);
-    void *pool_vals = pool_keys ? static_cast<void *>(pool_keys + sa) : nullptr;
-    uint32_t *pool_occ = pool_keys ? pool_keys + 3 * sa : nullptr;
-    GSP_CUDA(cudaMemsetAsync(mb.nbig, 0, sizeof(uint32_t), s));
 #define GSP_WAVE(WT, F64, SYNC) \
-    launch_wave<WT, F64, SYNC>(cl, a, wave, pool_keys, pool_vals, pool_occ, mb.big, mb.nbig, s)
+    launch_wave<WT, F64, SYNC>(cl, a, wave, mb.pool, mb.big, mb.nbig, s)
     if (g.wt == GSP_W_F32) {
         if (fp64) { if (sync) GSP_WAVE(float, true, true); else GSP_WAVE(float, true, false); }
         else { if (sync) GSP_WAVE(float, false, true); else GSP_WAVE(float, false, false); }
@@ -2128,10 +2182,6 @@ void move_wave(const DevGraph &g, const Classes &cl, MoveBuffers &mb, int wave, 
         else { if (sync) GSP_WAVE(double, false, true); else GSP_WAVE(double, false, false); }
     }
 #undef GSP_WAVE
-    if (cl.count(CLS_HUGE, wave)) {  // hub movers re-mark their neighbours
-        k_mark_big<<<dim3(sm_count(), 16), 256, 0, s>>>(g.off, g.tgt, mb.big, mb.nbig, a.mark);
-        GSP_CHECK_LAUNCH();
-    }
 }
 
 void apply_moves(const DevGraph &g, MoveBuffers &mb, uint32_t n_hint, cudaStream_t s) {
