@@ -6,6 +6,7 @@
 //     paper's "holey" CSR with gaps);
 //  3. per community, an open-addressing table over the edges of all members
 //     (self-loops included) merges the weights per neighbouring community:
+//       total degree <= 64   : one warp, 128-slot table in shared memory
 //       total degree <= 512  : one warp, 1024-slot table in shared memory
 //       total degree <= 2048 : one block, 4096-slot table in shared memory
 //       larger               : the whole grid, edge-chunk tasks combined in
@@ -20,9 +21,10 @@
 // Weights are stored in float64; sums of float32-exact weights are exact in
 // float64, so every merged weight is order-independent and the output is
 // canonical.  The tables accumulate in integer units of the weights' lowest
-// set bit (64-bit integer atomics, native in shared memory) whenever the total
-// weight stays below 2^52 such units, and in float64 otherwise; the two give
-// the same sums.
+// set bit whenever the total weight stays below 2^52 such units: in 32 bits
+// that share a 64-bit word with their key when the total is below 2^32 (one
+// compare-and-swap claims a slot and stores its first weight), else in 64 bits
+// beside the keys; and in float64 otherwise.  All give the same sums.
 #include <climits>
 #include <cmath>
 
@@ -30,8 +32,8 @@
 
 namespace gsp {
 
-enum { ACLS_W = 0, ACLS_B, ACLS_L, NUM_ACLS };
-constexpr uint64_t ACLS_MAX[NUM_ACLS] = {512, 2048, ~0ull};
+enum { ACLS_S = 0, ACLS_W, ACLS_B, ACLS_L, NUM_ACLS };
+constexpr uint64_t ACLS_MAX[NUM_ACLS] = {64, 512, 2048, ~0ull};
 enum { RCLS_W = 0, RCLS_B, RCLS_L, NUM_RCLS };
 constexpr uint64_t RCLS_MAX[NUM_RCLS] = {32, 2048, ~0ull};
 
@@ -97,7 +99,7 @@ __global__ void k_cls_fill(const uint64_t *__restrict__ sz, uint32_t k, const ui
 
 struct IdClasses {
     uint32_t *list = nullptr;
-    uint32_t start[4] = {0, 0, 0, 0};
+    uint32_t start[5] = {0, 0, 0, 0, 0};
 };
 
 template <int NC>
@@ -119,6 +121,80 @@ static void classify_ids(const uint64_t *sz, uint32_t k, const uint64_t (&maxes)
     k_cls_fill<NC><<<gr, 256, 0, s>>>(sz, k, dmax, counts + NC, ic.list);
     GSP_CHECK_LAUNCH();
 }
+
+// Open-addressing table of the sums per neighbouring community, linear probing,
+// 2^logcap slots, more than the keys it meets.  add() returns the slot that the
+// call claimed, or EMPTY when the key was there.
+// The rows of the next level come out in slot order, so these tables hash with
+// another multiplier than those of local moving: with the same one, a row's
+// consecutive edges went to neighbouring slots there and collided (R-MAT 24,
+// second pass: 21.7 ms of moving instead of 17.3).
+__device__ __forceinline__ uint32_t agg_hash(uint32_t x) { return x * 0x85EBCA77u; }
+
+template <typename AV> struct AggTable {  // values beside the keys
+    uint32_t *keys;
+    AV *vals;
+    static constexpr size_t slot_bytes = sizeof(uint32_t) + sizeof(AV);
+    __device__ AggTable(unsigned char *base, uint32_t cap)  // the values first: their alignment
+        : keys(reinterpret_cast<uint32_t *>(base + (size_t)cap * sizeof(AV))), vals(reinterpret_cast<AV *>(base)) {}
+    __device__ AggTable(unsigned char *base, uint64_t cap, uint64_t first) : AggTable(base, 0u) {
+        keys = reinterpret_cast<uint32_t *>(base + cap * sizeof(AV)) + first;
+        vals += first;
+    }
+    __device__ void clear(uint64_t s) {
+        keys[s] = EMPTY;
+        vals[s] = AV(0);
+    }
+    __device__ uint32_t get(uint64_t s, AV &v) const {
+        const uint32_t k = keys[s];
+        if (k != EMPTY) v = vals[s];
+        return k;
+    }
+    template <bool SHARED> __device__ uint32_t add(int logcap, uint32_t c, AV w) {
+        const uint32_t mask = (1u << logcap) - 1u;
+        uint32_t h = logcap ? (agg_hash(c) >> (32 - logcap)) : 0u;
+        for (uint32_t probe = 0; probe <= mask; probe++) {
+            uint32_t old = SHARED ? *(volatile uint32_t *)(keys + h) : EMPTY;
+            if (old == EMPTY) old = atomicCAS(keys + h, EMPTY, c);
+            if (old == EMPTY || old == c) {
+                atomicAdd(vals + h, w);
+                return old == EMPTY ? h : EMPTY;
+            }
+            h = (h + 1) & mask;
+        }
+        return EMPTY;
+    }
+};
+template <> struct AggTable<uint32_t> {  // key and value in one word
+    unsigned long long *t;
+    static constexpr size_t slot_bytes = 8;
+    static constexpr unsigned long long FREE = ~0ull;
+    __device__ AggTable(unsigned char *base, uint32_t) : t(reinterpret_cast<unsigned long long *>(base)) {}
+    __device__ AggTable(unsigned char *base, uint64_t, uint64_t first)
+        : t(reinterpret_cast<unsigned long long *>(base) + first) {}
+    __device__ void clear(uint64_t s) { t[s] = FREE; }
+    __device__ uint32_t get(uint64_t s, uint32_t &v) const {
+        const unsigned long long e = t[s];
+        v = (uint32_t)e;
+        return (uint32_t)(e >> 32);
+    }
+    template <bool SHARED> __device__ uint32_t add(int logcap, uint32_t c, uint32_t w) {
+        const uint32_t mask = (1u << logcap) - 1u;
+        uint32_t h = logcap ? (agg_hash(c) >> (32 - logcap)) : 0u;
+        const unsigned long long e = ((unsigned long long)c << 32) | w;
+        for (uint32_t probe = 0; probe <= mask; probe++) {
+            unsigned long long old = SHARED ? *(volatile unsigned long long *)(t + h) : FREE;
+            if (old == FREE) old = atomicCAS(t + h, FREE, e);
+            if (old == FREE) return h;
+            if ((uint32_t)(old >> 32) == c) {
+                atomicAdd(reinterpret_cast<uint32_t *>(t + h), w);
+                return EMPTY;
+            }
+            h = (h + 1) & mask;
+        }
+        return EMPTY;
+    }
+};
 
 struct AggArgs {
     const uint64_t *off;
@@ -150,6 +226,34 @@ __device__ __forceinline__ void emit_slot(const AggArgs &a, uint32_t c, uint32_t
         uint64_t pos = a.yoff[c] + base + __popc(ballot & ((1u << lane) - 1u));
         a.htgt[pos] = key;
         a.hw[pos] = val;
+    }
+}
+
+// The same for N slots per lane, one reservation per warp: the rows of giant
+// communities are appended to by every block.
+template <int N, typename AV>
+__device__ __forceinline__ void emit_slots(const AggArgs &a, uint32_t c, const uint32_t (&key)[N], const AV (&val)[N],
+                                           uint32_t *cursor) {
+    const uint32_t FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    uint32_t bal[N], total = 0;
+#pragma unroll
+    for (int u = 0; u < N; u++) {
+        bal[u] = __ballot_sync(FULL, key[u] != EMPTY);
+        total += __popc(bal[u]);
+    }
+    if (!total) return;
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(cursor, total);
+    uint64_t pos = a.yoff[c] + __shfl_sync(FULL, base, 0);
+#pragma unroll
+    for (int u = 0; u < N; u++) {
+        if (key[u] != EMPTY) {
+            const uint64_t q = pos + __popc(bal[u] & ((1u << lane) - 1u));
+            a.htgt[q] = key[u];
+            a.hw[q] = Acc<AV>::val(val[u], a.xlsb);
+        }
+        pos += __popc(bal[u]);
     }
 }
 
@@ -197,27 +301,30 @@ __device__ __forceinline__ void warp_row_edges(const uint32_t *__restrict__ list
     }
 }
 
-constexpr int AGG_WCAP = 1024;
-constexpr int AGG_WWARPS = 4;
+// One warp per community of at most CAP / 2 edges.  Most communities of a
+// level are tiny (a grid's first pass has three vertices each): what counts is
+// how many warps are in flight, so communities of up to 64 edges get a 128-slot
+// table and fill an SM's warps, where 1024 slots for all left 16 warps
+// (2048^2 grid, first pass: 1.92 ms).
+constexpr int AGG_SCAP = 128, AGG_SWARPS = 8;
+constexpr int AGG_WCAP = 1024, AGG_WWARPS = 4;
 
-template <typename WT, typename AV>
-__global__ void __launch_bounds__(AGG_WWARPS * 32) k_agg_merge_warp(AggArgs a, const uint32_t *__restrict__ list,
-                                                                    uint32_t count) {
+template <int CAP, int WARPS, typename WT, typename AV>
+__global__ void __launch_bounds__(WARPS * 32) k_agg_merge_warp(AggArgs a, const uint32_t *__restrict__ list,
+                                                               uint32_t count) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    __shared__ uint32_t s_cur[AGG_WWARPS];
+    const uint32_t FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t *keys = reinterpret_cast<uint32_t *>(dyn_smem) + wid * AGG_WCAP;
-    AV *vals = reinterpret_cast<AV *>(dyn_smem + sizeof(uint32_t) * AGG_WCAP * AGG_WWARPS) + wid * AGG_WCAP;
+    AggTable<AV> tab(dyn_smem + (size_t)wid * CAP * AggTable<AV>::slot_bytes, (uint32_t)CAP);
     const WT *w = static_cast<const WT *>(a.w);
-    for (uint32_t t = blockIdx.x * AGG_WWARPS + wid; t < count; t += gridDim.x * AGG_WWARPS) {
+    for (uint32_t t = blockIdx.x * WARPS + wid; t < count; t += gridDim.x * WARPS) {
         uint32_t c = list[t];
         uint64_t cd = a.cdeg[c];
         uint64_t bound = cd < a.k ? cd : a.k;
         int logcap = ceil_log2((uint32_t)(2 * bound));
         if (logcap < 1) logcap = 1;
         uint32_t cap = 1u << logcap;
-        for (uint32_t s = lane; s < cap; s += 32) { keys[s] = EMPTY; vals[s] = AV(0); }
-        if (lane == 0) s_cur[wid] = 0;
+        for (uint32_t s = lane; s < cap; s += 32) tab.clear(s);
         __syncwarp();
         // edges inside the community (the super-vertex's self-loop) are summed
         // in registers: they are the most frequent key of the table
@@ -228,48 +335,58 @@ __global__ void __launch_bounds__(AGG_WWARPS * 32) k_agg_merge_warp(AggArgs a, c
             const uint32_t d = a.Cd[a.tgt[p]];
             const WT x = w[p];
             if (d == c) { selfw += Acc<AV>::of(x, a.xlsb); nself++; }
-            else ht_add<AV>(keys, vals, logcap, d, Acc<AV>::of(x, a.xlsb));
+            else tab.template add<true>(logcap, d, Acc<AV>::of(x, a.xlsb));
         });
         selfw = warp_sum(selfw);
         nself = warp_sum(nself);
         __syncwarp();
-        if (lane == 0 && nself) ht_add<AV>(keys, vals, logcap, c, selfw);
-        __syncwarp();
-        for (uint32_t s0 = 0; s0 < cap; s0 += 32) {
-            uint32_t s = s0 + lane;
-            uint32_t key = s < cap ? keys[s] : EMPTY;
-            emit_slot(a, c, key, s < cap ? Acc<AV>::val(vals[s], a.xlsb) : 0.0, key != EMPTY, &s_cur[wid]);
+        // the row: the self-loop, then the table in slot order
+        const uint64_t row = a.yoff[c];
+        uint32_t n = 0;
+        if (nself) {
+            if (lane == 0) {
+                a.htgt[row] = c;
+                a.hw[row] = Acc<AV>::val(selfw, a.xlsb);
+            }
+            n = 1;
         }
-        __syncwarp();
-        if (lane == 0) a.rowlen[c] = s_cur[wid];
+        for (uint32_t s0 = 0; s0 < cap; s0 += 32) {
+            const uint32_t s = s0 + lane;
+            AV v = AV(0);
+            const uint32_t key = s < cap ? tab.get(s, v) : EMPTY;
+            const uint32_t ballot = __ballot_sync(FULL, key != EMPTY);
+            if (key != EMPTY) {
+                const uint64_t pos = row + n + __popc(ballot & ((1u << lane) - 1u));
+                a.htgt[pos] = key;
+                a.hw[pos] = Acc<AV>::val(v, a.xlsb);
+            }
+            n += __popc(ballot);
+        }
+        if (lane == 0) a.rowlen[c] = n;
         __syncwarp();
     }
 }
 
-// One block per community; 4096-slot table in dynamic shared memory with a
-// list of occupied slots (emission and clearing touch only those).  The
-// members' edges are numbered through a prefix of member degrees in shared
-// memory and dealt out evenly over the block (a member-per-warp split leaves
-// warps waiting on the longest member).
+// One block per community; 4096-slot table in dynamic shared memory, empty
+// between communities.  The members' edges are numbered through a prefix of
+// member degrees in shared memory and dealt out evenly over the block (a
+// member-per-warp split leaves warps waiting on the longest member).
 constexpr int AGG_BCAP = 4096;
 constexpr int AGG_BMEM = 2048;  // members staged in shared memory (total degree <= 2048 bounds them)
 
 template <typename WT, typename AV>
 __global__ void __launch_bounds__(256) k_agg_merge_block(AggArgs a, const uint32_t *__restrict__ list, uint32_t count) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    uint32_t *keys = reinterpret_cast<uint32_t *>(dyn_smem);
-    AV *vals = reinterpret_cast<AV *>(dyn_smem + sizeof(uint32_t) * AGG_BCAP);
-    uint16_t *occ = reinterpret_cast<uint16_t *>(dyn_smem + (sizeof(uint32_t) + sizeof(double)) * AGG_BCAP);
-    uint64_t *s_base = reinterpret_cast<uint64_t *>(
-        dyn_smem + (sizeof(uint32_t) + sizeof(double) + sizeof(uint16_t)) * AGG_BCAP);
+    AggTable<AV> tab(dyn_smem, (uint32_t)AGG_BCAP);
+    uint64_t *s_base = reinterpret_cast<uint64_t *>(dyn_smem + AggTable<AV>::slot_bytes * AGG_BCAP);
     uint32_t *s_pre = reinterpret_cast<uint32_t *>(s_base + AGG_BMEM);  // AGG_BMEM + 1 entries
-    __shared__ uint32_t s_cur, s_nocc;
+    __shared__ uint32_t s_cur;
     __shared__ AV s_red[32];
     __shared__ uint32_t s_redn[32], s_wsum[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
     const WT *w = static_cast<const WT *>(a.w);
-    for (uint32_t s = threadIdx.x; s < AGG_BCAP; s += blockDim.x) { keys[s] = EMPTY; vals[s] = AV(0); }
+    for (uint32_t s = threadIdx.x; s < AGG_BCAP; s += blockDim.x) tab.clear(s);
     for (uint32_t t = blockIdx.x; t < count; t += gridDim.x) {
         uint32_t c = list[t];
         uint64_t cd = a.cdeg[c];
@@ -277,7 +394,7 @@ __global__ void __launch_bounds__(256) k_agg_merge_block(AggArgs a, const uint32
         int logcap = ceil_log2((uint32_t)(2 * bound));
         if (logcap < 1) logcap = 1;
         __syncthreads();
-        if (threadIdx.x == 0) { s_cur = 0; s_nocc = 0; }
+        if (threadIdx.x == 0) s_cur = 0;
         __syncthreads();
         uint64_t q0 = a.coff[c], q1 = a.coff[c + 1];
         const uint32_t nm = (uint32_t)(q1 - q0);
@@ -287,7 +404,7 @@ __global__ void __launch_bounds__(256) k_agg_merge_block(AggArgs a, const uint32
             const uint32_t d = a.Cd[a.tgt[p]];
             const WT x = w[p];
             if (d == c) { selfw += Acc<AV>::of(x, a.xlsb); nself++; }
-            else smem_add<AV>(keys, vals, logcap, occ, &s_nocc, d, Acc<AV>::of(x, a.xlsb));
+            else tab.template add<true>(logcap, d, Acc<AV>::of(x, a.xlsb));
         };
         if (nm <= AGG_BMEM) {
             // member degrees -> exclusive prefix s_pre[0..nm], bases s_base
@@ -344,21 +461,16 @@ __global__ void __launch_bounds__(256) k_agg_merge_block(AggArgs a, const uint32
         }
         selfw = block_sum(selfw, s_red);
         nself = block_sum(nself, s_redn);
-        if (threadIdx.x == 0 && nself) smem_add<AV>(keys, vals, logcap, occ, &s_nocc, c, selfw);
+        if (threadIdx.x == 0 && nself) tab.template add<true>(logcap, c, selfw);
         __syncthreads();
-        uint32_t nocc = s_nocc;
-        for (uint32_t k0 = wid * 32; k0 < nocc; k0 += blockDim.x) {
-            uint32_t k = k0 + lane;
-            uint32_t slot = k < nocc ? occ[k] : 0;
-            emit_slot(a, c, k < nocc ? keys[slot] : EMPTY, k < nocc ? Acc<AV>::val(vals[slot], a.xlsb) : 0.0, k < nocc,
-                      &s_cur);
+        for (uint32_t s0 = wid * 32; s0 < (1u << logcap); s0 += blockDim.x) {
+            const uint32_t s = s0 + lane;
+            AV v = AV(0);
+            const uint32_t key = s < (1u << logcap) ? tab.get(s, v) : EMPTY;
+            if (key != EMPTY) tab.clear(s);  // leave the table empty for the next community
+            emit_slot(a, c, key, key != EMPTY ? Acc<AV>::val(v, a.xlsb) : 0.0, key != EMPTY, &s_cur);
         }
         __syncthreads();
-        for (uint32_t k = threadIdx.x; k < nocc; k += blockDim.x) {
-            uint32_t slot = occ[k];
-            keys[slot] = EMPTY;
-            vals[slot] = AV(0);
-        }
         if (threadIdx.x == 0) a.rowlen[c] = s_cur;
     }
 }
@@ -368,10 +480,10 @@ __global__ void __launch_bounds__(256) k_agg_merge_block(AggArgs a, const uint32
 // of member degrees in community-vertex order, so community c owns
 // [yoff[c], yoff[c+1])) and cut into AGG_CHUNK-edge tasks.  A block combines a
 // task's neighbour communities in a shared-memory table (each warp finds its
-// first member by binary search and walks the members forward), then
-// publishes the distinct ones to the community's global table; keys new to it
-// append their slot to the community's occupied list, which the extraction
-// walks.
+// first member by binary search and walks the members forward); a warp lists
+// the slots its lanes claimed (positions from ballots: one counter per block
+// took an add per distinct key) and publishes them to the community's global
+// table, which the extraction reads through.
 constexpr uint32_t AGG_CHUNK = 2048;
 constexpr uint32_t AGG_TASK_WARPS = 8;                    // k_agg_large_insert runs 256-thread blocks
 constexpr uint32_t AGG_SUB = AGG_CHUNK / AGG_TASK_WARPS;  // edges of a task per warp
@@ -422,19 +534,16 @@ __global__ void __launch_bounds__(256) k_agg_large_insert(AggArgs a, const uint3
                                                           const uint32_t *__restrict__ task_c,
                                                           const uint32_t *__restrict__ wstart,
                                                           const uint64_t *__restrict__ medge,
-                                                          const uint64_t *__restrict__ pool_off, uint32_t *pool_keys,
-                                                          AV *pool_vals, uint32_t *pool_occ, uint32_t *occ_n) {
+                                                          const uint64_t *__restrict__ pool_off, uint64_t pool_slots,
+                                                          unsigned char *pool) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    uint32_t *skeys = reinterpret_cast<uint32_t *>(dyn_smem);
-    AV *svals = reinterpret_cast<AV *>(dyn_smem + sizeof(uint32_t) * (1u << AGG_SLOG));
-    uint16_t *socc = reinterpret_cast<uint16_t *>(dyn_smem + (sizeof(uint32_t) + sizeof(AV)) * (1u << AGG_SLOG));
-    __shared__ uint32_t s_nocc;
-    __shared__ AV s_red[32];
-    __shared__ uint32_t s_redn[32];
     const WT *w = static_cast<const WT *>(a.w);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (uint32_t s = threadIdx.x; s < (1u << AGG_SLOG); s += blockDim.x) { skeys[s] = EMPTY; svals[s] = AV(0); }
-    if (threadIdx.x == 0) s_nocc = 0;
+    AggTable<AV> tab(dyn_smem, 1u << AGG_SLOG);
+    // slots claimed by the warp: at most one per edge of its slice
+    uint16_t *claimed = reinterpret_cast<uint16_t *>(dyn_smem + (AggTable<AV>::slot_bytes << AGG_SLOG)) + wid * AGG_SUB;
+    for (uint32_t s = threadIdx.x; s < (1u << AGG_SLOG); s += blockDim.x) tab.clear(s);
+    __syncthreads();
     const uint64_t total = tasks[count];
     for (uint64_t task = blockIdx.x; task < total; task += gridDim.x) {
         uint32_t t = task_c[task];
@@ -444,7 +553,7 @@ __global__ void __launch_bounds__(256) k_agg_large_insert(AggArgs a, const uint3
         uint64_t ch = a.yoff[c] + (task - tasks[t]) * AGG_CHUNK + (uint64_t)wid * AGG_SUB;
         uint64_t cend = min(ch + AGG_SUB, E1);
         AV selfw = AV(0);
-        uint32_t nself = 0;
+        uint32_t nself = 0, nclaimed = 0;
         if (ch < E1) {
             const uint64_t lo = wstart[task * AGG_TASK_WARPS + wid];  // last member with medge <= ch
             // A window of 32 members (lane l: member q + l, its end in the
@@ -481,60 +590,74 @@ __global__ void __launch_bounds__(256) k_agg_large_insert(AggArgs a, const uint3
                 const uint64_t rbase = __shfl_sync(FULL, wbase_l, r);
                 const uint64_t rprev = __shfl_sync(FULL, wend_l, (r + 31) & 31);
                 const uint64_t rstart = r ? rprev : wstart;
+                uint32_t slot = EMPTY;
                 if (tt < rend) {
                     const uint64_t p = rbase + (tt - rstart);
                     const uint32_t dd = a.Cd[a.tgt[p]];
                     if (dd == c) { selfw += Acc<AV>::of(w[p], a.xlsb); nself++; }
-                    else smem_add<AV>(skeys, svals, AGG_SLOG, socc, &s_nocc, dd, Acc<AV>::of(w[p], a.xlsb));
+                    else slot = tab.template add<true>(AGG_SLOG, dd, Acc<AV>::of(w[p], a.xlsb));
                 }
+                const uint32_t fresh = __ballot_sync(FULL, slot != EMPTY);
+                if (slot != EMPTY) claimed[nclaimed + __popc(fresh & ((1u << lane) - 1u))] = (uint16_t)slot;
+                nclaimed += __popc(fresh);
                 // members ending at or before rend are done
                 q += __popc(__ballot_sync(FULL, wend_l <= rend));
                 t0 = rend;
             }
         }
-        // the task's edges inside the community enter the table once
-        selfw = block_sum(selfw, s_red);
-        nself = block_sum(nself, s_redn);
-        if (threadIdx.x == 0 && nself)
-            smem_add<AV>(skeys, svals, AGG_SLOG, socc, &s_nocc, c, selfw);
-        uint64_t cd = a.cdeg[c];
-        uint64_t bound = cd < a.k ? cd : a.k;
+        const uint64_t cd = a.cdeg[c];
+        const uint64_t bound = cd < a.k ? cd : a.k;
         int glog = ceil_log2((uint32_t)(2 * bound));
         if (glog < 1) glog = 1;
-        publish_block_table<AV>(skeys, svals, socc, &s_nocc, pool_keys + pool_off[t], pool_vals + pool_off[t],
-                                    glog, pool_occ + pool_off[t], occ_n + t);
+        AggTable<AV> gtab(pool, pool_slots, pool_off[t]);
+        // the slice's edges inside the community go out once
+        nself = warp_sum(nself);
+        selfw = warp_sum(selfw);
+        if (lane == 0 && nself) gtab.template add<false>(glog, c, selfw);
+        __syncthreads();  // the task is combined
+        AV v[AGG_SUB / 32];
+        uint32_t key[AGG_SUB / 32];
+#pragma unroll
+        for (uint32_t u = 0; u < AGG_SUB / 32; u++) {
+            const uint32_t x = u * 32 + lane;
+            key[u] = EMPTY;
+            if (x >= nclaimed) continue;
+            const uint32_t s = claimed[x];
+            key[u] = tab.get(s, v[u]);
+            tab.clear(s);
+        }
+        __syncthreads();  // the shared table is empty
+#pragma unroll
+        for (uint32_t u = 0; u < AGG_SUB / 32; u++)
+            if (key[u] != EMPTY) gtab.template add<false>(glog, key[u], v[u]);
     }
 }
 
-// Extraction uses the insert's task split: task k of a community emits its
-// occupied entries [k * AGG_CHUNK, (k+1) * AGG_CHUNK) (a community has at
-// most one distinct neighbour community per edge).
+// Extraction uses the insert's task split: task k of a community's n tasks
+// emits the slots [cap k / n, cap (k + 1) / n) of its table.
 template <typename AV>
 __global__ void __launch_bounds__(256) k_agg_large_extract(AggArgs a, const uint32_t *__restrict__ list,
                                                            uint32_t count, const uint64_t *__restrict__ tasks,
                                                            const uint32_t *__restrict__ task_c,
                                                            const uint64_t *__restrict__ pool_off,
-                                                           const uint32_t *__restrict__ pool_keys,
-                                                           const AV *__restrict__ pool_vals,
-                                                           const uint32_t *__restrict__ pool_occ,
-                                                           const uint32_t *__restrict__ occ_n) {
+                                                           uint64_t pool_slots, unsigned char *pool) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t total = tasks[count];
     for (uint64_t task = blockIdx.x; task < total; task += gridDim.x) {
-        uint32_t t = task_c[task];
-        uint32_t c = list[t];
-        const uint32_t *keys = pool_keys + pool_off[t];
-        const AV *vals = pool_vals + pool_off[t];
-        const uint32_t *occ = pool_occ + pool_off[t];
-        uint64_t k0 = (task - tasks[t]) * AGG_CHUNK;
-        uint64_t k1 = min(k0 + AGG_CHUNK, (uint64_t)occ_n[t]);
-        // warp-uniform trip counts so emit_slot's ballots see full warps
-        for (uint64_t kb = k0 + wid * 32; kb < k1; kb += blockDim.x) {
-            uint64_t k = kb + lane;
-            bool valid = k < k1;
-            uint32_t slot = valid ? occ[k] : 0;
-            emit_slot(a, c, valid ? keys[slot] : EMPTY, valid ? Acc<AV>::val(vals[slot], a.xlsb) : 0.0, valid,
-                      a.rowlen + c);
+        const uint32_t t = task_c[task], c = list[t];
+        const AggTable<AV> tab(pool, pool_slots, pool_off[t]);
+        const uint64_t n = tasks[t + 1] - tasks[t], k = task - tasks[t], cap = pool_off[t + 1] - pool_off[t];
+        const uint64_t s1 = cap * (k + 1) / n;
+        // warp-uniform trip counts so emit_slots' ballots see full warps
+        for (uint64_t sb = cap * k / n + wid * 32; sb < s1; sb += blockDim.x * 4ull) {
+            uint32_t key[4];
+            AV v[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const uint64_t s = sb + (uint64_t)u * blockDim.x + lane;
+                key[u] = s < s1 ? tab.get(s, v[u]) : EMPTY;
+            }
+            emit_slots<4>(a, c, key, v, a.rowlen + c);
         }
     }
 }
@@ -714,21 +837,19 @@ template <typename WT, typename AV>
 static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &ic, const unsigned long long *cdeg,
                          const uint32_t *cverts, uint32_t k, uint32_t n, cudaStream_t s) {
     auto cnt_of = [&](int c) { return ic.start[c + 1] - ic.start[c]; };
-    if (cnt_of(ACLS_W)) {
-        constexpr size_t smem = (size_t)AGG_WWARPS * AGG_WCAP * (sizeof(uint32_t) + sizeof(AV));
-        static bool wattr = false;
-        if (!wattr) {
-            GSP_CUDA(cudaFuncSetAttribute(k_agg_merge_warp<WT, AV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
-            wattr = true;
-        }
-        k_agg_merge_warp<WT, AV><<<grid_for((uint64_t)cnt_of(ACLS_W) * 32, AGG_WWARPS * 32, sms(4)), AGG_WWARPS * 32,
-                               smem, s>>>(a, ic.list + ic.start[ACLS_W], cnt_of(ACLS_W));
+    auto warp_class = [&](auto fn, int cls, int cap, int warps, unsigned per_sm) {
+        if (!cnt_of(cls)) return;
+        const size_t smem = (size_t)warps * cap * AggTable<AV>::slot_bytes;
+        GSP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        fn<<<grid_for((uint64_t)cnt_of(cls) * 32, warps * 32, sms(per_sm)), warps * 32, smem, s>>>(
+            a, ic.list + ic.start[cls], cnt_of(cls));
         GSP_CHECK_LAUNCH();
-    }
+    };
+    warp_class(k_agg_merge_warp<AGG_SCAP, AGG_SWARPS, WT, AV>, ACLS_S, AGG_SCAP, AGG_SWARPS, 32);
+    warp_class(k_agg_merge_warp<AGG_WCAP, AGG_WWARPS, WT, AV>, ACLS_W, AGG_WCAP, AGG_WWARPS, 8);
     if (cnt_of(ACLS_B)) {
-        constexpr size_t smem = (size_t)AGG_BCAP * (sizeof(uint32_t) + sizeof(AV) + sizeof(uint16_t)) +
-                                (size_t)AGG_BMEM * sizeof(uint64_t) + (size_t)(AGG_BMEM + 1) * sizeof(uint32_t);
+        constexpr size_t smem = (size_t)AGG_BCAP * AggTable<AV>::slot_bytes + (size_t)AGG_BMEM * sizeof(uint64_t) +
+                                (size_t)(AGG_BMEM + 1) * sizeof(uint32_t);
         static bool attr = false;
         if (!attr) {
             GSP_CUDA(cudaFuncSetAttribute(k_agg_merge_block<WT, AV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -749,13 +870,16 @@ static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &i
         uint64_t slots;
         GSP_CUDA(cudaMemcpyAsync(&slots, poff + nl, sizeof(slots), cudaMemcpyDeviceToHost, s));
         GSP_CUDA(cudaStreamSynchronize(s));
-        uint32_t *pk = arena().get<uint32_t>(slots);
-        AV *pv = arena().get<AV>(slots);
-        uint32_t *po = arena().get<uint32_t>(slots);
-        uint32_t *on = arena().get<uint32_t>(nl);
-        GSP_CUDA(cudaMemsetAsync(pk, 0xFF, sizeof(uint32_t) * slots, s));
-        GSP_CUDA(cudaMemsetAsync(pv, 0, sizeof(AV) * slots, s));
-        GSP_CUDA(cudaMemsetAsync(on, 0, sizeof(uint32_t) * nl, s));
+        // packed slots are free with all bits set; otherwise the values (0)
+        // come first, the keys behind them
+        constexpr bool packed = sizeof(AV) == sizeof(uint32_t);
+        unsigned char *pool = static_cast<unsigned char *>(arena().alloc(AggTable<AV>::slot_bytes * slots));
+        if (packed) {
+            GSP_CUDA(cudaMemsetAsync(pool, 0xFF, AggTable<AV>::slot_bytes * slots, s));
+        } else {
+            GSP_CUDA(cudaMemsetAsync(pool, 0, sizeof(AV) * slots, s));
+            GSP_CUDA(cudaMemsetAsync(pool + sizeof(AV) * slots, 0xFF, sizeof(uint32_t) * slots, s));
+        }
         uint64_t *medge = arena().get<uint64_t>((size_t)n + 1);
         uint64_t *mdeg = arena().get<uint64_t>(n);
         k_member_deg<<<grid_for(n, 256), 256, 0, s>>>(g.off, cverts, n, mdeg);
@@ -775,18 +899,18 @@ static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &i
         k_agg_warp_starts<<<grid_for(task_bound * AGG_TASK_WARPS, 256, sms(16)), 256, 0, s>>>(
             a, llist, tasks, nl, task_c, medge, wstart);
         GSP_CHECK_LAUNCH();
-        constexpr size_t lsmem = (sizeof(uint32_t) + sizeof(AV) + sizeof(uint16_t)) << AGG_SLOG;
+        constexpr size_t lsmem = (AggTable<AV>::slot_bytes << AGG_SLOG) + AGG_CHUNK * sizeof(uint16_t);
         static bool lattr = false;
         if (!lattr) {
             GSP_CUDA(cudaFuncSetAttribute(k_agg_large_insert<WT, AV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)lsmem));
             lattr = true;
         }
-        const unsigned lgrid = resident_grid((const void *)k_agg_large_insert<WT, AV>, AGG_TASK_WARPS * 32, lsmem, 4);
+        const unsigned lgrid = resident_grid((const void *)k_agg_large_insert<WT, AV>, AGG_TASK_WARPS * 32, lsmem, 8);
         k_agg_large_insert<WT, AV><<<lgrid, AGG_TASK_WARPS * 32, lsmem, s>>>(a, llist, nl, tasks, task_c, wstart, medge,
-                                                                          poff, pk, pv, po, on);
+                                                                          poff, slots, pool);
         GSP_CHECK_LAUNCH();
-        k_agg_large_extract<AV><<<sms(4), 256, 0, s>>>(a, llist, nl, tasks, task_c, poff, pk, pv, po, on);
+        k_agg_large_extract<AV><<<sms(8), 256, 0, s>>>(a, llist, nl, tasks, task_c, poff, slots, pool);
         GSP_CHECK_LAUNCH();
     }
 
@@ -794,7 +918,7 @@ static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &i
 
 template <typename WT>
 static uint64_t aggregate_impl(const DevGraph &g, const uint32_t *Cd, uint32_t k, uint64_t *out_off,
-                               uint32_t *out_tgt, double *out_w, bool sorted, int *lsb_cache, cudaStream_t s) {
+                               uint32_t *out_tgt, double *out_w, bool sorted, const WeightUnit *known, cudaStream_t s) {
     size_t mk = arena().mark();
     uint32_t n = g.n;
     uint32_t *cnt = arena().get<uint32_t>(k);
@@ -821,12 +945,13 @@ static uint64_t aggregate_impl(const DevGraph &g, const uint32_t *Cd, uint32_t k
     AggArgs a{g.off, g.tgt, g.w, Cd, coff, cverts, cdeg, yoff, htgt, hw, rowlen, k, 0};
     // exact fixed-point table values when the weights allow it (same result,
     // native shared-memory integer atomics instead of float64 ones)
-    int lsb = lsb_cache ? *lsb_cache : INT_MAX;
-    if (lsb == INT_MAX) lsb = exact_lsb(g, s);
-    if (lsb_cache) *lsb_cache = lsb;
+    WeightUnit unit = known ? *known : exact_unit(g, s);
+    const int lsb = unit.lsb;
+    const bool units32 = unit.fits32;
     if (lsb != INT_MIN) {
         a.xlsb = lsb;
-        merge_tables<WT, unsigned long long>(g, a, ic, cdeg, cverts, k, n, s);
+        if (units32) merge_tables<WT, uint32_t>(g, a, ic, cdeg, cverts, k, n, s);
+        else merge_tables<WT, unsigned long long>(g, a, ic, cdeg, cverts, k, n, s);
     } else {
         merge_tables<WT, double>(g, a, ic, cdeg, cverts, k, n, s);
     }
@@ -900,9 +1025,9 @@ static uint64_t aggregate_impl(const DevGraph &g, const uint32_t *Cd, uint32_t k
 }
 
 uint64_t aggregate(const DevGraph &g, const uint32_t *Cd, uint32_t k, uint64_t *out_off, uint32_t *out_tgt,
-                   double *out_w, cudaStream_t s, bool sorted, int *lsb_cache) {
-    if (g.wt == GSP_W_F64) return aggregate_impl<double>(g, Cd, k, out_off, out_tgt, out_w, sorted, lsb_cache, s);
-    return aggregate_impl<float>(g, Cd, k, out_off, out_tgt, out_w, sorted, lsb_cache, s);
+                   double *out_w, cudaStream_t s, bool sorted, const WeightUnit *known) {
+    if (g.wt == GSP_W_F64) return aggregate_impl<double>(g, Cd, k, out_off, out_tgt, out_w, sorted, known, s);
+    return aggregate_impl<float>(g, Cd, k, out_off, out_tgt, out_w, sorted, known, s);
 }
 
 }  // namespace gsp

@@ -435,7 +435,8 @@ void louvain_batched_run(const DevGraph &g0, uint32_t G, const uint64_t *h_gvo0,
     int pb = 0, passes = 0;
     // exact integer unit of the input weights (INT_MIN: float64 sums), valid
     // for every pass: aggregated weights are sums of input weights
-    int lsb_cache = exact_lsb(g0, s);
+    const WeightUnit unit = exact_unit(g0, s);
+    const int lsb_cache = unit.lsb;
     mb.lsb = lsb_cache;
     uint32_t remaining = G;
     for (int lp = 0; lp < o.max_passes && remaining; lp++) {
@@ -579,7 +580,7 @@ void louvain_batched_run(const DevGraph &g0, uint32_t G, const uint64_t *h_gvo0,
         nxt.tgt = gtgt[pb];
         nxt.w = gw[pb];
         nxt.wt = GSP_W_F64;
-        nxt.nnz = aggregate(cur, Cd, k, goff[pb], gtgt[pb], gw[pb], s, /*sorted=*/false, &lsb_cache);
+        nxt.nnz = aggregate(cur, Cd, k, goff[pb], gtgt[pb], gw[pb], s, /*sorted=*/false, &unit);
         pb ^= 1;
         cur = nxt;
         tau = tau / o.tolerance_drop;

@@ -718,7 +718,8 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
     int pb = 0;
     // exact integer unit of the input weights (INT_MIN: float64 sums), valid
     // for every pass: aggregated weights are sums of input weights
-    int lsb_cache = exact_lsb(g0, s);
+    const WeightUnit unit = exact_unit(g0, s);
+    const int lsb_cache = unit.lsb;
     mb.lsb = lsb_cache;
     for (int lp = 0; lp < o.max_passes; lp++) {
         const uint32_t nv = cur.n;
@@ -804,7 +805,7 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
         nxt.tgt = gtgt[pb];
         nxt.w = gw[pb];
         nxt.wt = GSP_W_F64;
-        nxt.nnz = aggregate(cur, A, k, goff[pb], gtgt[pb], gw[pb], s, /*sorted=*/false, &lsb_cache);
+        nxt.nnz = aggregate(cur, A, k, goff[pb], gtgt[pb], gw[pb], s, /*sorted=*/false, &unit);
         pb ^= 1;
         cur = nxt;
         tau = tau / o.tolerance_drop;

@@ -264,14 +264,23 @@ void split_labels(const DevGraph &g, const Classes &cl, const uint32_t *C, int m
 // Renumber: C_dense[v] = rank of C[v] among the distinct ids; returns k.
 uint32_t renumber(uint32_t n, const uint32_t *C, uint32_t *C_dense, cudaStream_t s);
 
+// Exact unit of a graph's weights (exact_unit): every weight is a multiple of
+// 2^lsb and the total is below 2^52 units (lsb INT_MIN: there is no such unit,
+// sums stay float64); fits32: the total is below 2^32 units.
+struct WeightUnit {
+    int lsb;
+    bool fits32;
+};
+WeightUnit exact_unit(const DevGraph &g, cudaStream_t s);
+
 // Aggregation (Algorithm 5) into out (offsets k+1, targets/weights nnz); returns nnz''.
 // sorted: rows in increasing target order (the canonical form); otherwise
-// each row's entries come in table order.  lsb_cache (optional) carries the
-// exponent of the exact fixed-point unit of the weights between the passes
-// of one run (INT_MAX: not known yet; the weights of every aggregated graph
-// are sums of the input weights, so the input's unit and bound hold for all).
+// each row's entries come in table order.  known (optional) carries the
+// exact fixed-point unit of the weights between the passes
+// of one run (the weights of every aggregated graph are sums of the input
+// weights, so the input's unit and bounds hold for all).
 uint64_t aggregate(const DevGraph &g, const uint32_t *Cd, uint32_t k, uint64_t *out_off, uint32_t *out_tgt,
-                   double *out_w, cudaStream_t s, bool sorted = true, int *lsb_cache = nullptr);
+                   double *out_w, cudaStream_t s, bool sorted = true, const WeightUnit *known = nullptr);
 
 // Exponent lsb such that every weight of g is a multiple of 2^lsb and the
 // total weight is below 2^52 * 2^lsb, or INT_MIN (then sums stay float64).
@@ -372,25 +381,7 @@ __device__ __forceinline__ int ht_add(uint32_t *keys, V *vals, int logcap, uint3
     return -1;
 }
 
-// Global-table insert that claims with atomicCAS first (one round trip when
-// the home slot is free or already holds c); reports the slot used.
-template <typename V>
-__device__ __forceinline__ int ht_add_slot_cas(uint32_t *keys, V *vals, int logcap, uint32_t c, V w, uint32_t *slot) {
-    uint32_t mask = (1u << logcap) - 1u;
-    uint32_t h = logcap ? (hash32(c) >> (32 - logcap)) : 0u;
-    for (uint32_t probe = 0; probe <= mask; probe++) {
-        uint32_t old = atomicCAS(&keys[h], EMPTY, c);
-        if (old == EMPTY || old == c) {
-            atomicAdd(&vals[h], w);
-            *slot = h;
-            return old == EMPTY;
-        }
-        h = (h + 1) & mask;
-    }
-    return -1;
-}
-
-// As ht_add, also reporting the slot used (for occupied-slot lists).
+// As ht_add, also reporting the slot used.
 template <typename V>
 __device__ __forceinline__ int ht_add_slot(uint32_t *keys, V *vals, int logcap, uint32_t c, V w, uint32_t *slot) {
     uint32_t mask = (1u << logcap) - 1u;
@@ -406,48 +397,6 @@ __device__ __forceinline__ int ht_add_slot(uint32_t *keys, V *vals, int logcap, 
         h = (h + 1) & mask;
     }
     return -1;
-}
-
-// Combine-then-publish: the block's shared table (2^slog slots, whose
-// occupied slots are listed in socc[0..*s_nocc)) is merged into a global
-// table (2^glog slots); keys new to the global table append their slot to
-// occ (count in *occ_n).  The shared table is left empty.  Every thread of
-// the block must call this.
-constexpr uint32_t PUBLISH_MAX = 2048;  // most distinct keys one block publishes at once
-
-template <typename V>
-__device__ void publish_block_table(uint32_t *skeys, V *svals, uint16_t *socc, uint32_t *s_nocc, uint32_t *gkeys,
-                                    V *gvals, int glog, uint32_t *occ, uint32_t *occ_n) {
-    __shared__ uint32_t s_newslot[PUBLISH_MAX];
-    __shared__ uint32_t s_new, s_base;
-    __syncthreads();
-    if (threadIdx.x == 0) s_new = 0;
-    __syncthreads();
-    uint32_t n = min(*s_nocc, PUBLISH_MAX);
-    for (uint32_t t = threadIdx.x; t < n; t += blockDim.x) {
-        uint32_t s = socc[t];
-        uint32_t slot;
-        if (ht_add_slot_cas<V>(gkeys, gvals, glog, skeys[s], svals[s], &slot) == 1)
-            s_newslot[atomicAdd(&s_new, 1u)] = slot;
-        skeys[s] = EMPTY;
-        svals[s] = V(0);
-    }
-    __syncthreads();
-    // one reservation per block in the global occupied list
-    if (threadIdx.x == 0) s_base = s_new ? atomicAdd(occ_n, s_new) : 0;
-    __syncthreads();
-    for (uint32_t t = threadIdx.x; t < s_new; t += blockDim.x) occ[s_base + t] = s_newslot[t];
-    __syncthreads();
-    if (threadIdx.x == 0) *s_nocc = 0;
-    __syncthreads();
-}
-
-// Insert into a shared table, listing slots new to it in socc.
-template <typename V>
-__device__ __forceinline__ void smem_add(uint32_t *skeys, V *svals, int slog, uint16_t *socc, uint32_t *s_nocc,
-                                         uint32_t c, V w) {
-    uint32_t slot;
-    if (ht_add_slot<V>(skeys, svals, slog, c, w, &slot) == 1) socc[atomicAdd(s_nocc, 1u)] = (uint16_t)slot;
 }
 
 // Exact sums of edge weights.  They are accumulated either as float64
@@ -477,6 +426,10 @@ template <> struct Acc<double> {
     template <typename WT> __device__ static double of(WT x, int) { return (double)x; }
     __device__ static double val(double v, int) { return v; }
 };
+template <> struct Acc<uint32_t> {  // totals below 2^32 units
+    template <typename WT> __device__ static uint32_t of(WT x, int lsb) { return (uint32_t)units_of(x, lsb); }
+    __device__ static double val(uint32_t v, int lsb);
+};
 template <> struct Acc<unsigned long long> {
     template <typename WT> __device__ static unsigned long long of(WT x, int lsb) { return units_of(x, lsb); }
     // v < 2^52: the conversion is exact, and so is the power-of-two scaling
@@ -487,6 +440,10 @@ template <> struct Acc<unsigned long long> {
         return __longlong_as_double(__double_as_longlong(d) + ((long long)lsb << 52));
     }
 };
+
+__device__ __forceinline__ double Acc<uint32_t>::val(uint32_t v, int lsb) {
+    return Acc<unsigned long long>::val(v, lsb);
+}
 
 // Exponent of the lowest set bit of a positive finite weight (INT_MIN for a
 // value that is not, INT_MAX for zero).

@@ -42,8 +42,9 @@ __global__ void k_weight_range(const WT *__restrict__ w, uint64_t nnz, int *minl
 // estimated with float32 partial sums (relative error far below the factor 2
 // of margin kept under 2^53).
 template <typename WT>
-static int exact_lsb_t(const DevGraph &g, cudaStream_t s) {
-    if (!g.nnz || !g.w) return INT_MIN;
+static WeightUnit exact_unit_t(const DevGraph &g, cudaStream_t s) {
+    const WeightUnit none{INT_MIN, false};
+    if (!g.nnz || !g.w) return none;
     size_t mk = arena().mark();
     int *dlo = arena().get<int>(1);
     double *dsum = arena().get<double>(1);
@@ -58,15 +59,16 @@ static int exact_lsb_t(const DevGraph &g, cudaStream_t s) {
     GSP_CUDA(cudaMemcpyAsync(&sum, dsum, sizeof(double), cudaMemcpyDeviceToHost, s));
     GSP_CUDA(cudaStreamSynchronize(s));
     arena().release(mk);
-    if (lo < -1000 || lo > 1000) return INT_MIN;
-    // the sum is an estimate: keep a factor 2 of margin below 2^53
-    if (!(sum > 0.0) || !(sum < std::ldexp(1.0, 52 + lo))) return INT_MIN;
-    return lo;
+    if (lo < -1000 || lo > 1000) return none;
+    // the sum is an estimate: keep a factor 2 of margin below 2^53 (and 2^32)
+    if (!(sum > 0.0) || !(sum < std::ldexp(1.0, 52 + lo))) return none;
+    return {lo, sum < std::ldexp(1.0, 31 + lo)};
 }
 
-int exact_lsb(const DevGraph &g, cudaStream_t s) {
-    return g.wt == GSP_W_F64 ? exact_lsb_t<double>(g, s) : exact_lsb_t<float>(g, s);
+WeightUnit exact_unit(const DevGraph &g, cudaStream_t s) {
+    return g.wt == GSP_W_F64 ? exact_unit_t<double>(g, s) : exact_unit_t<float>(g, s);
 }
+int exact_lsb(const DevGraph &g, cudaStream_t s) { return exact_unit(g, s).lsb; }
 
 
 __global__ void k_iota(uint32_t *p, uint32_t n) {
