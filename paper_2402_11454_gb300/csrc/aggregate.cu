@@ -839,8 +839,7 @@ static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &i
     auto cnt_of = [&](int c) { return ic.start[c + 1] - ic.start[c]; };
     auto warp_class = [&](auto fn, int cls, int cap, int warps, unsigned per_sm) {
         if (!cnt_of(cls)) return;
-        const size_t smem = (size_t)warps * cap * AggTable<AV>::slot_bytes;
-        GSP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const size_t smem = (size_t)warps * cap * AggTable<AV>::slot_bytes;  // at most 48 KB: no opt-in
         fn<<<grid_for((uint64_t)cnt_of(cls) * 32, warps * 32, sms(per_sm)), warps * 32, smem, s>>>(
             a, ic.list + ic.start[cls], cnt_of(cls));
         GSP_CHECK_LAUNCH();

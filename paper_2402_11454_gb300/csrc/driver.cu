@@ -383,12 +383,14 @@ int wave_repeats_at(const MoveBuffers &mb, int it) { return (it == 0 && mb.repea
 void sweep_launches(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool sync, bool fp64, bool rule,
                     bool pruned, int it, int max_it, const uint32_t *wave_n, bool reset_ctr, cudaStream_t s) {
     if (reset_ctr) GSP_CUDA(cudaMemsetAsync(mb.ctr, 0, sizeof(MoveCounters), s));
-    const int R = wave_repeats_at(mb, it);
+    const int R = std::min(wave_repeats_at(mb, it), MAX_REPEATS);
+    // a move counter for each run of a wave, cleared together
+    if (sync) GSP_CUDA(cudaMemsetAsync(mb.mv_cnts, 0, sizeof(uint32_t) * cl.W * R, s));
     for (int wv = 0; wv < cl.W; wv++) {
         if (!wave_n[wv]) continue;
         for (int r = 0; r < R; r++) {
             mb.cur_repeat = r;
-            if (sync) GSP_CUDA(cudaMemsetAsync(mb.mv_cnt, 0, sizeof(uint32_t), s));
+            mb.mv_cnt = mb.mv_cnts + wv * R + r;
             move_wave(g, cl, mb, wv, sync, fp64, rule, pruned, it, max_it, s);
             if (sync) apply_moves(g, mb, wave_n[wv], s);
         }
@@ -573,8 +575,8 @@ void alloc_move_state(MoveBuffers &mb, uint32_t n) {
     mb.mark = arena().get<uint8_t>(n);
     mb.mv_vtx = arena().get<uint32_t>(n);
     mb.mv_cmt = arena().get<uint32_t>(n);
-    mb.mv_cnt = arena().get<uint32_t>(1);
     mb.mv_cnts = arena().get<uint32_t>(MAX_WAVES * MAX_REPEATS);
+    mb.mv_cnt = mb.mv_cnts;
     mb.bar = arena().get<GridBar>(1);
     mb.big = arena().get<uint32_t>(n);
     mb.nbig = arena().get<uint32_t>(1);

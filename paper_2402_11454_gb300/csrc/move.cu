@@ -958,19 +958,46 @@ __device__ __forceinline__ void flush_delta(const uint32_t *keys, const double *
     if (dn[t] != 0) atomicAdd(size + c, (uint32_t)dn[t]);
 }
 
+// act |= mark, mark = 0 (16 bytes per thread step) by blocks lb of nb.
+__device__ __forceinline__ void merge_marks(uint8_t *act, uint8_t *mark, uint32_t n, uint32_t lb, uint32_t nb) {
+    uint32_t n16 = n / 16;
+    uint4 *a4 = reinterpret_cast<uint4 *>(act);
+    uint4 *m4 = reinterpret_cast<uint4 *>(mark);
+    for (uint32_t t = lb * blockDim.x + threadIdx.x; t < n16; t += nb * blockDim.x) {
+        uint4 mk = m4[t];
+        if (mk.x | mk.y | mk.z | mk.w) {
+            uint4 ac = a4[t];
+            ac.x |= mk.x; ac.y |= mk.y; ac.z |= mk.z; ac.w |= mk.w;
+            a4[t] = ac;
+            m4[t] = make_uint4(0, 0, 0, 0);
+        }
+    }
+    for (uint32_t v = n16 * 16 + lb * blockDim.x + threadIdx.x; v < n; v += nb * blockDim.x) {
+        if (mark[v]) { act[v] = 1; mark[v] = 0; }
+    }
+}
+
+// The first `appliers` blocks apply the moves, the others merge the marks (two
+// launches less the gap between them on a chain of launches per wave).
 __global__ void __launch_bounds__(256) k_apply_moves(const uint32_t *__restrict__ mv_vtx,
                                                      const uint32_t *__restrict__ mv_cmt,
                                                      const uint32_t *__restrict__ mv_cnt, const double *__restrict__ K,
                                                      uint32_t *C, double *Sig, uint32_t *size, int lsb, uint32_t *left,
-                                                     int *left_it, const int *iteration_dev) {
+                                                     int *left_it, const int *iteration_dev, unsigned appliers,
+                                                     uint8_t *act, uint8_t *mark, uint32_t n) {
+    if (blockIdx.x >= appliers) {
+        merge_marks(act, mark, n, blockIdx.x - appliers, gridDim.x - appliers);
+        return;
+    }
+    const uint32_t cnt = *mv_cnt;
+    if (blockIdx.x * blockDim.x >= cnt) return;
     __shared__ uint32_t skeys[1 << APPLY_SLOG];
     __shared__ double sds[1 << APPLY_SLOG];
     __shared__ int sdn[1 << APPLY_SLOG];
     for (int t = threadIdx.x; t < (1 << APPLY_SLOG); t += blockDim.x) { skeys[t] = EMPTY; sds[t] = 0.0; sdn[t] = 0; }
     __syncthreads();
-    uint32_t cnt = *mv_cnt;
     const int iteration = *iteration_dev;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x) {
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += appliers * blockDim.x) {
         uint32_t i = mv_vtx[t], c = mv_cmt[t];
         uint32_t d = C[i];
         double Ki = K[i];
@@ -983,25 +1010,6 @@ __global__ void __launch_bounds__(256) k_apply_moves(const uint32_t *__restrict_
     }
     __syncthreads();
     for (int t = threadIdx.x; t < (1 << APPLY_SLOG); t += blockDim.x) flush_delta(skeys, sds, sdn, t, Sig, size, lsb);
-}
-
-// act |= mark, mark = 0 (16 bytes per thread step).
-__global__ void k_merge_marks(uint8_t *act, uint8_t *mark, uint32_t n) {
-    uint32_t n16 = n / 16;
-    uint4 *a4 = reinterpret_cast<uint4 *>(act);
-    uint4 *m4 = reinterpret_cast<uint4 *>(mark);
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n16; t += gridDim.x * blockDim.x) {
-        uint4 mk = m4[t];
-        if (mk.x | mk.y | mk.z | mk.w) {
-            uint4 ac = a4[t];
-            ac.x |= mk.x; ac.y |= mk.y; ac.z |= mk.z; ac.w |= mk.w;
-            a4[t] = ac;
-            m4[t] = make_uint4(0, 0, 0, 0);
-        }
-    }
-    for (uint32_t v = n16 * 16 + blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        if (mark[v]) { act[v] = 1; mark[v] = 0; }
-    }
 }
 
 // Re-mark the neighbours of the big movers: block column x takes movers
@@ -1177,9 +1185,8 @@ __global__ void __launch_bounds__(256) k_sweep_persistent(MoveArgs a, const uint
 //     the barrier: Sigma and size by atomics that nobody waits for, marks
 //     straight into the flags (no vertex is deciding then).
 // A cluster has at most 16 of the 152 SMs, so the host takes this path only
-// while a wave's work fits them (move_level).  Measured (611 vertices, 153
-// wave runs): 5.7 us a run against 21 as launches, of which the visit takes
-// 2.2, each barrier with its release and acquire 0.7-1.3.
+// while a wave's work fits them (move_level), with as few CTAs as give each
+// task a warp.  Measured (611 vertices, 153 wave runs, one CTA): 5.4 us a run.
 //
 // Batches: per-graph gains and stopping as in the host loop (a graph whose
 // gain of the sweep is <= tau stops, and its vertices become inactive).
@@ -1208,11 +1215,16 @@ struct LevelArgs {
     uint32_t *nlive;               // 3 counts of the graphs still iterating, zero at start
 };
 
-__device__ __forceinline__ void cluster_arrive() {
+// Barrier of all CTAs, split into arrival and wait; alone, a CTA's own barrier
+// at the wait (a cluster barrier's release and acquire cost 0.7-1.3 us).
+__device__ __forceinline__ void level_arrive(bool alone) {
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (!alone) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void level_wait(bool alone) {
+    if (alone) __syncthreads();
+    else asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 struct LevelMover {
     uint64_t b;
@@ -1324,6 +1336,7 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
     __shared__ double s_red[32];
     __shared__ uint32_t s_bv[LEVEL_BMOVERS], s_bc[LEVEL_BMOVERS], s_bn;
     const uint32_t lb = blockIdx.x, nb = gridDim.x;
+    const bool alone = nb == 1;
     const uint32_t tid = lb * LEVEL_THREADS + threadIdx.x, nt = nb * LEVEL_THREADS;
     const uint32_t wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // warp w of CTA b is number w * nb + b, so that few tasks spread over the CTAs
@@ -1397,14 +1410,14 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
                     level_fetch(a, v.list, sm.start, v.W, wv, x, m0, inv0, t);
                     level_visit<WT, F64>(a, t, it, ws, mv, nmv, lc);
                 }
-                cluster_arrive();  // every vertex of the wave has decided
+                level_arrive(alone);  // every vertex of the wave has decided
                 __syncwarp();      // the warp's movers are visible to its lanes
                 if (r + 1 == rep) {
                     const int nx = after < v.W ? after : wave0;
                     if (nx != fetched) level_fetch(a, v.list, sm.start, v.W, nx, wb, m0, inv0, t0);
                     fetched = nx;
                 }
-                cluster_wait();
+                level_wait(alone);
                 for (uint32_t x = lane; x < nmv; x += 32) {
                     const LevelMover q = mv[x];
                     level_apply(a, q.i, q.c, q.d, q.K, it);
@@ -1439,16 +1452,16 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
                     }
                     __syncthreads();
                 }
-                cluster_arrive();  // the wave's moves and marks are in place
-                cluster_wait();
+                level_arrive(alone);  // the wave's moves and marks are in place
+                level_wait(alone);
             }
             wv = after;
         }
         // the sweep's gain; then every CTA takes the same decision
         const double dq = block_sum<double>(lc.dq, s_red);
         if (threadIdx.x == 0 && dq != 0.0) atomicAdd(v.dq + sum, dq);
-        cluster_arrive();
-        cluster_wait();
+        level_arrive(alone);
+        level_wait(alone);
         if (!v.G) {
             if (it + 1 >= v.max_it || __ldcg(v.dq + sum) <= v.tau) break;
             continue;
@@ -1463,13 +1476,13 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
         }
         alive = (uint32_t)__syncthreads_count(alive != 0);
         if (threadIdx.x == 0 && alive) atomicAdd(v.nlive + sum, alive);
-        cluster_arrive();
-        cluster_wait();
+        level_arrive(alone);
+        level_wait(alone);
         if (it + 1 >= v.max_it || !__ldcg(v.nlive + sum)) break;
         for (uint32_t i = tid; i < v.n; i += nt)
             if (!ldcg(v.live + a.gid[i])) a.act[i] = 0;
-        cluster_arrive();
-        cluster_wait();
+        level_arrive(alone);
+        level_wait(alone);
     }
     lc.dq = 0.0;  // reported per sweep
     flush_counters(lc, a.ctr);
@@ -2086,7 +2099,7 @@ bool sweep_persistent(const DevGraph &g, const Classes &cl, MoveBuffers &mb, boo
 }
 
 template <typename WT, bool F64>
-static bool launch_level(const MoveArgs &a, const LevelArgs &v, int ctas_needed, cudaStream_t s) {
+static bool launch_level(const MoveArgs &a, const LevelArgs &v, int ctas_needed, int ctas_wanted, cudaStream_t s) {
     constexpr size_t smem = sizeof(LevelSmem<F64>);
     static int ctas[64] = {0};  // CTAs of the cluster, per device (-1: cannot run)
     int dev = 0;
@@ -2116,30 +2129,37 @@ static bool launch_level(const MoveArgs &a, const LevelArgs &v, int ctas_needed,
         ctas[dev] = found;
     }
     if (ctas[dev] < ctas_needed) return false;
-    at[0].val.clusterDim.x = ctas[dev];
-    cfg.gridDim = dim3(ctas[dev]);
+    const int c = std::min(ctas[dev], ctas_wanted);
+    at[0].val.clusterDim.x = c;
+    cfg.gridDim = dim3(c);
     GSP_CUDA(cudaLaunchKernelEx(&cfg, fn, a, v));
     count_launch();
     return true;
 }
 
 // Most stored entries of a graph that one cluster moves.  Measured on GB300,
-// whole local-moving phase (gsp_local_move), launches against cluster:
-// planted 2 K vertices / 30 K entries 3.36 against 1.07 ms, 10 K / 151 K 4.02
-// against 1.30, 20 K / 995 K 2.54 against 1.94, 60 K / 906 K 4.44 against 3.68,
-// 300^2 grid 2.84 against 1.48; R-MAT 3 K / 75 K 3.96 against 1.90, 60 K / 879 K
-// 5.03 against 4.39, 12 K / 1.32 M 5.70 against 5.98.  The float64 mode's
-// divisions need more SMs sooner: planted 10 K / 151 K 5.16 against 3.15, R-MAT
-// 9 K / 252 K 10.7 against 7.4, planted 20 K / 542 K 4.30 against 5.46.
-constexpr uint64_t LEVEL_MAX_EDGES = 1u << 20, LEVEL_MAX_EDGES_F64 = 1u << 18;
+// whole local-moving phase (gsp_local_move), launches against cluster, ms:
+// planted 2 K vertices / 30 K entries 2.08 and 1.17, 10 K / 151 K 2.45 and 1.40,
+// 10 K / 496 K 1.49 and 1.27, 20 K / 542 K 2.03 and 1.96, 30 K / 863 K 1.85 and
+// 2.31; 300^2 grid 1.80 and 1.46; R-MAT 3 K / 75 K 2.55 and 1.69, 30 K / 431 K
+// 2.64 and 2.35, 12 K / 602 K 3.36 and 3.80.  The float64 mode's divisions need
+// more SMs sooner: planted 10 K / 151 K 3.16 and 2.74, 200^2 grid / 151 K 1.96 and
+// 1.82, R-MAT 9 K / 252 K 5.50 and 6.43; dense graphs of few vertices gain a
+// little longer (540 vertices / 254 K entries 2.47 and 1.72).
+constexpr uint64_t LEVEL_MAX_EDGES = 1u << 19, LEVEL_MAX_EDGES_F64 = 160000, LEVEL_MAX_EDGES_F64_DENSE = 1u << 18;
+constexpr uint32_t LEVEL_DENSE_VERTICES = 2048;
 
 bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64, bool rule, double tau, int max_it,
                 LevelResult &out, uint32_t G, uint8_t *live, int *li, cudaStream_t s) {
-    if (g.nnz > (fp64 ? LEVEL_MAX_EDGES_F64 : LEVEL_MAX_EDGES) || mb.feat_kept || mb.choice || !cl.dstart) return false;
+    const uint64_t most = !fp64                              ? LEVEL_MAX_EDGES
+                          : g.n <= LEVEL_DENSE_VERTICES ? LEVEL_MAX_EDGES_F64_DENSE
+                                                        : LEVEL_MAX_EDGES_F64;
+    if (g.nnz > most || mb.feat_kept || mb.choice || !cl.dstart) return false;
     // a vertex's communities must fit the block classes' table
     if (g.n > LEVEL_CAP * 3 / 4 && cl.cls_count(CLS_HUGE)) return false;
     // a wave must fit the warps' task and mover lists, and the CTAs' lists of block-class movers
     int need = 1;
+    uint64_t busiest = 0;
     for (int wv = 0; wv < cl.W; wv++) {
         uint64_t tasks = 0, blk = 0;
         for (int k = CLS_G4; k <= CLS_W512; k++) tasks += level_tasks(k, cl.count(k, wv));
@@ -2149,7 +2169,13 @@ bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64
                                     (blk + LEVEL_BMOVERS - 4) / (LEVEL_BMOVERS - 3));
         if (c > LEVEL_CTAS) return false;
         need = std::max(need, (int)c);
+        busiest = std::max(busiest, tasks + 64 * blk);
     }
+    // one task per warp where that takes more than one CTA; fewer CTAs make the
+    // barriers cheaper, and one needs none between CTAs
+    int want = LEVEL_CTAS;
+    while (want > 1 && busiest <= (uint64_t)(want / 2) * LEVEL_WARPS) want /= 2;
+    while (want < need) want *= 2;
     MoveArgs a = make_move_args(g, mb, true, rule, 0, max_it);
     struct Scratch { double dq[3]; uint32_t nlive[3]; int iterations; };
     static_assert(sizeof(Scratch) <= sizeof(uint32_t) * MAX_WAVES * MAX_REPEATS, "the persistent sweep's counters hold it");
@@ -2159,8 +2185,8 @@ bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64
     const LevelArgs v{cl.list, cl.dstart, cl.W, std::min(std::max(mb.repeats, 1), MAX_REPEATS), g.n, tau, max_it,
                       d->dq, &d->iterations, G, live, li, d->nlive};
     bool ran;
-    if (g.wt == GSP_W_F32) ran = fp64 ? launch_level<float, true>(a, v, need, s) : launch_level<float, false>(a, v, need, s);
-    else ran = fp64 ? launch_level<double, true>(a, v, need, s) : launch_level<double, false>(a, v, need, s);
+    if (g.wt == GSP_W_F32) ran = fp64 ? launch_level<float, true>(a, v, need, want, s) : launch_level<float, false>(a, v, need, want, s);
+    else ran = fp64 ? launch_level<double, true>(a, v, need, want, s) : launch_level<double, false>(a, v, need, want, s);
     if (ran) {
         GSP_CUDA(cudaMemcpyAsync(&out.iterations, &d->iterations, sizeof(int), cudaMemcpyDeviceToHost, s));
         GSP_CUDA(cudaMemcpyAsync(&out.ctr, mb.ctr, sizeof(MoveCounters), cudaMemcpyDeviceToHost, s));
@@ -2185,11 +2211,11 @@ void move_wave(const DevGraph &g, const Classes &cl, MoveBuffers &mb, int wave, 
 }
 
 void apply_moves(const DevGraph &g, MoveBuffers &mb, uint32_t n_hint, cudaStream_t s) {
-    k_apply_moves<<<grid_for(n_hint, 256, sms(4)), 256, 0, s>>>(mb.mv_vtx, mb.mv_cmt, mb.mv_cnt, mb.K, mb.C,
-                                                                 mb.Sigma, mb.size, mb.lsb, mb.left, mb.left_it,
-                                                                 mb.it_dev);
-    GSP_CHECK_LAUNCH();
-    k_merge_marks<<<grid_for(g.n / 16 + 1, 256, sms(8)), 256, 0, s>>>(mb.act, mb.mark, g.n);
+    const unsigned appliers = grid_for(n_hint, 256, sms(4));
+    const unsigned mergers = grid_for(g.n / 16 + 1, 256, sms(4));
+    k_apply_moves<<<appliers + mergers, 256, 0, s>>>(mb.mv_vtx, mb.mv_cmt, mb.mv_cnt, mb.K, mb.C, mb.Sigma, mb.size,
+                                                     mb.lsb, mb.left, mb.left_it, mb.it_dev, appliers, mb.act, mb.mark,
+                                                     g.n);
     GSP_CHECK_LAUNCH();
 }
 
