@@ -37,23 +37,71 @@ constexpr uint64_t ACLS_MAX[NUM_ACLS] = {64, 512, 2048, ~0ull};
 enum { RCLS_W = 0, RCLS_B, RCLS_L, NUM_RCLS };
 constexpr uint64_t RCLS_MAX[NUM_RCLS] = {32, 2048, ~0ull};
 
-template <typename WT>
-__global__ void k_agg_count(const uint64_t *__restrict__ off, const uint32_t *__restrict__ Cd, uint32_t n,
-                            uint32_t *cnt, unsigned long long *cdeg) {
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        uint32_t c = Cd[v];
-        atomicAdd(cnt + c, 1u);
-        uint64_t deg = off[v + 1] - off[v];
-        if (deg) atomicAdd(cdeg + c, (unsigned long long)deg);
+// Members and total degree of each community, and the members' lists.  A level
+// often has a few communities with a tenth of the vertices each, whose counters
+// took every vertex's atomics one after the other: a block first counts a tile
+// of vertices in a shared table (as many slots as twice the tile's vertices)
+// and then adds, or reserves, once per community that it met.  R-MAT 20 with a
+// star partition: count 434 us and scatter 388 us before.
+constexpr int TILE_PER = 4, TILE = 256 * TILE_PER, TILE_SLOTS = 2 * TILE;
+
+__device__ __forceinline__ uint32_t tile_slot(uint32_t *keys, uint32_t c) {
+    uint32_t h = hash32(c) / (0xFFFFFFFFu / TILE_SLOTS + 1u);
+    for (;;) {  // ends: the table holds twice the tile's vertices
+        uint32_t old = *(volatile uint32_t *)(keys + h);
+        if (old == EMPTY) old = atomicCAS(keys + h, EMPTY, c);
+        if (old == EMPTY || old == c) return h;
+        h = (h + 1) & (TILE_SLOTS - 1);
     }
 }
 
-__global__ void k_agg_scatter(const uint32_t *__restrict__ Cd, uint32_t n, const uint64_t *__restrict__ coff,
-                              uint32_t *cnt, uint32_t *cverts) {
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        uint32_t c = Cd[v];
-        uint32_t pos = atomicSub(cnt + c, 1u) - 1u;
-        cverts[coff[c] + pos] = v;
+__global__ void __launch_bounds__(256) k_agg_count(const uint64_t *__restrict__ off, const uint32_t *__restrict__ Cd,
+                                                   uint32_t n, uint32_t *cnt, unsigned long long *cdeg) {
+    __shared__ uint32_t keys[TILE_SLOTS], num[TILE_SLOTS];
+    __shared__ unsigned long long deg[TILE_SLOTS];
+    for (uint64_t t0 = (uint64_t)blockIdx.x * TILE; t0 < n; t0 += (uint64_t)gridDim.x * TILE) {
+        for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) { keys[s] = EMPTY; num[s] = 0; deg[s] = 0; }
+        __syncthreads();
+        for (uint64_t v = t0 + threadIdx.x; v < min(t0 + TILE, (uint64_t)n); v += 256) {
+            const uint32_t s = tile_slot(keys, Cd[v]);
+            atomicAdd(num + s, 1u);
+            atomicAdd(deg + s, (unsigned long long)(off[v + 1] - off[v]));
+        }
+        __syncthreads();
+        for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) {
+            if (keys[s] == EMPTY) continue;
+            atomicAdd(cnt + keys[s], num[s]);
+            if (deg[s]) atomicAdd(cdeg + keys[s], deg[s]);
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k_agg_scatter(const uint32_t *__restrict__ Cd, uint32_t n,
+                                                     const uint64_t *__restrict__ coff, uint32_t *cnt,
+                                                     uint32_t *cverts) {
+    __shared__ uint32_t keys[TILE_SLOTS], num[TILE_SLOTS];
+    for (uint64_t t0 = (uint64_t)blockIdx.x * TILE; t0 < n; t0 += (uint64_t)gridDim.x * TILE) {
+        for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) { keys[s] = EMPTY; num[s] = 0; }
+        __syncthreads();
+        uint32_t slot[TILE_PER], rank[TILE_PER];
+#pragma unroll
+        for (int u = 0; u < TILE_PER; u++) {
+            const uint64_t v = t0 + u * 256 + threadIdx.x;
+            slot[u] = EMPTY;
+            if (v >= n) continue;
+            slot[u] = tile_slot(keys, Cd[v]);
+            rank[u] = atomicAdd(num + slot[u], 1u);
+        }
+        __syncthreads();
+        for (int s = threadIdx.x; s < TILE_SLOTS; s += 256)  // the members' places end at cnt: take num of them
+            if (keys[s] != EMPTY) num[s] = atomicSub(cnt + keys[s], num[s]) - num[s];
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < TILE_PER; u++)
+            if (slot[u] != EMPTY)
+                cverts[coff[keys[slot[u]]] + num[slot[u]] + rank[u]] = (uint32_t)(t0 + u * 256 + threadIdx.x);
+        __syncthreads();
     }
 }
 
@@ -931,8 +979,8 @@ static uint64_t aggregate_impl(const DevGraph &g, const uint32_t *Cd, uint32_t k
     GSP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * k, s));
     GSP_CUDA(cudaMemsetAsync(cdeg, 0, sizeof(unsigned long long) * k, s));
     GSP_CUDA(cudaMemsetAsync(rowlen, 0, sizeof(uint32_t) * k, s));
-    unsigned gr = grid_for(n, 256);
-    k_agg_count<WT><<<gr, 256, 0, s>>>(g.off, Cd, n, cnt, cdeg);
+    unsigned gr = grid_for(n, TILE, sms(8));
+    k_agg_count<<<gr, 256, 0, s>>>(g.off, Cd, n, cnt, cdeg);
     GSP_CHECK_LAUNCH();
     exclusive_scan_u32_to_u64(cnt, coff, k, s);
     exclusive_scan_u64(reinterpret_cast<const uint64_t *>(cdeg), yoff, k, s);

@@ -8,6 +8,7 @@
 // when the total fits 2^52 such units (exact_lsb), otherwise in float64 over
 // float32-representable weights whose partial sums stay representable.
 #include <cmath>
+#include <cstring>
 
 #include "internal.cuh"
 
@@ -15,16 +16,43 @@ namespace gsp {
 
 constexpr uint32_t SHORT_ROW = 64;
 
+// f(x) for every x[i], i < n, 16 bytes at a time and four of them in flight;
+// x need only be aligned to its elements (the ends are read one by one).
+template <typename T, typename F> __device__ __forceinline__ void for_each_16b(const T *__restrict__ x, uint64_t n, F &&f) {
+    constexpr int PER = 16 / sizeof(T);
+    const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, nt = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t head = min(n, (uint64_t)((16 - (reinterpret_cast<uintptr_t>(x) & 15)) & 15) / sizeof(T));
+    const uint64_t vecs = (n - head) / PER;
+    const uint4 *v = reinterpret_cast<const uint4 *>(x + head);
+    auto each = [&](const uint4 &q) {
+        T e[PER];
+        memcpy(e, &q, 16);
+#pragma unroll
+        for (int k = 0; k < PER; k++) f(e[k]);
+    };
+    uint64_t i = tid;
+    for (; i + 3 * nt < vecs; i += 4 * nt) {
+        uint4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) q[u] = __ldg(v + i + u * nt);
+#pragma unroll
+        for (int u = 0; u < 4; u++) each(q[u]);
+    }
+    for (; i < vecs; i += nt) each(__ldg(v + i));
+    const uint64_t tail = head + vecs * PER;
+    if (tid < head) f(x[tid]);
+    if (tid < n - tail) f(x[tail + tid]);
+}
+
 // Smallest lowest-set-bit exponent over the weights and their (rounded) sum.
 template <typename WT>
 __global__ void k_weight_range(const WT *__restrict__ w, uint64_t nnz, int *minlow, double *sum) {
     int lo = INT_MAX;
     float acc = 0.0f;  // an estimate for the range test (float64 is slow here)
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
-        const WT x = w[p];
+    for_each_16b(w, nnz, [&](WT x) {
         lo = min(lo, low_bit_exp(x));
         acc += (float)x;
-    }
+    });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lo = min(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
     acc = warp_sum(acc);
@@ -51,7 +79,7 @@ static WeightUnit exact_unit_t(const DevGraph &g, cudaStream_t s) {
     const int init = INT_MAX;
     GSP_CUDA(cudaMemcpyAsync(dlo, &init, sizeof(int), cudaMemcpyHostToDevice, s));
     GSP_CUDA(cudaMemsetAsync(dsum, 0, sizeof(double), s));
-    k_weight_range<WT><<<grid_for(g.nnz, 256, sms(8)), 256, 0, s>>>(static_cast<const WT *>(g.w), g.nnz, dlo, dsum);
+    k_weight_range<WT><<<grid_for(g.nnz, 256 * 16, sms(8)), 256, 0, s>>>(static_cast<const WT *>(g.w), g.nnz, dlo, dsum);
     GSP_CHECK_LAUNCH();
     int lo = 0;
     double sum = 0.0;
@@ -97,6 +125,42 @@ void task_items(const uint64_t *prefix, uint32_t nitems, uint32_t *out, cudaStre
     GSP_CHECK_LAUNCH();
 }
 
+// Sigma of the communities that a block's rows belong to, summed in a shared
+// table before the global adds: a few communities hold most rows, and one
+// float64 atomic per row on their totals took 1.4 of the 1.55 ms of the row
+// sums of a 2 M vertex graph (R-MAT, star partition).  Integer units only (the
+// sums are exact, so their grouping does not show); float64 sums go out as they
+// come.
+struct SigmaSums {
+    static constexpr int LOG = 10;
+    static constexpr uint32_t SLOTS = 1u << LOG;
+    uint32_t keys[SLOTS];
+    unsigned long long sums[SLOTS];
+    __device__ void clear() {
+        for (uint32_t s = threadIdx.x; s < SLOTS; s += blockDim.x) { keys[s] = EMPTY; sums[s] = 0; }
+        __syncthreads();
+    }
+    __device__ void add(double *Sig, uint32_t c, unsigned long long k, int lsb) {
+        uint32_t h = hash32(c) >> (32 - LOG);
+        for (int probe = 0; probe < 4; probe++) {
+            uint32_t old = *(volatile uint32_t *)(keys + h);
+            if (old == EMPTY) old = atomicCAS(keys + h, EMPTY, c);
+            if (old == EMPTY || old == c) {
+                atomicAdd(sums + h, k);
+                return;
+            }
+            h = (h + 1) & (SLOTS - 1);
+        }
+        atomicAdd(Sig + c, Acc<unsigned long long>::val(k, lsb));  // crowded
+    }
+    __device__ void add(double *Sig, uint32_t c, double k, int) { atomicAdd(Sig + c, k); }
+    __device__ void flush(double *Sig, int lsb) {
+        __syncthreads();
+        for (uint32_t s = threadIdx.x; s < SLOTS; s += blockDim.x)
+            if (sums[s]) atomicAdd(Sig + keys[s], Acc<unsigned long long>::val(sums[s], lsb));
+    }
+};
+
 // Per row i: K_i, and the intra-community part sum_{j: C_j = C_i} w_ij when C
 // is given; Sigma_c += K_i when Sig is given.  Long rows are deferred to a
 // list for the block kernel.
@@ -106,6 +170,8 @@ __global__ void k_row_sums(const uint64_t *__restrict__ off, const uint32_t *__r
                            double *Sig, AV *acc /* [0]=2m, [1]=intra */, uint32_t *longlist,
                            uint32_t *nlong, int lsb) {
     __shared__ AV red[32];
+    __shared__ SigmaSums sig;
+    if (Sig) sig.clear();
     AV two_m = 0, intra = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint64_t b = off[i], e = off[i + 1];
@@ -136,12 +202,12 @@ __global__ void k_row_sums(const uint64_t *__restrict__ off, const uint32_t *__r
             k += wv;
             if (C && C[tgt[p]] == ci) in += wv;
         }
-        const double kd = Acc<AV>::val(k, lsb);
-        if (K) K[i] = kd;
-        if (Sig) atomicAdd(Sig + ci, kd);
+        if (K) K[i] = Acc<AV>::val(k, lsb);
+        if (Sig) sig.add(Sig, ci, k, lsb);
         two_m += k;
         intra += in;
     }
+    if (Sig) sig.flush(Sig, lsb);
     two_m = block_sum(two_m, red);
     intra = block_sum(intra, red);
     if (threadIdx.x == 0) {
@@ -158,6 +224,8 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
                                 const WT *__restrict__ w, const uint32_t *__restrict__ C, double *K, double *Sig,
                                 AV *acc, const uint32_t *longlist, const uint32_t *nlong, int lsb) {
     __shared__ AV red[32];
+    __shared__ SigmaSums sig;
+    if (Sig) sig.clear();
     uint32_t cnt = *nlong;
     const int lane = threadIdx.x & 31;
     uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -193,9 +261,8 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
         k = warp_sum(k);
         in = warp_sum(in);
         if (lane == 0) {
-            const double kd = Acc<AV>::val(k, lsb);
-            if (K) K[i] = kd;
-            if (Sig) atomicAdd(Sig + ci, kd);
+            if (K) K[i] = Acc<AV>::val(k, lsb);
+            if (Sig) sig.add(Sig, ci, k, lsb);
             wk += k;
             win += in;
         }
@@ -232,13 +299,13 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
         k = block_sum(k, red);
         in = block_sum(in, red);
         if (threadIdx.x == 0) {
-            const double kd = Acc<AV>::val(k, lsb);
-            if (K) K[i] = kd;
-            if (Sig) atomicAdd(Sig + ci, kd);
+            if (K) K[i] = Acc<AV>::val(k, lsb);
+            if (Sig) sig.add(Sig, ci, k, lsb);
             wk += k;
             win += in;
         }
     }
+    if (Sig) sig.flush(Sig, lsb);
     wk = block_sum(wk, red);
     win = block_sum(win, red);
     if (threadIdx.x == 0) {
@@ -374,8 +441,7 @@ double modularity_scratch(const DevGraph &g, const uint32_t *C, double *Sig, dou
 
 __global__ void k_count_ge(const uint32_t *__restrict__ x, uint64_t n, uint32_t bound, unsigned long long *out) {
     unsigned long long b = 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        if (x[i] >= bound) b++;
+    for_each_16b(x, n, [&](uint32_t v) { b += v >= bound; });
     if (b) atomicAdd(out, b);
 }
 
@@ -385,7 +451,7 @@ unsigned long long count_out_of_range(const uint32_t *x, uint64_t n, uint32_t bo
                                       cudaStream_t s) {
     GSP_CUDA(cudaMemsetAsync(counter, 0, sizeof(*counter), s));
     if (n) {
-        k_count_ge<<<grid_for(n, 256), 256, 0, s>>>(x, n, bound, counter);
+        k_count_ge<<<grid_for(n, 256 * 16, sms(8)), 256, 0, s>>>(x, n, bound, counter);
         GSP_CHECK_LAUNCH();
     }
     unsigned long long h = 0;

@@ -1,4 +1,4 @@
-"""Aggregation at the total degrees where a community changes kernel (64, 512,
+"""The shared-table sums of the phase calls.  Aggregation at the total degrees where a community changes kernel (64, 512,
 2048 entries, tasks of 2048) and in each form of the table values: 32-bit units
 beside their key, 64-bit units, float64."""
 import numpy as np
@@ -58,3 +58,35 @@ def test_aggregate_at_class_boundaries(gsp, values, self_edges):
     assert np.array_equal(gt.cpu().numpy().astype(np.uint32), ot)
     # "wide" spans 60 binary orders: float64 sums in any order, n terms
     assert np.allclose(gw.cpu().numpy(), ow, rtol=0 if values != "wide" else 9000 * 2.0 ** -53, atol=0)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("parts", ["giant", "few", "own"])
+def test_sums_on_views_and_crowded_communities(gsp, shift, parts):
+    """Targets and weights that start off a 16-byte boundary, and communities
+    that hold most rows, a handful or one row each: K, Q and the super-graph
+    are exact (whole weights)."""
+    off, tgt, _ = graphgen.rmat(12, 10, seed=3)
+    n = len(off) - 1
+    rng = np.random.default_rng(shift)
+    w = rng.integers(1, 50, len(tgt)).astype(np.float32)
+    C = {"giant": np.where(rng.random(n) < 0.9, 7, np.arange(n)), "few": rng.integers(0, 5, n),
+         "own": np.arange(n)}[parts].astype(np.uint32)
+    g = oracle.Graph(off, tgt, w.astype(np.float64))
+
+    def view(x):
+        t = torch.from_numpy(np.concatenate([np.zeros(shift, x.dtype), x])).cuda()
+        return t[shift:]
+
+    dev = (torch.from_numpy(off.astype(np.int64)).cuda(), view(tgt.astype(np.int32)), view(w))
+    K, m = gsp.vertex_weights(*dev)
+    Ko, mo = oracle.vertex_weights(g)
+    assert np.array_equal(K.cpu().numpy(), Ko) and m == mo
+    dC = torch.from_numpy(C.astype(np.int32)).cuda()
+    assert gsp.modularity(*dev, dC) == pytest.approx(oracle.modularity(g, C), rel=1e-12, abs=1e-14)
+    D, k = gsp.renumber(dC)
+    want = oracle.aggregate(g, oracle.renumber(C)[0], k)
+    go, gt, gw = gsp.aggregate(*dev, D, k)
+    assert np.array_equal(go.cpu().numpy().astype(np.uint64), want.offsets)
+    assert np.array_equal(gt.cpu().numpy().astype(np.uint32), want.targets)
+    assert np.array_equal(gw.cpu().numpy(), want.weights)
