@@ -641,21 +641,31 @@ void alloc_pool(MoveBuffers &mb, const Classes &cl, bool fp64, cudaStream_t s) {
 }
 
 // --------------------------------------------------------- GSP-Louvain run
+// Times of a run's phases: each lap records an event and says where its time
+// goes; resolve() reads them all at the end, so that no phase waits for the one
+// before (a wait per lap left the device idle four times a pass, 0.1 ms of a
+// small graph's call).
 struct Timer {
+    struct Lap {
+        cudaEvent_t a, b;
+        float *ms;
+    };
+    std::vector<Lap> laps;
     cudaEvent_t a;
     cudaStream_t s;
     explicit Timer(cudaStream_t st) : s(st) {
         a = g_events.get();
         GSP_CUDA(cudaEventRecord(a, s));
     }
-    float lap() {  // ms since the previous lap
+    void lap(float *ms) {  // *ms: the time since the previous lap (nullptr: not wanted)
         cudaEvent_t b = g_events.get();
         GSP_CUDA(cudaEventRecord(b, s));
-        GSP_CUDA(cudaEventSynchronize(b));
-        float ms = 0;
-        GSP_CUDA(cudaEventElapsedTime(&ms, a, b));
+        if (ms) laps.push_back({a, b, ms});
         a = b;
-        return ms;
+    }
+    void resolve() {
+        GSP_CUDA(cudaEventSynchronize(a));
+        for (const Lap &l : laps) GSP_CUDA(cudaEventElapsedTime(l.ms, l.a, l.b));
     }
 };
 
@@ -726,7 +736,8 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
     for (int lp = 0; lp < o.max_passes; lp++) {
         const uint32_t nv = cur.n;
         size_t pass_mark = arena().mark();
-        t.lap();
+        const bool record = lp < GSP_MAX_PASS_STATS;
+        t.lap(nullptr);
         // K' = Sigma' = vertexWeights(G'), C' = [0..|V'|), all unprocessed;
         // with refinement, after an aggregation, C' holds each super-vertex's
         // bound community and Sigma' sums K' over it
@@ -755,28 +766,25 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
         Classes cl;
         classify_vertices(cur, cl, W, s);
         alloc_pool(mb, cl, fp64, s);
-        float ms_other = t.lap();
+        t.lap(record ? &local.ms_other[lp] : nullptr);
         MoveLoopResult mr{0, 0, 0, 0, 0, 0.0, 0.0f};
         if (m > 0.0) mr = move_loop(cur, cl, mb, tau, o.max_iterations, sync, fp64, o.singleton_rule != 0, pr, s);
         int li = mr.iterations;
         Cp = mb.C;
-        float ms_move = t.lap();
+        t.lap(record ? &local.ms_move[lp] : nullptr);
         if (split_pass) {
             split_labels(cur, cl, Cp, o.split, labels, s);
             Cp = labels;
         }
         // |Gamma| = communities after the split; |Gamma_old| = |V'|
         uint32_t k = renumber(nv, Cp, Cd, s);
-        float ms_split = t.lap();
+        t.lap(record ? &local.ms_split[lp] : nullptr);
         passes = lp + 1;
-        if (lp < GSP_MAX_PASS_STATS) {
+        if (record) {
             local.iterations[lp] = li;
             local.vertices[lp] = nv;
             local.communities[lp] = k;
             local.edges[lp] = cur.nnz;
-            local.ms_move[lp] = ms_move;
-            local.ms_split[lp] = ms_split;
-            local.ms_other[lp] = ms_other;
             local.vertices_processed[lp] = mr.vertices;
             local.edges_scanned[lp] = mr.edges;
             local.vertices_skipped[lp] = mr.skipped;
@@ -792,11 +800,8 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
             refine_partition(cur, cl, Cp, Rf, K, m, o.refine_theta, o.seed, (uint32_t)lp, fp64, s);
             k = renumber(nv, Rf, Rd, s);
             A = Rd;
-            float ms_ref = t.lap();
-            if (lp < GSP_MAX_PASS_STATS) {
-                local.refined[lp] = k;
-                local.ms_refine[lp] = ms_ref;
-            }
+            t.lap(record ? &local.ms_refine[lp] : nullptr);
+            if (record) local.refined[lp] = k;
         }
         if ((double)k / (double)nv > o.aggregation_tolerance) break;  // low shrink
         // renumber, dendrogram lookup, aggregate, threshold scaling
@@ -813,8 +818,7 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
         tau = tau / o.tolerance_drop;
         // C' on the new graph: the identity, or each super-vertex's bound community
         if (refine) scatter_bound(A, Cd, mb.C, nv, s);
-        float ms_agg = t.lap();
-        if (lp < GSP_MAX_PASS_STATS) local.ms_aggregate[lp] = ms_agg;
+        t.lap(record ? &local.ms_aggregate[lp] : nullptr);
         arena().release(pass_mark);
         if (!refine) iota_u32(mb.C, cur.n, s);
         Cp = mb.C;
@@ -838,7 +842,9 @@ void louvain_run(const DevGraph &g0, const gsp_opts &o, uint32_t *membership, do
     local.passes = passes;
     local.final_communities = kf;
     local.modularity = q;
-    local.ms_total = total.lap();
+    total.lap(&local.ms_total);
+    total.resolve();
+    t.resolve();
     local.disconnected = o.count_disconnected ? count_disconnected(g0, membership, nullptr, s) : GSP_NOT_COUNTED;
     local.workspace_bytes = workspace_peak();
     if (modularity_out) *modularity_out = q;
