@@ -42,10 +42,14 @@ constexpr uint64_t RCLS_MAX[NUM_RCLS] = {32, 2048, ~0ull};
 // took every vertex's atomics one after the other: a block first counts a tile
 // of vertices in a shared table (as many slots as twice the tile's vertices)
 // and then adds, or reserves, once per community that it met.  R-MAT 20 with a
-// star partition: count 434 us and scatter 388 us before.
-constexpr int TILE_PER = 4, TILE = 256 * TILE_PER, TILE_SLOTS = 2 * TILE;
+// star partition: count 434 us and scatter 388 us before.  Small graphs have
+// too few vertices for blocks of 1024 to hide a block's chain of clearing,
+// counting and reserving: tiles of 256 there (aggregate_impl).
+template <int PER> struct Tile {
+    static constexpr int N = 256 * PER, SLOTS = 2 * N;
+};
 
-__device__ __forceinline__ uint32_t tile_slot(uint32_t *keys, uint32_t c) {
+template <int TILE_SLOTS> __device__ __forceinline__ uint32_t tile_slot(uint32_t *keys, uint32_t c) {
     uint32_t h = hash32(c) / (0xFFFFFFFFu / TILE_SLOTS + 1u);
     for (;;) {  // ends: the table holds twice the tile's vertices
         uint32_t old = *(volatile uint32_t *)(keys + h);
@@ -55,15 +59,17 @@ __device__ __forceinline__ uint32_t tile_slot(uint32_t *keys, uint32_t c) {
     }
 }
 
+template <int PER>
 __global__ void __launch_bounds__(256) k_agg_count(const uint64_t *__restrict__ off, const uint32_t *__restrict__ Cd,
                                                    uint32_t n, uint32_t *cnt, unsigned long long *cdeg) {
+    constexpr int TILE = Tile<PER>::N, TILE_SLOTS = Tile<PER>::SLOTS;
     __shared__ uint32_t keys[TILE_SLOTS], num[TILE_SLOTS];
     __shared__ unsigned long long deg[TILE_SLOTS];
     for (uint64_t t0 = (uint64_t)blockIdx.x * TILE; t0 < n; t0 += (uint64_t)gridDim.x * TILE) {
         for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) { keys[s] = EMPTY; num[s] = 0; deg[s] = 0; }
         __syncthreads();
         for (uint64_t v = t0 + threadIdx.x; v < min(t0 + TILE, (uint64_t)n); v += 256) {
-            const uint32_t s = tile_slot(keys, Cd[v]);
+            const uint32_t s = tile_slot<TILE_SLOTS>(keys, Cd[v]);
             atomicAdd(num + s, 1u);
             atomicAdd(deg + s, (unsigned long long)(off[v + 1] - off[v]));
         }
@@ -77,20 +83,22 @@ __global__ void __launch_bounds__(256) k_agg_count(const uint64_t *__restrict__ 
     }
 }
 
+template <int PER>
 __global__ void __launch_bounds__(256) k_agg_scatter(const uint32_t *__restrict__ Cd, uint32_t n,
                                                      const uint64_t *__restrict__ coff, uint32_t *cnt,
                                                      uint32_t *cverts) {
+    constexpr int TILE = Tile<PER>::N, TILE_SLOTS = Tile<PER>::SLOTS;
     __shared__ uint32_t keys[TILE_SLOTS], num[TILE_SLOTS];
     for (uint64_t t0 = (uint64_t)blockIdx.x * TILE; t0 < n; t0 += (uint64_t)gridDim.x * TILE) {
         for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) { keys[s] = EMPTY; num[s] = 0; }
         __syncthreads();
-        uint32_t slot[TILE_PER], rank[TILE_PER];
+        uint32_t slot[PER], rank[PER];
 #pragma unroll
-        for (int u = 0; u < TILE_PER; u++) {
+        for (int u = 0; u < PER; u++) {
             const uint64_t v = t0 + u * 256 + threadIdx.x;
             slot[u] = EMPTY;
             if (v >= n) continue;
-            slot[u] = tile_slot(keys, Cd[v]);
+            slot[u] = tile_slot<TILE_SLOTS>(keys, Cd[v]);
             rank[u] = atomicAdd(num + slot[u], 1u);
         }
         __syncthreads();
@@ -98,7 +106,7 @@ __global__ void __launch_bounds__(256) k_agg_scatter(const uint32_t *__restrict_
             if (keys[s] != EMPTY) num[s] = atomicSub(cnt + keys[s], num[s]) - num[s];
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < TILE_PER; u++)
+        for (int u = 0; u < PER; u++)
             if (slot[u] != EMPTY)
                 cverts[coff[keys[slot[u]]] + num[slot[u]] + rank[u]] = (uint32_t)(t0 + u * 256 + threadIdx.x);
         __syncthreads();
@@ -885,15 +893,20 @@ template <typename WT, typename AV>
 static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &ic, const unsigned long long *cdeg,
                          const uint32_t *cverts, uint32_t k, uint32_t n, cudaStream_t s) {
     auto cnt_of = [&](int c) { return ic.start[c + 1] - ic.start[c]; };
-    auto warp_class = [&](auto fn, int cls, int cap, int warps, unsigned per_sm) {
-        if (!cnt_of(cls)) return;
+    auto warp_class = [&](auto fn, uint32_t first, uint32_t last, int cap, int warps, unsigned per_sm) {
+        if (first == last) return;
         const size_t smem = (size_t)warps * cap * AggTable<AV>::slot_bytes;  // at most 48 KB: no opt-in
-        fn<<<grid_for((uint64_t)cnt_of(cls) * 32, warps * 32, sms(per_sm)), warps * 32, smem, s>>>(
-            a, ic.list + ic.start[cls], cnt_of(cls));
+        fn<<<grid_for((uint64_t)(last - first) * 32, warps * 32, sms(per_sm)), warps * 32, smem, s>>>(
+            a, ic.list + first, last - first);
         GSP_CHECK_LAUNCH();
     };
-    warp_class(k_agg_merge_warp<AGG_SCAP, AGG_SWARPS, WT, AV>, ACLS_S, AGG_SCAP, AGG_SWARPS, 32);
-    warp_class(k_agg_merge_warp<AGG_WCAP, AGG_WWARPS, WT, AV>, ACLS_W, AGG_WCAP, AGG_WWARPS, 8);
+    // the two classes lie side by side in the list: as long as 8 warps an SM
+    // hold them all, the larger tables serve both in one launch.  With the
+    // smaller tiles, R-MAT of 6 K vertices / 190 K entries: aggregation 420 ->
+    // 378 us, 25 K 536 -> 493, 70 K 614 -> 566; above (110 K) 735 either way
+    const uint32_t e = ic.start[ACLS_W + 1], mid = cnt_of(ACLS_W) && e <= sms(8) ? 0 : ic.start[ACLS_W];
+    warp_class(k_agg_merge_warp<AGG_SCAP, AGG_SWARPS, WT, AV>, 0, mid, AGG_SCAP, AGG_SWARPS, 32);
+    warp_class(k_agg_merge_warp<AGG_WCAP, AGG_WWARPS, WT, AV>, mid, e, AGG_WCAP, AGG_WWARPS, 8);
     if (cnt_of(ACLS_B)) {
         constexpr size_t smem = (size_t)AGG_BCAP * AggTable<AV>::slot_bytes + (size_t)AGG_BMEM * sizeof(uint64_t) +
                                 (size_t)(AGG_BMEM + 1) * sizeof(uint32_t);
@@ -979,12 +992,16 @@ static uint64_t aggregate_impl(const DevGraph &g, const uint32_t *Cd, uint32_t k
     GSP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * k, s));
     GSP_CUDA(cudaMemsetAsync(cdeg, 0, sizeof(unsigned long long) * k, s));
     GSP_CUDA(cudaMemsetAsync(rowlen, 0, sizeof(uint32_t) * k, s));
-    unsigned gr = grid_for(n, TILE, sms(8));
-    k_agg_count<<<gr, 256, 0, s>>>(g.off, Cd, n, cnt, cdeg);
+    // tiles of 1024 vertices; of 256 where those are at most two blocks an SM
+    const bool few = n <= 256ull * sms(2);
+    const unsigned gr = grid_for(n, few ? Tile<1>::N : Tile<4>::N, sms(8));
+    if (few) k_agg_count<1><<<gr, 256, 0, s>>>(g.off, Cd, n, cnt, cdeg);
+    else k_agg_count<4><<<gr, 256, 0, s>>>(g.off, Cd, n, cnt, cdeg);
     GSP_CHECK_LAUNCH();
     exclusive_scan_u32_to_u64(cnt, coff, k, s);
     exclusive_scan_u64(reinterpret_cast<const uint64_t *>(cdeg), yoff, k, s);
-    k_agg_scatter<<<gr, 256, 0, s>>>(Cd, n, coff, cnt, cverts);
+    if (few) k_agg_scatter<1><<<gr, 256, 0, s>>>(Cd, n, coff, cnt, cverts);
+    else k_agg_scatter<4><<<gr, 256, 0, s>>>(Cd, n, coff, cnt, cverts);
     GSP_CHECK_LAUNCH();
 
     IdClasses ic;
