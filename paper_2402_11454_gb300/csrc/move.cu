@@ -8,7 +8,7 @@
 //   groups of G = 4/8/16/32 lanes per vertex, table in shared memory (one
 //     fused launch for the four group classes);
 //   one warp per vertex, 1024-slot shared table (degree <= 512);
-//   one block per vertex, table in shared memory (degree <= 2048);
+//   one block per vertex, table in shared memory (degree <= 2048, <= 8192);
 //   the whole grid per vertex for larger degrees ("hubs"): edge-chunk tasks
 //     combined in shared memory, published to a global-memory table.
 // Duplicate community keys meet in the table through atomicCAS on the key and
