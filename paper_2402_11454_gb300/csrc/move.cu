@@ -1216,12 +1216,16 @@ struct LevelArgs {
 };
 
 // Barrier of all CTAs, split into arrival and wait; alone, a CTA's own barrier
-// at the wait (a cluster barrier's release and acquire cost 0.7-1.3 us).
+// at the wait (a cluster barrier's release and acquire cost 0.7-1.3 us).  The
+// aligned forms take whole warps, and the code before them parts the lanes
+// (level_fetch between arrival and wait leaves the lanes without a vertex
+// early): each half brings its warp together first.
 __device__ __forceinline__ void level_arrive(bool alone) {
     __syncwarp();
     if (!alone) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void level_wait(bool alone) {
+    __syncwarp();
     if (alone) __syncthreads();
     else asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
