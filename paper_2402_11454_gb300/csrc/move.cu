@@ -630,6 +630,7 @@ __device__ void group_body(const MoveArgs &a, const uint32_t *__restrict__ list,
     const int wl = threadIdx.x & 31, gl = wl % G, gw = wl / G;
     Table<V> tab(warp_smem, NGW * CAP, gw * CAP);
     for (int t = gl; t < CAP; t += G) tab.clear(t);
+    __syncwarp();  // votes and shuffles do not order shared memory
     const WT *w = static_cast<const WT *>(a.w);
     const double m0 = *a.m, inv0 = a.m[1];
     const int it = *a.iteration;
@@ -1352,6 +1353,7 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
     auto clear_tables = [&]() {
         Table<V> tab(ws, W512_CAP, 0);
         for (int t = lane; t < W512_CAP; t += 32) tab.clear(t);
+        __syncwarp();  // votes and shuffles do not order shared memory
     };
     clear_tables();
     __syncthreads();
