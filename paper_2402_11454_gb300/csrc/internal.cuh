@@ -356,6 +356,21 @@ __device__ __forceinline__ int select_bit(unsigned m, int q) {
     return pos;
 }
 
+// Tables of the largest degree class in the global pool: a power of two of
+// slots, at least two per edge, up to 2^32 (there are fewer communities than
+// that).  The largest capacity does not fit 32 bits: the kernels carry the slot
+// mask, capacity - 1, which does.
+__host__ __device__ __forceinline__ uint64_t hub_slots(uint64_t deg) {
+    uint64_t cap = 2;
+    while (cap < 2 * deg && cap < (1ull << 32)) cap <<= 1;
+    return cap;
+}
+// Home slot, the top bits of the hash: hash * (mask + 1) / 2^32.
+__host__ __device__ __forceinline__ uint32_t hub_home(uint32_t hash, uint32_t mask) {
+    return (uint32_t)(((uint64_t)hash * mask + hash) >> 32);
+}
+// First slot of task k of the n that share a table of cap slots.
+__host__ __device__ __forceinline__ uint64_t hub_share(uint64_t cap, uint64_t k, uint64_t n) { return cap * k / n; }
 
 // Open-addressing insert of (c, w) with linear probing: the key is claimed
 // with atomicCAS, the value accumulated with atomicAdd.  The table holds

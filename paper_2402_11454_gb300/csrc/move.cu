@@ -145,25 +145,25 @@ template <> struct Table<float> {
     __device__ Table(unsigned char *base, uint32_t, uint32_t first)
         : t(reinterpret_cast<unsigned long long *>(base) + first) {}
     __device__ explicit Table(unsigned long long *global) : t(global) {}
-    // Add N distinct communities (EMPTY: none) to a table of cap slots in global
-    // memory, all first probes in flight together.
-    template <int N> __device__ void publish(uint32_t cap, const uint32_t (&c)[N], const float (&v)[N]) {
+    // Add N distinct communities (EMPTY: none) to a table of mask + 1 slots in
+    // global memory, all first probes in flight together.
+    template <int N> __device__ void publish(uint32_t mask, const uint32_t (&c)[N], const float (&v)[N]) {
         unsigned long long old[N];
 #pragma unroll
         for (int u = 0; u < N; u++)
             if (c[u] != EMPTY)
-                old[u] = atomicCAS(t + __umulhi(hash32(c[u]), cap), FREE,
+                old[u] = atomicCAS(t + hub_home(hash32(c[u]), mask), FREE,
                                    ((unsigned long long)c[u] << 32) | __float_as_uint(v[u]));
 #pragma unroll
         for (int u = 0; u < N; u++) {
             if (c[u] == EMPTY || old[u] == FREE) continue;
-            uint32_t h = __umulhi(hash32(c[u]), cap);
-            for (uint32_t probe = 0; probe < cap; probe++) {
+            uint32_t h = hub_home(hash32(c[u]), mask);
+            for (uint64_t probe = 0; probe <= mask; probe++) {
                 if ((uint32_t)(old[u] >> 32) == c[u]) {
                     atomicAdd(reinterpret_cast<float *>(t + h), v[u]);
                     break;
                 }
-                if (++h == cap) h = 0;
+                h = (h + 1) & mask;
                 old[u] = atomicCAS(t + h, FREE, ((unsigned long long)c[u] << 32) | __float_as_uint(v[u]));
                 if (old[u] == FREE) break;
             }
@@ -200,18 +200,18 @@ template <> struct Table<double> {
         : keys(reinterpret_cast<uint32_t *>(base) + first),
           vals(reinterpret_cast<double *>(base + (size_t)total * sizeof(uint32_t)) + first) {}
     __device__ Table(uint32_t *gkeys, double *gvals) : keys(gkeys), vals(gvals) {}
-    template <int N> __device__ void publish(uint32_t cap, const uint32_t (&c)[N], const double (&v)[N]) {
+    template <int N> __device__ void publish(uint32_t mask, const uint32_t (&c)[N], const double (&v)[N]) {
 #pragma unroll
         for (int u = 0; u < N; u++) {
             if (c[u] == EMPTY) continue;
-            uint32_t h = __umulhi(hash32(c[u]), cap);
-            for (uint32_t probe = 0; probe < cap; probe++) {
+            uint32_t h = hub_home(hash32(c[u]), mask);
+            for (uint64_t probe = 0; probe <= mask; probe++) {
                 const uint32_t old = atomicCAS(keys + h, EMPTY, c[u]);
                 if (old == EMPTY || old == c[u]) {
                     atomicAdd(vals + h, v[u]);
                     break;
                 }
-                if (++h == cap) h = 0;
+                h = (h + 1) & mask;
             }
         }
     }
@@ -1603,7 +1603,7 @@ __global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_insert(MoveArg
             tab.clear(slot[u]);
         }
         __syncthreads();  // the shared table is empty
-        hub_table<V>(h, t).template publish<HUB_EPT>((uint32_t)(h.pool_off[t + 1] - h.pool_off[t]), c, val);
+        hub_table<V>(h, t).template publish<HUB_EPT>((uint32_t)(h.pool_off[t + 1] - h.pool_off[t] - 1), c, val);
     }
 }
 
@@ -1674,7 +1674,8 @@ __global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_score(MoveArgs
         const uint64_t n = h.tasks[t + 1] - h.tasks[t], k = task + base - h.tasks[t];
         const uint32_t i = h.hubs[t], d = h.d[t];
         const uint64_t cap = h.pool_off[t + 1] - h.pool_off[t];
-        const uint32_t s0 = (uint32_t)(cap * k / n), s1 = (uint32_t)(cap * (k + 1) / n);
+        const uint64_t first = hub_share(cap, k, n);
+        const uint32_t s0 = (uint32_t)first, slots = (uint32_t)(hub_share(cap, k + 1, n) - first);
         Table<V> tab = hub_table<V>(h, t);
         const SC sc = make_score<F64>(a.K[i], kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
                                       vertex_inv_m(a, i, inv0), true);
@@ -1682,20 +1683,20 @@ __global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_score(MoveArgs
         uint32_t bestc = EMPTY, ncand = 0;
         // U slots per thread per round, their gathers of Sigma issued at once
         constexpr int U = 4;
-        for (uint32_t sb = s0 + threadIdx.x; sb < s1; sb += U * HUB_THREADS) {
+        for (uint32_t x = threadIdx.x; x < slots; x += U * HUB_THREADS) {
             uint32_t c[U];
             V val[U];
             double sg[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                const uint32_t s = sb + u * HUB_THREADS;
-                c[u] = s < s1 ? tab.get(s, val[u]) : EMPTY;
+                const uint32_t y = x + u * HUB_THREADS;
+                c[u] = y < slots ? tab.get(s0 + y, val[u]) : EMPTY;
             }
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 sg[u] = 0.0;
                 if (c[u] == EMPTY) continue;
-                tab.clear(sb + u * HUB_THREADS);
+                tab.clear(s0 + x + u * HUB_THREADS);
                 sg[u] = ld_state<SYNC>(a.Sig + c[u]);
             }
 #pragma unroll
@@ -1829,10 +1830,7 @@ __global__ void k_pool_caps(const uint64_t *__restrict__ off, const uint32_t *__
                             uint64_t *caps) {
     for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < count; t += gridDim.x * blockDim.x) {
         uint32_t v = list[t];
-        uint64_t deg = off[v + 1] - off[v];
-        uint64_t cap = 2;
-        while (cap < 2 * deg) cap <<= 1;
-        caps[t] = cap;
+        caps[t] = hub_slots(off[v + 1] - off[v]);
     }
 }
 
