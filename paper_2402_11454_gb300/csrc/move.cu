@@ -326,8 +326,9 @@ template <> struct Score<false> {
 // m and inv_m = 1/m of the vertex's graph (the float64 score uses m only).
 // The float32 operations are spelled out, so that every kernel that may serve
 // a vertex decides exact ties of s_c and s_d alike: the candidates' scores
-// round once (fused); the score of staying rounds twice, but once for the
-// vertices of the largest degree class (hub), whichever kernel serves them.
+// round once (fused); the score of staying rounds twice, but once for a vertex
+// of more than BIG_MAX_LIMIT edges (hub).  That is a property of the vertex: the
+// boundaries between the classes may be tuned, and must not change a decision.
 template <bool F64>
 __device__ __forceinline__ Score<F64> make_score(double Ki, typename std::conditional<F64, double, float>::type kid,
                                                  double Sd, double m, double inv_m, bool hub = false);
@@ -348,6 +349,8 @@ __device__ __forceinline__ Score<false> make_score<false>(double Ki, float kid, 
     s.inv_m = inv_m;
     return s;
 }
+
+__device__ __forceinline__ bool rounds_as_hub(uint64_t deg) { return deg > BIG_MAX_LIMIT; }
 
 // m of vertex i's graph (batches) or of the single graph.
 __device__ __forceinline__ double vertex_m(const MoveArgs &a, uint32_t i, double m0) {
@@ -755,7 +758,7 @@ __global__ void __launch_bounds__(256, F64 ? 2 : 3) k_move_w512(MoveArgs a, cons
 // --------------------------------------------------------------------------
 template <int CAP, int U, typename WT, bool F64, int SYNC>
 __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list, uint32_t count, uint32_t lb,
-                           uint32_t nb, unsigned char *dyn_smem, LocalCtr &lc, uint32_t slots = CAP, bool hub = false) {
+                           uint32_t nb, unsigned char *dyn_smem, LocalCtr &lc, uint32_t slots = CAP) {
     using V = typename std::conditional<F64, double, float>::type;
     using SC = Score<F64>;
     using S = typename SC::S;
@@ -842,7 +845,7 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
             __syncthreads();  // every edge inserted
             kid = warp_sum(lane < nw ? red_k[lane] : V(0));
             const double m = vertex_m(a, i, m0);
-            const SC sc = make_score<F64>(Ki, kid, Sd, m, vertex_inv_m(a, i, inv0), hub);
+            const SC sc = make_score<F64>(Ki, kid, Sd, m, vertex_inv_m(a, i, inv0), rounds_as_hub(deg));
             S best = -INFINITY;
             uint32_t bestc = EMPTY, ncand = 0;
             if (held) score_slots<U, SYNC>(tab, slot, a.Sig, sc, best, bestc, ncand);
@@ -1406,7 +1409,7 @@ __global__ void __launch_bounds__(LEVEL_THREADS, 1) k_move_level(MoveArgs a, Lev
                     for (int k = CLS_HUGE; k >= CLS_BLOCK; k--) {
                         const uint32_t cnt = cls(k, wv, beg);
                         const uint32_t slots = k == CLS_BLOCK ? 4096u : (uint32_t)CAP;
-                        if (cnt) block_body<CAP, 4, WT, F64, 2>(ab, v.list + beg, cnt, lb, nb, sm.tables, lc, slots, k == CLS_HUGE);
+                        if (cnt) block_body<CAP, 4, WT, F64, 2>(ab, v.list + beg, cnt, lb, nb, sm.tables, lc, slots);
                     }
                     clear_tables();
                 }
@@ -1635,7 +1638,8 @@ __device__ void hub_decide(const MoveArgs &a, const HubArgs &h, uint32_t t, Loca
     const double Ki = a.K[i];
     const uint64_t deg = a.off[i + 1] - a.off[i];
     const double m = vertex_m(a, i, a.m[0]);
-    const SC sc = make_score<F64>(Ki, kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, a.m[1]), true);
+    const SC sc = make_score<F64>(Ki, kidv[t], ld_state<SYNC>(a.Sig + d), m, vertex_inv_m(a, i, a.m[1]),
+                                  rounds_as_hub(deg));
     const double gain = (bestc == EMPTY) ? 0.0 : sc.gain(best);
     int mv = 0;
     if (bestc != EMPTY && sc.gains(best)) mv = decide_move<SYNC>(a, i, d, bestc, Ki);
@@ -1677,8 +1681,9 @@ __global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_score(MoveArgs
         const uint64_t first = hub_share(cap, k, n);
         const uint32_t s0 = (uint32_t)first, slots = (uint32_t)(hub_share(cap, k + 1, n) - first);
         Table<V> tab = hub_table<V>(h, t);
+        // hub_decide takes the score of staying; the candidates' do not read it in the mixed mode
         const SC sc = make_score<F64>(a.K[i], kidv[t], ld_state<SYNC>(a.Sig + d), vertex_m(a, i, m0),
-                                      vertex_inv_m(a, i, inv0), true);
+                                      vertex_inv_m(a, i, inv0));
         S best = -INFINITY;
         uint32_t bestc = EMPTY, ncand = 0;
         // U slots per thread per round, their gathers of Sigma issued at once
