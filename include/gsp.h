@@ -459,7 +459,10 @@ typedef struct {
      * with grid-wide barriers) instead of several launches per wave; 0
      * disables it.  Default 0: on a GB300 the per-wave launches replayed
      * from a CUDA graph were as fast (a wave's dependent loads, not its
-     * launches, set the time).  The result is the same either way. */
+     * launches, set the time).  The setting comes before the library's own
+     * choice for small graphs (below about half a million stored entries:
+     * all sweeps of a pass in one thread-block cluster), which the graphs it
+     * does not cover keep.  The result is the same either way. */
     uint32_t persist_max_vertices;
     /* Class boundaries: the largest degree served by the group kernel (33..128,
      * default 128), the warp kernel (..512, default 512), the 4096-slot block

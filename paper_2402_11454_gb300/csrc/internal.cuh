@@ -170,7 +170,7 @@ bool sweep_persistent(const DevGraph &g, const Classes &cl, MoveBuffers &mb, boo
 // The whole local-moving phase of a small graph (every sweep until the gain
 // is <= tau or max_it) as one launch of one thread-block cluster, frozen-state
 // waves.  Returns false (launching nothing) when the graph or the run does
-// not qualify; otherwise *out is filled once the stream is synchronised.
+// not qualify, or the persistent sweep is asked for; otherwise *out is filled once the stream is synchronised.
 // Batches: G graphs, live (device, in/out) the graphs still iterating, li
 // (device) the sweeps of each; mb.dq_g zero at the call.
 struct LevelResult {

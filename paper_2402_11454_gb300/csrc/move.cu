@@ -2115,11 +2115,16 @@ static bool launch_persistent(const MoveArgs &a, const Classes &cl, uint32_t n, 
     return true;
 }
 
+// The caller asked for the persistent sweep on graphs of this size
+// (gsp_tuning.persist_max_vertices), and the graph and the run qualify.
+static bool persistent_asked(const DevGraph &g, const Classes &cl, const MoveBuffers &mb) {
+    return g.n <= tuning().persist_max_vertices && !cl.cls_count(CLS_HUGE) && !cl.cls_count(CLS_BIG) &&
+           !mb.feat_kept && !mb.choice && cl.dstart && mb.bar;
+}
+
 bool sweep_persistent(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64, bool rule, int iteration,
                       int max_iterations, cudaStream_t s) {
-    if (cl.cls_count(CLS_HUGE) || cl.cls_count(CLS_BIG) || mb.feat_kept || mb.choice || !cl.dstart || !mb.bar)
-        return false;
-    if (g.n > tuning().persist_max_vertices) return false;
+    if (!persistent_asked(g, cl, mb)) return false;
     MoveArgs a = make_move_args(g, mb, true, rule, iteration, max_iterations);
     if (g.wt == GSP_W_F32) return fp64 ? launch_persistent<float, true>(a, cl, g.n, mb, iteration, s)
                                        : launch_persistent<float, false>(a, cl, g.n, mb, iteration, s);
@@ -2183,7 +2188,7 @@ bool move_level(const DevGraph &g, const Classes &cl, MoveBuffers &mb, bool fp64
     const uint64_t most = !fp64                              ? LEVEL_MAX_EDGES
                           : g.n <= LEVEL_DENSE_VERTICES ? LEVEL_MAX_EDGES_F64_DENSE
                                                         : LEVEL_MAX_EDGES_F64;
-    if (g.nnz > most || mb.feat_kept || mb.choice || !cl.dstart) return false;
+    if (g.nnz > most || mb.feat_kept || mb.choice || !cl.dstart || persistent_asked(g, cl, mb)) return false;
     // a vertex's communities must fit the block classes' table
     if (g.n > LEVEL_CAP * 3 / 4 && cl.cls_count(CLS_HUGE)) return false;
     // a wave must fit the warps' task and mover lists, and the CTAs' lists of block-class movers
