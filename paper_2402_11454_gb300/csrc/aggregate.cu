@@ -44,7 +44,10 @@ constexpr uint64_t RCLS_MAX[NUM_RCLS] = {32, 2048, ~0ull};
 // and then adds, or reserves, once per community that it met.  R-MAT 20 with a
 // star partition: count 434 us and scatter 388 us before.  Small graphs have
 // too few vertices for blocks of 1024 to hide a block's chain of clearing,
-// counting and reserving: tiles of 256 there (aggregate_impl).
+// counting and reserving: tiles of 256 there (aggregate_impl).  A tile's degrees
+// are summed in two 32-bit halves: a 64-bit add in shared memory is a loop of
+// compare-and-swaps, and the vertices of a hot community queued in it (1.5 K
+// vertices in 32 communities: 14.8 us for the counts, 4.0 without a table).
 template <int PER> struct Tile {
     static constexpr int N = 256 * PER, SLOTS = 2 * N;
 };
@@ -64,20 +67,25 @@ __global__ void __launch_bounds__(256) k_agg_count(const uint64_t *__restrict__ 
                                                    uint32_t n, uint32_t *cnt, unsigned long long *cdeg) {
     constexpr int TILE = Tile<PER>::N, TILE_SLOTS = Tile<PER>::SLOTS;
     __shared__ uint32_t keys[TILE_SLOTS], num[TILE_SLOTS];
-    __shared__ unsigned long long deg[TILE_SLOTS];
+    // sums of the degrees' low 16 bits and of the rest: both below 2^32 while a
+    // row has fewer than 2^38 entries
+    __shared__ uint32_t deg_lo[TILE_SLOTS], deg_hi[TILE_SLOTS];
     for (uint64_t t0 = (uint64_t)blockIdx.x * TILE; t0 < n; t0 += (uint64_t)gridDim.x * TILE) {
-        for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) { keys[s] = EMPTY; num[s] = 0; deg[s] = 0; }
+        for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) { keys[s] = EMPTY; num[s] = 0; deg_lo[s] = 0; deg_hi[s] = 0; }
         __syncthreads();
         for (uint64_t v = t0 + threadIdx.x; v < min(t0 + TILE, (uint64_t)n); v += 256) {
             const uint32_t s = tile_slot<TILE_SLOTS>(keys, Cd[v]);
             atomicAdd(num + s, 1u);
-            atomicAdd(deg + s, (unsigned long long)(off[v + 1] - off[v]));
+            const uint64_t deg = off[v + 1] - off[v];
+            atomicAdd(deg_lo + s, (uint32_t)deg & 0xFFFFu);
+            if (deg >> 16) atomicAdd(deg_hi + s, (uint32_t)(deg >> 16));
         }
         __syncthreads();
         for (int s = threadIdx.x; s < TILE_SLOTS; s += 256) {
             if (keys[s] == EMPTY) continue;
             atomicAdd(cnt + keys[s], num[s]);
-            if (deg[s]) atomicAdd(cdeg + keys[s], deg[s]);
+            const unsigned long long deg = ((unsigned long long)deg_hi[s] << 16) + deg_lo[s];
+            if (deg) atomicAdd(cdeg + keys[s], deg);
         }
         __syncthreads();
     }
@@ -901,9 +909,11 @@ static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &i
         GSP_CHECK_LAUNCH();
     };
     // the two classes lie side by side in the list: as long as 8 warps an SM
-    // hold them all, the larger tables serve both in one launch.  With the
-    // smaller tiles, R-MAT of 6 K vertices / 190 K entries: aggregation 420 ->
-    // 378 us, 25 K 536 -> 493, 70 K 614 -> 566; above (110 K) 735 either way
+    // hold them all, the larger tables serve both in one launch.  Two launches
+    // and tiles of 1024 against this, R-MAT of 6 K vertices / 190 K entries:
+    // aggregation 420 and 378 us, 25 K 536 and 493, 70 K 614 and 566; above
+    // (110 K) 735 either way.  Since then the tiles' degree sums made it 361 at
+    // 6 K and 476 at 25 K (one atomic a vertex and no tiles: 366 and 513)
     const uint32_t e = ic.start[ACLS_W + 1], mid = cnt_of(ACLS_W) && e <= sms(8) ? 0 : ic.start[ACLS_W];
     warp_class(k_agg_merge_warp<AGG_SCAP, AGG_SWARPS, WT, AV>, 0, mid, AGG_SCAP, AGG_SWARPS, 32);
     warp_class(k_agg_merge_warp<AGG_WCAP, AGG_WWARPS, WT, AV>, mid, e, AGG_WCAP, AGG_WWARPS, 8);
