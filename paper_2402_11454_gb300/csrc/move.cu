@@ -264,21 +264,135 @@ __device__ __forceinline__ void score_slots(Table<V> &tab, const uint32_t *slot,
     }
 }
 
+// Float64 scores of a warp's candidates, packed: what bounds them is the issue
+// of two float64 divisions per candidate and warp, whether one lane scores or
+// all do, and after the first sweeps a row of many edges has few communities, a
+// lane's slots mostly none.  So the lanes hand their candidates to a queue of one
+// per lane, and a full queue is scored at once.  R-MAT of 60 K vertices, a wave
+// run, scored where they were claimed -> packed: degrees 2049-8192 154 -> 85 us,
+// 513-2048 40 -> 35, hubs 36 -> 22; the phase 11.1 -> 7.1 ms.
+template <typename V> struct ScoreQueue {
+    uint32_t c = EMPTY;
+    V v = V(0);
+    int n = 0;  // lanes 0..n-1 hold a candidate
+
+    template <int SYNC, typename SC, typename S>
+    __device__ void score(bool on, uint32_t x, V k, const double *Sig, const SC &sc, S &best, uint32_t &bestc) {
+        if (!on) return;
+        const S val = sc.score(k, ld_state<SYNC>(Sig + x));
+        if (better(val, x, best, bestc)) { best = val; bestc = x; }
+    }
+    // Take the candidates x[] with values k[] (EMPTY: none) of all 32 lanes.
+    template <int SYNC, int U, typename SC, typename S>
+    __device__ void put(const uint32_t (&x)[U], const V (&k)[U], const double *Sig, const SC &sc, S &best,
+                        uint32_t &bestc) {
+        constexpr unsigned FULL = 0xFFFFFFFFu;
+        const int lane = threadIdx.x & 31;
+        unsigned bal[U];
+        int total = 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            bal[u] = __ballot_sync(FULL, x[u] != EMPTY);
+            total += __popc(bal[u]);
+        }
+        if (total > 32 * (U - 1)) {  // packing would save no round: their gathers in flight together
+            double sg[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) sg[u] = x[u] != EMPTY ? ld_state<SYNC>(Sig + x[u]) : 0.0;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (x[u] == EMPTY) continue;
+                const S val = sc.score(k[u], sg[u]);
+                if (better(val, x[u], best, bestc)) { best = val; bestc = x[u]; }
+            }
+            return;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (!bal[u]) continue;
+            // the q-th candidate goes to lane n + q, round the end to the next queue
+            const int m = __popc(bal[u]), q = (lane - n) & 31;
+            const int src = q < m ? select_bit(bal[u], q) : 0;
+            const uint32_t xs = __shfl_sync(FULL, x[u], src);
+            const V ks = __shfl_sync(FULL, k[u], src);
+            const bool next = lane < n;
+            if (q < m && !next) { c = xs; v = ks; }
+            if (n + m >= 32) {
+                score<SYNC>(true, c, v, Sig, sc, best, bestc);
+                if (q < m && next) { c = xs; v = ks; }
+                n -= 32;
+            }
+            n += m;
+        }
+    }
+    template <int SYNC, typename SC, typename S>
+    __device__ void finish(const double *Sig, const SC &sc, S &best, uint32_t &bestc) {
+        score<SYNC>((int)(threadIdx.x & 31) < n, c, v, Sig, sc, best, bestc);
+        n = 0;
+    }
+};
+
+// As score_slots, by all lanes of a warp together.
+template <int N, int SYNC, typename SC, typename S, typename V>
+__device__ __forceinline__ void score_slots_warp(Table<V> &tab, const uint32_t *slot, const double *Sig, const SC &sc,
+                                                 S &best, uint32_t &bestc, uint32_t &ncand) {
+    if constexpr (std::is_same<V, float>::value) {
+        score_slots<N, SYNC>(tab, slot, Sig, sc, best, bestc, ncand);
+    } else {
+        ScoreQueue<V> queue;
+        constexpr int U = N < 4 ? N : 4;
+#pragma unroll
+        for (int s0 = 0; s0 < N; s0 += U) {
+            uint32_t c[U];
+            V v[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                c[u] = EMPTY;
+                v[u] = V(0);
+                if (slot[s0 + u] == EMPTY) continue;
+                c[u] = tab.get(slot[s0 + u], v[u]);
+                tab.clear(slot[s0 + u]);
+                ncand++;
+            }
+            queue.template put<SYNC>(c, v, Sig, sc, best, bestc);
+        }
+        queue.template finish<SYNC>(Sig, sc, best, bestc);
+    }
+}
+
 // The same over a whole table of cap slots, this thread's lane, lane + step, ...
+// (step: a multiple of the warp).
 template <int SYNC, typename SC, typename S, typename V>
 __device__ __forceinline__ void score_table(Table<V> &tab, uint32_t cap, uint32_t lane, uint32_t step,
                                             const double *Sig, const SC &sc, S &best, uint32_t &bestc,
                                             uint32_t &ncand) {
-    for (uint32_t s0 = lane; s0 < cap; s0 += 4 * step) {
+    ScoreQueue<V> queue;
+    for (uint32_t s0 = 0; s0 < cap; s0 += 4 * step) {
         uint32_t slot[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const uint32_t s = s0 + u * step;
+            const uint32_t s = s0 + u * step + lane;
             V v;
             slot[u] = s < cap && tab.get(s, v) != EMPTY ? s : EMPTY;
         }
-        score_slots<4, SYNC>(tab, slot, Sig, sc, best, bestc, ncand);
+        if constexpr (std::is_same<V, float>::value) {
+            score_slots<4, SYNC>(tab, slot, Sig, sc, best, bestc, ncand);
+        } else {
+            uint32_t c[4];
+            V v[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                c[u] = EMPTY;
+                v[u] = V(0);
+                if (slot[u] == EMPTY) continue;
+                c[u] = tab.get(slot[u], v[u]);
+                tab.clear(slot[u]);
+                ncand++;
+            }
+            queue.template put<SYNC>(c, v, Sig, sc, best, bestc);
+        }
     }
+    if constexpr (!std::is_same<V, float>::value) queue.template finish<SYNC>(Sig, sc, best, bestc);
 }
 
 // Equation 2, evaluated in the order written, with no contraction.
@@ -848,7 +962,7 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
             const SC sc = make_score<F64>(Ki, kid, Sd, m, vertex_inv_m(a, i, inv0), rounds_as_hub(deg));
             S best = -INFINITY;
             uint32_t bestc = EMPTY, ncand = 0;
-            if (held) score_slots<U, SYNC>(tab, slot, a.Sig, sc, best, bestc, ncand);
+            if (held) score_slots_warp<U, SYNC>(tab, slot, a.Sig, sc, best, bestc, ncand);
             else score_table<SYNC>(tab, slots, threadIdx.x, blockDim.x, a.Sig, sc, best, bestc, ncand);
             lc.candidates += ncand;
 #pragma unroll
@@ -1688,30 +1802,45 @@ __global__ void __launch_bounds__(HUB_THREADS, F64 ? 1 : 4) k_hub_score(MoveArgs
         uint32_t bestc = EMPTY, ncand = 0;
         // U slots per thread per round, their gathers of Sigma issued at once
         constexpr int U = 4;
-        for (uint32_t x = threadIdx.x; x < slots; x += U * HUB_THREADS) {
+        ScoreQueue<V> queue;
+        for (uint32_t x0 = 0; x0 < slots; x0 += U * HUB_THREADS) {  // the same trips for all lanes
+            const uint32_t x = x0 + threadIdx.x;
             uint32_t c[U];
             V val[U];
-            double sg[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 const uint32_t y = x + u * HUB_THREADS;
-                c[u] = y < slots ? tab.get(s0 + y, val[u]) : EMPTY;
+                c[u] = EMPTY;
+                val[u] = V(0);
+                if (y < slots) c[u] = tab.get(s0 + y, val[u]);
             }
+            if constexpr (F64) {
 #pragma unroll
-            for (int u = 0; u < U; u++) {
-                sg[u] = 0.0;
-                if (c[u] == EMPTY) continue;
-                tab.clear(s0 + x + u * HUB_THREADS);
-                sg[u] = ld_state<SYNC>(a.Sig + c[u]);
-            }
+                for (int u = 0; u < U; u++) {
+                    if (c[u] == EMPTY) continue;
+                    tab.clear(s0 + x + u * HUB_THREADS);
+                    ncand++;
+                }
+                queue.template put<SYNC>(c, val, a.Sig, sc, best, bestc);
+            } else {
+                double sg[U];
 #pragma unroll
-            for (int u = 0; u < U; u++) {
-                if (c[u] == EMPTY) continue;
-                ncand++;
-                const S v = sc.score(val[u], sg[u]);
-                if (better(v, c[u], best, bestc)) { best = v; bestc = c[u]; }
+                for (int u = 0; u < U; u++) {
+                    sg[u] = 0.0;
+                    if (c[u] == EMPTY) continue;
+                    tab.clear(s0 + x + u * HUB_THREADS);
+                    sg[u] = ld_state<SYNC>(a.Sig + c[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (c[u] == EMPTY) continue;
+                    ncand++;
+                    const S v = sc.score(val[u], sg[u]);
+                    if (better(v, c[u], best, bestc)) { best = v; bestc = c[u]; }
+                }
             }
         }
+        if constexpr (F64) queue.template finish<SYNC>(a.Sig, sc, best, bestc);
         lc.candidates += ncand;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
