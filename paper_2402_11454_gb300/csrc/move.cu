@@ -863,6 +863,29 @@ __global__ void __launch_bounds__(256, F64 ? 2 : 3) k_move_w512(MoveArgs a, cons
     flush_counters(lc, a.ctr);
 }
 
+// Float64 weights of one community met by several lanes go to the table as one:
+// a float64 add in shared memory is a loop of compare-and-swaps, in which the
+// edges of a row with few communities queue (9 K vertices of degree 7 K in ten
+// communities: a sweep 5.4 ms added one by one, 1.8 combined;
+// R-MAT of 60 K vertices, the phase 7.1 -> 5.3).  Sums of exactly
+// representable weights, exact in any order.  All 32 lanes; the first lane of a
+// community keeps it, the others are left with EMPTY.
+__device__ __forceinline__ void combine_lanes(uint32_t &c, double &v) {
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const unsigned peers = __match_any_sync(FULL, c);
+    unsigned m = c != EMPTY ? peers : 0u;
+    if (!__any_sync(FULL, m & (m - 1u))) return;
+    const int lane = threadIdx.x & 31, first = __ffs((int)m) - 1;
+    double sum = 0.0;
+    while (__any_sync(FULL, m)) {
+        const double x = __shfl_sync(FULL, v, m ? __ffs((int)m) - 1 : lane);
+        if (m) sum += x;
+        m &= m - 1u;
+    }
+    v = sum;
+    if (lane != first) c = EMPTY;
+}
+
 // --------------------------------------------------------------------------
 // One block per vertex, table of up to CAP slots in shared memory.  Two block
 // barriers a vertex: after the edges are inserted, and after their slots are
@@ -936,12 +959,12 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
 #pragma unroll
             for (int u = 0; u < U; u++) slot[u] = EMPTY;
             V kid = 0;
-            for (uint64_t p0 = b + threadIdx.x; p0 < e; p0 += (uint64_t)U * blockDim.x) {
+            for (uint64_t p0 = b; p0 < e; p0 += (uint64_t)U * blockDim.x) {  // the same trips for all threads
                 uint32_t j[U], c[U];
                 V wv[U];
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    const uint64_t p = p0 + (uint64_t)u * blockDim.x;
+                    const uint64_t p = p0 + (uint64_t)u * blockDim.x + threadIdx.x;
                     j[u] = p < e ? __ldg(a.tgt + p) : i;
                     wv[u] = p < e ? (V)__ldg(w + p) : V(0);
                 }
@@ -949,9 +972,12 @@ __device__ void block_body(const MoveArgs &a, const uint32_t *__restrict__ list,
                 for (int u = 0; u < U; u++) c[u] = j[u] != i ? ld_state<SYNC>(a.C + j[u]) : EMPTY;
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    if (c[u] == EMPTY) continue;
-                    if (c[u] == d) kid += wv[u];
-                    else slot[u] = tab.add(logcap, c[u], wv[u]);
+                    if (c[u] == d) {
+                        kid += wv[u];
+                        c[u] = EMPTY;
+                    }
+                    if constexpr (F64) combine_lanes(c[u], wv[u]);
+                    if (c[u] != EMPTY) slot[u] = tab.add(logcap, c[u], wv[u]);
                 }
             }
             kid = warp_sum(kid);
@@ -1013,7 +1039,8 @@ template <int CAP, int THREADS, typename WT, bool F64, int SYNC>
 __global__ void __launch_bounds__(THREADS, F64 ? 1 : 1024 / THREADS) k_move_block(MoveArgs a, const uint32_t *__restrict__ list, uint32_t count) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     LocalCtr lc;
-    block_body<CAP, 8, WT, F64, SYNC>(a, list, count, blockIdx.x, gridDim.x, dyn_smem, lc);
+    // the block's threads hold the slots of the class's longest row (CAP / 2 edges)
+    block_body<CAP, CAP / 2 / THREADS, WT, F64, SYNC>(a, list, count, blockIdx.x, gridDim.x, dyn_smem, lc);
     flush_counters(lc, a.ctr);
 }
 
