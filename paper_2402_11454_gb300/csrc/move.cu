@@ -1953,35 +1953,42 @@ __global__ void k_classify_count(const uint64_t *__restrict__ off, uint32_t n, i
 // The lists, a tile of vertices per block and round: ranked by key in shared
 // counters, then one reservation per key and tile.  (One per key and warp
 // queued 32 K atomics on each hot key of a million vertices: 1.17 ms on R-MAT
-// 24.)
-constexpr int FILL_PER = 8, FILL_TILE = 256 * FILL_PER;
+// 24.)  With one wave a tile has a handful of keys, and the ranks queue in their
+// counters: there the lanes of a key take theirs together (MATCH).  Small graphs
+// take tiles of 256 vertices, so that the few there are spread over the SMs.
+template <int PER, bool MATCH>
 __global__ void __launch_bounds__(256) k_classify_fill(const uint64_t *__restrict__ off, uint32_t n, int W,
                                                        uint32_t *cursor, uint32_t *list,
                                                        const uint32_t *__restrict__ gid,
                                                        const uint64_t *__restrict__ gvo, ClassBounds cb) {
     __shared__ uint32_t num[NUM_CLS * MAX_WAVES];
-    const int NK = NUM_CLS * W;
-    for (uint64_t v0 = (uint64_t)blockIdx.x * FILL_TILE; v0 < n; v0 += (uint64_t)gridDim.x * FILL_TILE) {
+    const int NK = NUM_CLS * W, lane = threadIdx.x & 31;
+    for (uint64_t v0 = (uint64_t)blockIdx.x * 256 * PER; v0 < n; v0 += (uint64_t)gridDim.x * 256 * PER) {
         for (int t = threadIdx.x; t < NK; t += 256) num[t] = 0;
         __syncthreads();
-        int key[FILL_PER];
-        uint32_t rank[FILL_PER];
+        int key[PER];
+        uint32_t rank[PER];
 #pragma unroll
-        for (int u = 0; u < FILL_PER; u++) {
+        for (int u = 0; u < PER; u++) {
             const uint64_t v = v0 + u * 256 + threadIdx.x;
-            key[u] = -1;
-            if (v >= n) continue;
-            const uint64_t deg = off[v + 1] - off[v];
-            if (!deg) continue;
-            key[u] = class_of(deg, cb) * W + wave_of((uint32_t)v, W, gid, gvo);
-            rank[u] = atomicAdd(num + key[u], 1u);
+            const uint64_t deg = v < n ? off[v + 1] - off[v] : 0;
+            key[u] = deg ? class_of(deg, cb) * W + wave_of((uint32_t)v, W, gid, gvo) : -1;
+            if (MATCH) {
+                const unsigned peers = __match_any_sync(0xFFFFFFFFu, key[u]);
+                const int leader = __ffs((int)peers) - 1;
+                uint32_t base = 0;
+                if (lane == leader && deg) base = atomicAdd(num + key[u], (uint32_t)__popc(peers));
+                rank[u] = __shfl_sync(0xFFFFFFFFu, base, leader) + __popc(peers & ((1u << lane) - 1u));
+            } else if (deg) {
+                rank[u] = atomicAdd(num + key[u], 1u);
+            }
         }
         __syncthreads();
         for (int t = threadIdx.x; t < NK; t += 256)
             if (num[t]) num[t] = atomicAdd(cursor + t, num[t]);
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < FILL_PER; u++)
+        for (int u = 0; u < PER; u++)
             if (key[u] >= 0) list[num[key[u]] + rank[u]] = (uint32_t)(v0 + u * 256 + threadIdx.x);
         __syncthreads();
     }
@@ -2016,7 +2023,12 @@ void classify_vertices(const DevGraph &g, Classes &cl, int waves, cudaStream_t s
     uint32_t *cursor = counts + NK;
     GSP_CUDA(cudaMemcpyAsync(cursor, cl.start, sizeof(uint32_t) * NK, cudaMemcpyHostToDevice, s));
     cl.list = arena().get<uint32_t>(cl.start[NK] + 1);
-    k_classify_fill<<<grid, 256, 0, s>>>(g.off, g.n, W, cursor, cl.list, gid, gvo, cb);
+    const bool few = g.n <= 256ull * sms(4);  // tiles of 256: at most four a SM
+    auto fill = [&](auto fn, unsigned tile) {
+        fn<<<grid_for(g.n, tile, sms(8)), 256, 0, s>>>(g.off, g.n, W, cursor, cl.list, gid, gvo, cb);
+    };
+    if (W == 1) few ? fill(k_classify_fill<1, true>, 256) : fill(k_classify_fill<8, true>, 2048);
+    else few ? fill(k_classify_fill<1, false>, 256) : fill(k_classify_fill<8, false>, 2048);
     GSP_CHECK_LAUNCH();
     cl.dstart = arena().get<uint32_t>(NK + 1);
     GSP_CUDA(cudaMemcpyAsync(cl.dstart, cl.start, sizeof(uint32_t) * (NK + 1), cudaMemcpyHostToDevice, s));
