@@ -9,6 +9,7 @@
 // float32-representable weights whose partial sums stay representable.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -133,7 +134,12 @@ void task_items(const uint64_t *prefix, uint32_t nitems, uint32_t *out, cudaStre
 // float64 atomic per row on their totals took 1.4 of the 1.55 ms of the row
 // sums of a 2 M vertex graph (R-MAT, star partition).  Integer units only (the
 // sums are exact, so their grouping does not show); float64 sums go out as they
-// come.
+// come, and so do those of graphs below SIGMA_MIN vertices, where too few rows
+// queue on a community to pay for the table (gsp_modularity, one atomic a row
+// against the table, us: planted 500 vertices 120 and 123, 8 K 125 and 128, 50 K
+// 139 and 142; R-MAT 1 K 132 and 137, 8 K 149 and 151, 16 K 169 and 168, 50 K
+// 251 and 206, 200 K 413 and 230).
+constexpr uint32_t SIGMA_MIN = 16384;
 struct SigmaSums {
     static constexpr int LOG = 10;
     static constexpr uint32_t SLOTS = 1u << LOG;
@@ -156,7 +162,6 @@ struct SigmaSums {
         }
         atomicAdd(Sig + c, Acc<unsigned long long>::val(k, lsb));  // crowded
     }
-    __device__ void add(double *Sig, uint32_t c, double k, int) { atomicAdd(Sig + c, k); }
     __device__ void flush(double *Sig, int lsb) {
         __syncthreads();
         for (uint32_t s = threadIdx.x; s < SLOTS; s += blockDim.x)
@@ -165,16 +170,17 @@ struct SigmaSums {
 };
 
 // Per row i: K_i, and the intra-community part sum_{j: C_j = C_i} w_ij when C
-// is given; Sigma_c += K_i when Sig is given.  Long rows are deferred to a
+// is given; Sigma_c += K_i when Sig is given (GROUPED: through a table, and Sig
+// must be).  Long rows are deferred to a
 // list for the block kernel.
-template <typename WT, typename AV>
+template <typename WT, typename AV, bool GROUPED>
 __global__ void k_row_sums(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tgt,
                            const WT *__restrict__ w, uint32_t n, const uint32_t *__restrict__ C, double *K,
                            double *Sig, AV *acc /* [0]=2m, [1]=intra */, uint32_t *longlist,
                            uint32_t *nlong, int lsb) {
     __shared__ AV red[32];
-    __shared__ SigmaSums sig;
-    if (Sig) sig.clear();
+    __shared__ typename std::conditional<GROUPED, SigmaSums, char>::type sig;
+    if constexpr (GROUPED) sig.clear();
     AV two_m = 0, intra = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint64_t b = off[i], e = off[i + 1];
@@ -206,11 +212,12 @@ __global__ void k_row_sums(const uint64_t *__restrict__ off, const uint32_t *__r
             if (C && C[tgt[p]] == ci) in += wv;
         }
         if (K) K[i] = Acc<AV>::val(k, lsb);
-        if (Sig) sig.add(Sig, ci, k, lsb);
+        if constexpr (GROUPED) sig.add(Sig, ci, k, lsb);
+        else if (Sig) atomicAdd(Sig + ci, Acc<AV>::val(k, lsb));
         two_m += k;
         intra += in;
     }
-    if (Sig) sig.flush(Sig, lsb);
+    if constexpr (GROUPED) sig.flush(Sig, lsb);
     two_m = block_sum(two_m, red);
     intra = block_sum(intra, red);
     if (threadIdx.x == 0) {
@@ -222,13 +229,13 @@ __global__ void k_row_sums(const uint64_t *__restrict__ off, const uint32_t *__r
 // Long rows: one warp per row up to 8192 entries, one block per longer row.
 constexpr uint32_t WARP_ROW = 8192;
 
-template <typename WT, typename AV>
+template <typename WT, typename AV, bool GROUPED>
 __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tgt,
                                 const WT *__restrict__ w, const uint32_t *__restrict__ C, double *K, double *Sig,
                                 AV *acc, const uint32_t *longlist, const uint32_t *nlong, int lsb) {
     __shared__ AV red[32];
-    __shared__ SigmaSums sig;
-    if (Sig) sig.clear();
+    __shared__ typename std::conditional<GROUPED, SigmaSums, char>::type sig;
+    if constexpr (GROUPED) sig.clear();
     uint32_t cnt = *nlong;
     const int lane = threadIdx.x & 31;
     uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -265,7 +272,8 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
         in = warp_sum(in);
         if (lane == 0) {
             if (K) K[i] = Acc<AV>::val(k, lsb);
-            if (Sig) sig.add(Sig, ci, k, lsb);
+            if constexpr (GROUPED) sig.add(Sig, ci, k, lsb);
+            else if (Sig) atomicAdd(Sig + ci, Acc<AV>::val(k, lsb));
             wk += k;
             win += in;
         }
@@ -303,12 +311,13 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
         in = block_sum(in, red);
         if (threadIdx.x == 0) {
             if (K) K[i] = Acc<AV>::val(k, lsb);
-            if (Sig) sig.add(Sig, ci, k, lsb);
+            if constexpr (GROUPED) sig.add(Sig, ci, k, lsb);
+            else if (Sig) atomicAdd(Sig + ci, Acc<AV>::val(k, lsb));
             wk += k;
             win += in;
         }
     }
-    if (Sig) sig.flush(Sig, lsb);
+    if constexpr (GROUPED) sig.flush(Sig, lsb);
     wk = block_sum(wk, red);
     win = block_sum(win, red);
     if (threadIdx.x == 0) {
@@ -317,18 +326,22 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
     }
 }
 
-template <typename WT, typename AV>
+template <typename WT, typename AV, bool GROUPED = false>
 static void row_sums(const DevGraph &g, const uint32_t *C, double *K, double *Sig, AV *acc, int lsb, cudaStream_t s) {
+    if constexpr (std::is_same<AV, unsigned long long>::value && !GROUPED)
+        if (Sig && g.n >= SIGMA_MIN) return row_sums<WT, AV, true>(g, C, K, Sig, acc, lsb, s);
     size_t mk = arena().mark();
     uint32_t *longlist = arena().get<uint32_t>(g.n + 1);
     uint32_t *nlong = arena().get<uint32_t>(1);
     GSP_CUDA(cudaMemsetAsync(nlong, 0, sizeof(uint32_t), s));
     const WT *w = static_cast<const WT *>(g.w);
-    k_row_sums<WT, AV><<<grid_for(g.n, 256), 256, 0, s>>>(g.off, g.tgt, w, g.n, C, K, Sig, acc, longlist, nlong, lsb);
+    k_row_sums<WT, AV, GROUPED><<<grid_for(g.n, 256), 256, 0, s>>>(g.off, g.tgt, w, g.n, C, K, Sig, acc, longlist,
+                                                                   nlong, lsb);
     GSP_CHECK_LAUNCH();
     // as many warps as fit: each long row is a chain of loads per lane
-    k_row_sums_long<WT, AV><<<resident_grid((const void *)k_row_sums_long<WT, AV>, 256, 0, 8), 256, 0, s>>>(
-        g.off, g.tgt, w, C, K, Sig, acc, longlist, nlong, lsb);
+    const auto long_rows = k_row_sums_long<WT, AV, GROUPED>;
+    long_rows<<<resident_grid((const void *)long_rows, 256, 0, 8), 256, 0, s>>>(g.off, g.tgt, w, C, K, Sig, acc,
+                                                                                longlist, nlong, lsb);
     GSP_CHECK_LAUNCH();
     arena().release(mk);
 }
@@ -420,10 +433,10 @@ static double modularity_scratch_t(const DevGraph &g, const uint32_t *C, double 
     GSP_CUDA(cudaMemsetAsync(acc, 0, 4 * sizeof(double), s));
     GSP_CUDA(cudaMemsetAsync(Sig, 0, sizeof(double) * g.n, s));
     GSP_CUDA(cudaMemsetAsync(nlong, 0, sizeof(uint32_t), s));
-    k_row_sums<WT, double><<<grid_for(g.n, 256), 256, 0, s>>>(g.off, g.tgt, w, g.n, C, nullptr, Sig, acc, longlist,
+    k_row_sums<WT, double, false><<<grid_for(g.n, 256), 256, 0, s>>>(g.off, g.tgt, w, g.n, C, nullptr, Sig, acc, longlist,
                                                               nlong, INT_MIN);
     GSP_CHECK_LAUNCH();
-    k_row_sums_long<WT, double><<<sms(4), 256, 0, s>>>(g.off, g.tgt, w, C, nullptr, Sig, acc, longlist, nlong,
+    k_row_sums_long<WT, double, false><<<sms(4), 256, 0, s>>>(g.off, g.tgt, w, C, nullptr, Sig, acc, longlist, nlong,
                                                        INT_MIN);
     GSP_CHECK_LAUNCH();
     k_sum_sq<<<grid_for(g.n, 256), 256, 0, s>>>(Sig, g.n, acc + 2);
