@@ -135,9 +135,12 @@ size_t workspace_peak() { return backing(&g_work_facade).peak; }
 void *Arena::alloc(size_t bytes) { return backing(this).alloc(bytes); }
 void *Arena::try_alloc(size_t bytes) {
     const size_t m = mark();
+    char before[sizeof(g_err)];  // the call goes on: its text is no failing call's
+    memcpy(before, g_err, sizeof(g_err));
     try {
         return alloc(bytes);
     } catch (const Error &) {
+        memcpy(g_err, before, sizeof(g_err));
         release(m);
         return nullptr;
     }
