@@ -487,7 +487,9 @@ gsp_status gsp_set_tuning(const gsp_tuning *t);
  * whole gsp_louvain calls on opts (its move mode, waves, wave repeats,
  * precision, split and refinement) under candidate caps and boundaries (each
  * boundary at its limit or half of it), one knob at a time, each trial the
- * better of two calls; keeps a candidate only when it is more than 1 % faster
+ * better of two calls; a cap that the call does not read (no vertex of its
+ * class, or a small graph whose passes run in one cluster) is left as it is;
+ * keeps a candidate only when it is more than 1 % faster
  * than the current choice, and finally times the pick against the settings
  * in effect at the call once more, keeping the faster.  Device graph as for
  * gsp_louvain (float32 weights); the graph is not modified.  *chosen

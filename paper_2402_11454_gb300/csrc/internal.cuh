@@ -39,6 +39,10 @@ struct ClassBounds {
     uint32_t group_max, warp_max, block_max, big_max;
 };
 Tuning &tuning();
+// A launch whose grid one of the caps bounds says so (gsp_autotune tries only
+// the caps that a call reads).
+enum Cap { CAP_GROUPS = 0, CAP_W512, CAP_BLOCK, CAP_HUB };
+void note_cap(Cap cap);
 
 // Degree classes of a vertex list.  Small degrees are served by groups of G
 // lanes with a shared-memory table, mid degrees by one block with a

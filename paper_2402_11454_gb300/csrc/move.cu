@@ -2125,6 +2125,7 @@ static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, void *po
     if (blocks) {
         k_move_groups<WT, F64, SYNC><<<blocks, 256, 0, s>>>(a, gl);
         GSP_CHECK_LAUNCH();
+        note_cap(CAP_GROUPS);
         main_free = false;
     }
     uint32_t nw5 = cl.count(CLS_W512, wave);
@@ -2139,6 +2140,7 @@ static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, void *po
         k_move_w512<WT, F64, SYNC><<<grid_for((uint64_t)nw5 * 32, 256, (uint32_t)(sm * tn.w512)), 256, smem, on(0)>>>(
             a, cl.list + cl.begin(CLS_W512, wave), nw5);
         GSP_CHECK_LAUNCH();
+        note_cap(CAP_W512);
     }
     uint32_t nb = cl.count(CLS_BLOCK, wave);
     if (nb) {
@@ -2153,6 +2155,7 @@ static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, void *po
         fn<<<grid_for(nb, 1, (uint32_t)(sm * tn.block)), THREADS, smem, on(1)>>>(a, cl.list + cl.begin(CLS_BLOCK, wave),
                                                                                 nb);
         GSP_CHECK_LAUNCH();
+        note_cap(CAP_BLOCK);
     }
     uint32_t ng = cl.count(CLS_BIG, wave);
     if (ng) {
@@ -2196,6 +2199,7 @@ static void launch_wave(const Classes &cl, const MoveArgs &a, int wave, void *po
         GSP_CHECK_LAUNCH();
         constexpr size_t hsmem = Table<V>::slot_bytes << HUB_SLOG;
         // one block per task at most: small waves launch only what they use
+        note_cap(CAP_HUB);
         const unsigned hub_grid = (unsigned)std::min<uint64_t>(ntasks, (uint64_t)sm * tn.hub);
         k_hub_insert<WT, F64, SYNC><<<hub_grid, HUB_THREADS, hsmem, s>>>(a, h);
         GSP_CHECK_LAUNCH();

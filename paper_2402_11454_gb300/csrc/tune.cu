@@ -25,6 +25,11 @@ static std::mutex g_tuning_mu;
 
 Tuning &tuning() { return g_tuning; }
 
+// The caps that launches have read (bit k: Cap k) since they were last cleared.
+static unsigned g_caps_read = 0;
+void note_cap(Cap cap) { __atomic_or_fetch(&g_caps_read, 1u << cap, __ATOMIC_RELAXED); }
+static bool cap_read(Cap cap) { return __atomic_load_n(&g_caps_read, __ATOMIC_RELAXED) >> cap & 1u; }
+
 int sm_count() {
     static int cached[64] = {0};
     int d = 0;
@@ -207,19 +212,21 @@ static void autotune_search(const std::function<void()> &one_run, TuneBuffers &t
     Tuning best = start;
     float t0 = 0.0f, tb = 0.0f;
     try {
+        __atomic_store_n(&g_caps_read, 0u, __ATOMIC_RELAXED);
         trial();  // first-touch effects (workspace, instruction cache)
         t0 = tb = trial();
         // a candidate replaces the current choice only when it is faster by
         // more than the run-to-run spread of a trial
         constexpr float ACCEPT = 0.99f;
         struct Knob {
+            Cap cap;
             int Tuning::*field;
             int cand[5];
         };
-        const Knob knobs[] = {{&Tuning::groups, {4, 6, 8, 12, 16}},
-                              {&Tuning::w512, {1, 2, 3, 4, 6}},
-                              {&Tuning::block, {2, 3, 4, 5, 8}},
-                              {&Tuning::hub, {2, 4, 8, 16, 32}}};
+        const Knob knobs[] = {{CAP_GROUPS, &Tuning::groups, {4, 6, 8, 12, 16}},
+                              {CAP_W512, &Tuning::w512, {1, 2, 3, 4, 6}},
+                              {CAP_BLOCK, &Tuning::block, {2, 3, 4, 5, 8}},
+                              {CAP_HUB, &Tuning::hub, {2, 4, 8, 16, 32}}};
         // class boundaries: each class may hand its upper half to the next
         // (larger) kernel; a boundary only moves down from the limit its
         // table allows
@@ -236,6 +243,9 @@ static void autotune_search(const std::function<void()> &one_run, TuneBuffers &t
                    t.big_max > t.block_max;
         };
         for (const Knob &k : knobs) {
+            // a cap that the call never reads (no vertex of its class, or the
+            // passes move inside one cluster) would be picked by noise
+            if (!cap_read(k.cap)) continue;
             for (int v : k.cand) {
                 if (v == best.*(k.field)) continue;
                 g_tuning = best;

@@ -56,3 +56,14 @@ def test_persistent_sweep_comes_first_where_asked_for(gsp, restore, n, k, precis
     # graphs above the setting keep the library's choice
     gsp.set_tuning(persist_max_vertices=1)
     assert launches(gsp, lambda: gsp.louvain(*d, precision=precision))[1] == without
+
+
+def test_autotune_leaves_caps_that_nothing_reads(gsp, restore):
+    d = dev(*graphgen.planted(n=3000, k=12, mean_degree=16, p_intra=0.8, seed=6))  # every pass on the cluster
+    odd = dict(groups_blocks_per_sm=5, w512_blocks_per_sm=5, block_blocks_per_sm=7, hub_blocks_per_sm=3)
+    gsp.set_tuning(**odd)
+    _, one = launches(gsp, lambda: gsp.louvain(*d))
+    (caps, _, _), all_runs = launches(gsp, lambda: gsp.autotune(*d))
+    assert {k: caps[k] for k in odd} == odd
+    # the four boundaries' trials and the final pair, not the 18 candidates of the caps twice each
+    assert all_runs < 36 * one
