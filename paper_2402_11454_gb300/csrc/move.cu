@@ -93,40 +93,6 @@ template <int SYNC, typename T> __device__ __forceinline__ T ld_state(const T *p
     else return ldcg(p);
 }
 
-template <typename V, typename WT> __device__ __forceinline__ V load_w(const WT *w, uint64_t e) {
-    return (V)__ldg(w + e);
-}
-
-// Scan the edges [b, e) of vertex i with stride `step` starting at b + lane:
-// the self-loop is skipped, K_{i->d} accumulates in kid, other communities
-// go to ins(c, w).  U edges per thread per round, their loads issued before
-// their use, so that U gathers of C[j] are in flight at once.
-template <int U, int SYNC, typename V, typename WT, typename F>
-__device__ __forceinline__ void scan_edges(const uint32_t *__restrict__ tgt, const WT *__restrict__ w,
-                                           const uint32_t *C, uint32_t i, uint32_t d, uint64_t b, uint64_t e,
-                                           uint32_t lane, uint32_t step, V &kid, F &&ins) {
-    for (uint64_t p0 = b + lane; p0 < e; p0 += (uint64_t)U * step) {
-        uint32_t j[U];
-        V wv[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            uint64_t p = p0 + (uint64_t)u * step;
-            bool ok = p < e;
-            j[u] = ok ? __ldg(tgt + p) : i;
-            wv[u] = ok ? (V)__ldg(w + p) : V(0);
-        }
-        uint32_t c[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) c[u] = (j[u] != i) ? ld_state<SYNC>(C + j[u]) : EMPTY;
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (c[u] == EMPTY) continue;
-            if (c[u] == d) kid += wv[u];
-            else ins(c[u], wv[u]);
-        }
-    }
-}
-
 // Open-addressing table of a vertex's K_{i->c} in shared memory, linear probing,
 // 2^logcap slots, at least twice the vertex's degree.  It is empty between
 // vertices: add() tells the thread that claimed a slot which one, that thread
