@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2402_11454_gb300 import graphgen
 
 pytestmark = pytest.mark.gpu
@@ -67,3 +68,39 @@ def test_autotune_leaves_caps_that_nothing_reads(gsp, restore):
     assert {k: caps[k] for k in odd} == odd
     # the four boundaries' trials and the final pair, not the 18 candidates of the caps twice each
     assert all_runs < 36 * one
+
+
+@pytest.fixture(scope="module")
+def above_the_cluster():
+    """R-MAT of 16 K vertices, above the cluster's float64 limits, and the oracle's partition."""
+    off, tgt, w = graphgen.rmat(14, 16, seed=2)
+    assert len(tgt) > 1 << 18
+    return dev(off, tgt, w), oracle.louvain(oracle.Graph(off, tgt, w.astype(np.float64)), oracle.LouvainOptions(sync=True))
+
+
+@pytest.mark.parametrize("caps", [{}, dict(groups_blocks_per_sm=1, w512_blocks_per_sm=1, block_blocks_per_sm=1, hub_blocks_per_sm=1),
+                                  dict(groups_blocks_per_sm=3, w512_blocks_per_sm=32, block_blocks_per_sm=2, hub_blocks_per_sm=7),
+                                  dict(group_max_degree=64, warp_max_degree=256, block_max_degree=1024, big_max_degree=1025)], ids=str)
+def test_class_kernels_equal_the_oracle_under_any_caps(gsp, restore, above_the_cluster, caps):
+    d, (Co, ost) = above_the_cluster
+    gsp.set_tuning(**caps)
+    (C, q, st), count = launches(gsp, lambda: gsp.louvain(*d, precision="fp64"))
+    assert count > 17 * 3 * 3  # the first sweep's wave runs: groups, warps, an application at least
+    assert st["iterations"] == ost["iterations"]
+    assert np.array_equal(C.cpu().numpy().astype(np.uint32), Co)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,k", [(700, 8), (9000, 60)])
+def test_small_graphs_move_in_one_launch(gsp, restore, n, k, precision):
+    """On the cluster a phase takes the same launches whatever its sweeps."""
+    d = dev(*graphgen.planted(n=n, k=k, mean_degree=14, p_intra=0.8, seed=3))
+    gsp.set_tuning(persist_max_vertices=0)
+    K, m = gsp.vertex_weights(*d)
+
+    def phase(sweeps):
+        C, S = torch.arange(n, dtype=torch.int32, device="cuda"), K.clone()
+        return gsp.local_move(*d, C, K, S, m, max_iterations=sweeps, precision=precision)
+
+    (one, first), (more, second) = launches(gsp, lambda: phase(1)), launches(gsp, lambda: phase(20))
+    assert one == 1 and more > 2 and first == second
