@@ -2320,14 +2320,23 @@ static bool launch_level(const MoveArgs &a, const LevelArgs &v, int ctas_needed,
 }
 
 // Most stored entries of a graph that one cluster moves.  Measured on GB300,
-// whole local-moving phase (gsp_local_move), launches against cluster, ms:
-// planted 2 K vertices / 30 K entries 2.08 and 1.17, 10 K / 151 K 2.45 and 1.40,
-// 10 K / 496 K 1.49 and 1.27, 20 K / 542 K 2.03 and 1.96, 30 K / 863 K 1.85 and
-// 2.31; 300^2 grid 1.80 and 1.46; R-MAT 3 K / 75 K 2.55 and 1.69, 30 K / 431 K
-// 2.64 and 2.35, 12 K / 602 K 3.36 and 3.80.  The float64 mode's divisions need
-// more SMs sooner: planted 10 K / 151 K 3.16 and 2.74, 200^2 grid / 151 K 1.96 and
-// 1.82, R-MAT 9 K / 252 K 5.50 and 6.43; dense graphs of few vertices gain a
-// little longer (540 vertices / 254 K entries 2.47 and 1.72).
+// whole local-moving phase (gsp_local_move), launches / cluster:
+//   mixed    planted, degree 16: 312 K entries 1.28, 408 K 1.08, 504 K 0.97, 536 K
+//            0.98; degree 48: 448 K 1.14, 537 K 1.11; grids 492 K 1.09, 519 K
+//            1.05, 548 K 0.98, 669 K 0.91; R-MAT 417 K 1.10, 541 K 1.07, 600 K
+//            1.01; dense graphs of 2 K vertices: planted 499 K 1.45, 940 K 1.31,
+//            R-MAT 416 K 1.08
+//   float64  planted, degree 16: 139 K 1.13, 171 K 1.03, 187 K 0.99, 203 K 0.87;
+//            degree 32: 148 K 1.16, 212 K 0.89; grids 151 K 1.06, 183 K 1.03,
+//            201 K 0.98, 237 K 0.94; R-MAT 75 K 1.04, 122 K 0.98, 157 K 1.03,
+//            200 K 0.98, 276 K 0.94
+//   float64, at most 2048 vertices: planted 225 K 1.33, 248 K 1.37, 328 K 1.18,
+//            410 K 1.08; 1500 vertices 210 K 1.15, 281 K 1.00, 377 K 0.94; R-MAT
+//            104 K 1.11, 152 K 0.95, 241 K 0.86
+// What the float64 mode costs on 16 SMs is its divisions, one pair a candidate:
+// rows whose neighbours soon share a few communities gain longer than rows whose
+// do not (R-MAT), which the entries cannot tell.  The dense limit is drawn for
+// the former: dense levels come from aggregation.
 constexpr uint64_t LEVEL_MAX_EDGES = 1u << 19, LEVEL_MAX_EDGES_F64 = 160000, LEVEL_MAX_EDGES_F64_DENSE = 1u << 18;
 constexpr uint32_t LEVEL_DENSE_VERTICES = 2048;
 
