@@ -1,7 +1,8 @@
 """Split ablation on the synthetic stand-ins of the paper's graphs: the split
 technique (none = GVE-Louvain, label propagation, label propagation with
-pruning, BFS, and hooking/shortcutting (SV), which is not in the paper) and
-its placement (after every pass, or once at the end), as in the paper's
+pruning, BFS, and hooking/shortcutting (SV), which is not in the paper; LPP and
+SV give the same labels by the same hooking pass, so their two rows are one
+measurement repeated) and its placement (after every pass, or once at the end), as in the paper's
 comparison of split variants (Section 4.1) and of GSP-Louvain against the
 method without a split (Section 5); and the Leiden refinement (Section 3.5)
 with and without the split (GSP-Leiden).
