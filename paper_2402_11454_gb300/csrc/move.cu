@@ -1108,16 +1108,37 @@ __global__ void __launch_bounds__(256) k_apply_moves(const uint32_t *__restrict_
     for (int t = threadIdx.x; t < (1 << APPLY_SLOG); t += blockDim.x) { skeys[t] = EMPTY; sds[t] = 0.0; sdn[t] = 0; }
     __syncthreads();
     const int iteration = *iteration_dev;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += appliers * blockDim.x) {
-        uint32_t i = mv_vtx[t], c = mv_cmt[t];
-        uint32_t d = C[i];
-        double Ki = K[i];
-        C[i] = c;
-        left[i] = d;
-        left_it[i] = iteration;
-        const unsigned long long u = lsb != INT_MIN ? units_of(Ki, lsb) : 0ull;
-        apply_delta(skeys, sds, sdn, d, Ki, u, -1, Sig, size, lsb);
-        apply_delta(skeys, sds, sdn, c, Ki, u, 1, Sig, size, lsb);
+    // four moves per thread and round, their loads in flight together: a warp of
+    // the deciding kernel lists its movers side by side, vertices from all over
+    // the wave's list (20 sweeps of one wave on a path of 470 K vertices: 3.9 ms
+    // one by one, 2.4 so; 3.2 while movers were listed as they came)
+    constexpr int U = 4;
+    const uint64_t step = (uint64_t)appliers * blockDim.x;
+    for (uint64_t t0 = blockIdx.x * blockDim.x + threadIdx.x; t0 < cnt; t0 += U * step) {
+        uint32_t i[U], c[U], d[U];
+        double k[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const uint64_t t = t0 + u * step;
+            i[u] = t < cnt ? mv_vtx[t] : EMPTY;
+            c[u] = t < cnt ? mv_cmt[t] : EMPTY;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (i[u] == EMPTY) continue;
+            d[u] = C[i[u]];
+            k[u] = K[i[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (i[u] == EMPTY) continue;
+            C[i[u]] = c[u];
+            left[i[u]] = d[u];
+            left_it[i[u]] = iteration;
+            const unsigned long long x = lsb != INT_MIN ? units_of(k[u], lsb) : 0ull;
+            apply_delta(skeys, sds, sdn, d[u], k[u], x, -1, Sig, size, lsb);
+            apply_delta(skeys, sds, sdn, c[u], k[u], x, 1, Sig, size, lsb);
+        }
     }
     __syncthreads();
     for (int t = threadIdx.x; t < (1 << APPLY_SLOG); t += blockDim.x) flush_delta(skeys, sds, sdn, t, Sig, size, lsb);
