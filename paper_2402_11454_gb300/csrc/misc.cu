@@ -235,8 +235,9 @@ __global__ void k_row_sums_long(const uint64_t *__restrict__ off, const uint32_t
                                 AV *acc, const uint32_t *longlist, const uint32_t *nlong, int lsb) {
     __shared__ AV red[32];
     __shared__ typename std::conditional<GROUPED, SigmaSums, char>::type sig;
-    if constexpr (GROUPED) sig.clear();
     uint32_t cnt = *nlong;
+    if (!cnt) return;
+    if constexpr (GROUPED) sig.clear();
     const int lane = threadIdx.x & 31;
     uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
