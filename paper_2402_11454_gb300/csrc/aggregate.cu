@@ -908,15 +908,18 @@ static void merge_tables(const DevGraph &g, const AggArgs &a, const IdClasses &i
             a, ic.list + first, last - first);
         GSP_CHECK_LAUNCH();
     };
-    // the two classes lie side by side in the list: as long as 8 warps an SM
-    // hold them all, the larger tables serve both in one launch.  Two launches
-    // and tiles of 1024 against this, R-MAT of 6 K vertices / 190 K entries:
-    // aggregation 420 and 378 us, 25 K 536 and 493, 70 K 614 and 566; above
-    // (110 K) 735 either way.  Since then the tiles' degree sums made it 361 at
-    // 6 K and 476 at 25 K (one atomic a vertex and no tiles: 366 and 513)
-    const uint32_t e = ic.start[ACLS_W + 1], mid = cnt_of(ACLS_W) && e <= sms(8) ? 0 : ic.start[ACLS_W];
+    // the two classes lie side by side in the list: as long as 32 warps an SM
+    // take them all, the larger tables serve both in one launch.  Two launches
+    // against one, gsp_aggregate: planted 5.6 K vertices in 2.4 K communities 297
+    // and 286 us, 12 K in 4.4 K 322 and 309, 40 K in 4 K 425 and 422; above (40 K
+    // in 8.8 K, R-MAT 110 K in 16 K) the small tables' launch stays, and they are
+    // level.  With tiles of 1024 and two launches R-MAT of 6 K vertices took 420,
+    // now 356 (one atomic a vertex, no tiles: 367); 25 K 536, now 468 (509)
+    const uint32_t e = ic.start[ACLS_W + 1], mid = cnt_of(ACLS_W) && e <= sms(32) ? 0 : ic.start[ACLS_W];
     warp_class(k_agg_merge_warp<AGG_SCAP, AGG_SWARPS, WT, AV>, 0, mid, AGG_SCAP, AGG_SWARPS, 32);
-    warp_class(k_agg_merge_warp<AGG_WCAP, AGG_WWARPS, WT, AV>, mid, e, AGG_WCAP, AGG_WWARPS, 8);
+    // as many blocks of the larger tables as an SM holds (4, or 6 of the packed ones)
+    constexpr unsigned per_sm = (227u << 10) / (AGG_WWARPS * AGG_WCAP * AggTable<AV>::slot_bytes + 1024);
+    warp_class(k_agg_merge_warp<AGG_WCAP, AGG_WWARPS, WT, AV>, mid, e, AGG_WCAP, AGG_WWARPS, per_sm);
     if (cnt_of(ACLS_B)) {
         constexpr size_t smem = (size_t)AGG_BCAP * AggTable<AV>::slot_bytes + (size_t)AGG_BMEM * sizeof(uint64_t) +
                                 (size_t)(AGG_BMEM + 1) * sizeof(uint32_t);
