@@ -104,3 +104,25 @@ def test_small_graphs_move_in_one_launch(gsp, restore, n, k, precision):
 
     (one, first), (more, second) = launches(gsp, lambda: phase(1)), launches(gsp, lambda: phase(20))
     assert one == 1 and more > 2 and first == second
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [150000, 200000, 700000, 1300000])
+def test_more_moves_than_threads_apply_them(gsp, n, precision):
+    """One wave in which most vertices of a path move: each thread of the
+    application takes up to four moves a round, for several rounds."""
+    i = np.arange(n - 1, dtype=np.uint64)
+    off, tgt, w = graphgen.edges_to_csr(n, i, i + 1, (1 + i * i % 7).astype(np.float32))  # whole weights
+    d = dev(off, tgt, w)
+    K, m = gsp.vertex_weights(*d)
+    C, S = torch.arange(n, dtype=torch.int32, device="cuda"), K.clone()
+    sweeps = gsp.local_move(*d, C, K, S, m, tolerance=0.0, max_iterations=3, waves=1, wave_repeats=1, no_return_from=0,
+                            precision=precision)
+    if precision == "fp64":
+        want = oracle.move(oracle.Graph(off, tgt, w.astype(np.float64)), np.arange(n), K.cpu().numpy(), K.cpu().numpy(), m,
+                           0.0, max_iterations=3, waves=1)
+        assert sweeps == want[2]
+        assert np.array_equal(C.cpu().numpy().astype(np.uint32), want[0])
+    total = torch.zeros(n, dtype=torch.float64, device="cuda").scatter_add_(0, C.long(), K)
+    assert torch.equal(S, total)  # whole sums
+    assert int((C != torch.arange(n, dtype=torch.int32, device="cuda")).sum()) > n // 3
