@@ -138,7 +138,8 @@ void task_items(const uint64_t *prefix, uint32_t nitems, uint32_t *out, cudaStre
 // queue on a community to pay for the table (gsp_modularity, one atomic a row
 // against the table, us: planted 500 vertices 120 and 123, 8 K 125 and 128, 50 K
 // 139 and 142; R-MAT 1 K 132 and 137, 8 K 149 and 151, 16 K 169 and 168, 50 K
-// 251 and 206, 200 K 413 and 230).
+// 251 and 206, 200 K 413 and 230; power laws of 60 to 80 K vertices whose
+// communities are all cold 213 and 221).
 constexpr uint32_t SIGMA_MIN = 16384;
 struct SigmaSums {
     static constexpr int LOG = 10;
